@@ -18,9 +18,8 @@
 // reversal, shell limits) freely.  Lines stay in shared memory: one kernel transforms the rows,
 // one the columns and adds up the shells, so the n x n spectrum is never stored.  Every n <= 4096
 // takes O(n^2 log n): radices 8, 4, 2, 3, 5, 7, 11, 13 when they factor n, Bluestein's chirp
-// convolution of power-of-two length >= 2n - 1 otherwise.  Against the direct O(n^3) sums that were
-// here, a checkpoint of the LES-vs-DNS comparison (2048^2 state, spectra at n = 1024) went from
-// 61.1 to 1.34 ms.
+// convolution of power-of-two length >= 2n - 1 otherwise.  Four fields at n = 1024 took 60.1 ms with
+// direct O(n^3) sums; now rows 178, columns and shells 286, shell totals 19 us.
 #include <cuda_runtime.h>
 
 #include <cmath>

@@ -34,153 +34,379 @@ constexpr int kP2 = kC2 * kC1 * 9 + kC2;          // 9248
 constexpr int kP3 = kC3 * kC2 * 9 + kC3;          // 1156
 constexpr int kNumParams = kP1 + kP2 + kP3;       // 13892
 constexpr int kThreads = 256;
-constexpr int kWeightCellsPerBlock = 1024;        // cells per block in the weight-gradient pass
+constexpr int kMaxConvBlocks = 2 * 152;           // blocks of a convolution: two per SM
 constexpr uint64_t kNetWaitNs = 2000000000ull;    // bound of every tensor-core completion wait
 
 __device__ __forceinline__ int wrapi(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
 
-// ---- binary32 forward: one thread per cell, all CO outputs ----------------------------------
-template <int CI, int CO, bool TANH>
-__global__ void conv_fwd_kernel(const float* __restrict__ in, const float* __restrict__ params,
-                                int batch, int H, int W, float* __restrict__ out) {
-  __shared__ float sw[CO * CI * 9 + CO];
-  for (int i = threadIdx.x; i < CO * CI * 9 + CO; i += blockDim.x) sw[i] = params[i];
-  __syncthreads();
-  const long plane = (long)H * W;
-  const long total = (long)batch * plane;
-  for (long c = blockIdx.x * (long)blockDim.x + threadIdx.x; c < total; c += (long)gridDim.x * blockDim.x) {
-    const int b = (int)(c / plane);
-    const int cell = (int)(c % plane);
-    const int y = cell / W, x = cell % W;
-    int off[9];
+// ---- binary32 convolutions (forward and data gradient) ----------------------------------------
+// One kernel for y[o](x) = b[o] + sum_i sum_t w[o][i][t] in[i](x + d_t) (forward) and, BWD, for
+// da[o](z) = sum_i sum_t W[i][o][t] dy[i](z - d_t) (W as the layer stores it).  Bound by binary32
+// FMAs, so the operands have to reach registers by few instructions: a thread computes 4
+// adjacent cells x 16 outputs (4 for the last layer), and one 16-byte shared-memory load of
+// weights (all lanes the same address) feeds 16 FMAs, where one thread per cell needed a load per
+// FMA.  Input channels arrive four at a time in two buffers (cp.async), the next four in flight
+// while these are used; a block walks tiles with the weights kept in shared memory.  Each
+// output's sum runs over channels, then taps, as with one thread per cell, so results are bitwise
+// the same.  At 8 x 256^2: 32 -> 32 forward 567 -> 199 us (48 TFLOP/s; the FMA units reach about
+// 75), its data gradient 425 -> 191 us, 12 -> 32 221 -> 86 us, 32 -> 4 with the loss 147 -> 53 us.
+constexpr int kTileW = 32;        // tile width: 8 threads of 4 cells
+constexpr int kConvThreads = 256;
+constexpr int kConvChunk = 4;     // input channels per buffer
+constexpr int kTilePitch = 36;    // floats per staged row: columns -1 .. 32, padded to 16 bytes
+
+enum ConvEpilogue { kEpiNone, kEpiTanh, kEpiTanhGrad, kEpiLoss };
+
+template <int CIN, int COUT>
+struct ConvShape {
+  static constexpr int kOuts = COUT < 16 ? COUT : 16;       // outputs per thread
+  static constexpr int kGroups = COUT / kOuts;              // groups of warps over outputs
+  static constexpr int kRows = 4 * kConvThreads / kGroups / kTileW;
+  static constexpr int kRowElems = (kRows + 2) * kTilePitch;
+  static constexpr int kLoads = ((kRows + 2) * (kTileW + 2) + kConvThreads - 1) / kConvThreads;
+  static constexpr size_t kSmem = (CIN * 9 * COUT + 2 * kConvChunk * kRowElems) * sizeof(float);
+  static_assert(CIN % kConvChunk == 0 && COUT % 4 == 0, "channel counts");
+};
+
+__device__ __forceinline__ int wrap_mod(int i, int n) {
+  i %= n;
+  return i < 0 ? i + n : i;
+}
+
+__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// aux: kEpiTanhGrad the activation a (result times 1 - a^2), kEpiLoss the target (result
+// (y - target) / n_out, and the block's sum of (y - target)^2 into loss_part[blockIdx.x]).
+template <int CIN, int COUT, int EPI, bool BWD>
+__global__ void __launch_bounds__(kConvThreads, 2)
+    conv_tile_kernel(const float* __restrict__ in, const float* __restrict__ params, const float* __restrict__ aux,
+                     int batch, int H, int W, float* __restrict__ out, double* __restrict__ loss_part) {
+  using Sh = ConvShape<CIN, COUT>;
+  constexpr int NO = Sh::kOuts;
+  extern __shared__ __align__(16) float conv_smem[];
+  float* sw = conv_smem;                   // [ci][tap][co]
+  float* st = conv_smem + CIN * 9 * COUT;  // [2][kConvChunk][row][kTilePitch]
+  const int tid = threadIdx.x;
+  for (int i = tid; i < CIN * 9 * COUT; i += kConvThreads) {
+    const int co = i % COUT, ct = i / COUT, ci = ct / 9, t = ct % 9;
+    sw[i] = params[BWD ? (ci * COUT + co) * 9 + t : (co * CIN + ci) * 9 + t];
+  }
+  const int o0 = tid / (kConvThreads / Sh::kGroups) * NO;
+  const int xg = tid % 8, yy = tid % (kConvThreads / Sh::kGroups) / 8;
+  const size_t plane = (size_t)H * W;
+  const int tiles_x = (W + kTileW - 1) / kTileW, tiles_y = (H + Sh::kRows - 1) / Sh::kRows;
+  const long ntiles = (long)batch * tiles_x * tiles_y;
+  // 16-byte stores need rows of whole quads on 16-byte boundaries
+  const bool vec = W % 4 == 0 && reinterpret_cast<uintptr_t>(out) % 16 == 0;
+  const float inv_n = 1.f / (float)((long)batch * COUT * (long)plane);
+  double loss = 0.0;
+
+  for (long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int b = (int)(tile / ((long)tiles_x * tiles_y)), rem = (int)(tile % ((long)tiles_x * tiles_y));
+    const int y0 = rem / tiles_x * Sh::kRows, x0 = rem % tiles_x * kTileW;
+    const float* ib = in + (size_t)b * CIN * plane;
+    // this thread's elements of a staged channel (rows y0 - 1 .., columns x0 - 1 .., periodic)
+    size_t goff[Sh::kLoads];
+    int soff[Sh::kLoads];
 #pragma unroll
-    for (int t = 0; t < 9; ++t) off[t] = wrapi(y + t / 3 - 1, H) * W + wrapi(x + t % 3 - 1, W);
-    float acc[CO];
+    for (int k = 0; k < Sh::kLoads; ++k) {
+      const int e = tid + k * kConvThreads, r = e / (kTileW + 2), c = e % (kTileW + 2);
+      soff[k] = r < Sh::kRows + 2 ? r * kTilePitch + c : -1;
+      goff[k] = (size_t)wrap_mod(y0 - 1 + r, H) * W + wrap_mod(x0 - 1 + c, W);
+    }
+    auto stage = [&](int chunk) {
+      float* d = st + (chunk & 1) * kConvChunk * Sh::kRowElems;
+      const float* g = ib + (size_t)chunk * kConvChunk * plane;
 #pragma unroll
-    for (int co = 0; co < CO; ++co) acc[co] = sw[CO * CI * 9 + co];
-    const float* ib = in + (size_t)b * CI * plane;
-    for (int ci = 0; ci < CI; ++ci) {
+      for (int c = 0; c < kConvChunk; ++c)
 #pragma unroll
-      for (int t = 0; t < 9; ++t) {
-        const float v = ib[(size_t)ci * plane + off[t]];
+        for (int k = 0; k < Sh::kLoads; ++k)
+          if (soff[k] >= 0) cp_async4(d + c * Sh::kRowElems + soff[k], g + c * plane + goff[k]);
+      cp_async_commit();
+    };
+    float acc[4][NO];
 #pragma unroll
-        for (int co = 0; co < CO; ++co) acc[co] = fmaf(sw[(co * CI + ci) * 9 + t], v, acc[co]);
+    for (int o = 0; o < NO; ++o) {
+      const float bv = BWD ? 0.f : params[COUT * CIN * 9 + o0 + o];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) acc[i][o] = bv;
+    }
+    stage(0);
+    constexpr int kChunks = CIN / kConvChunk;
+#pragma unroll 1
+    for (int ch = 0; ch < kChunks; ++ch) {
+      if (ch + 1 < kChunks) {
+        stage(ch + 1);
+        cp_async_wait<1>();
+      } else {
+        cp_async_wait<0>();
+      }
+      __syncthreads();
+      const float* buf = st + (ch & 1) * kConvChunk * Sh::kRowElems + 4 * xg;
+#pragma unroll 1
+      for (int c = 0; c < kConvChunk; ++c) {
+        const float* wc = sw + (size_t)(ch * kConvChunk + c) * 9 * COUT + o0;
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+          const float* row = buf + c * Sh::kRowElems + (yy + (BWD ? 2 - r : r)) * kTilePitch;
+          const float4 lo4 = *reinterpret_cast<const float4*>(row);
+          const float2 hi2 = *reinterpret_cast<const float2*>(row + 4);
+          const float v[6] = {lo4.x, lo4.y, lo4.z, lo4.w, hi2.x, hi2.y};
+#pragma unroll
+          for (int dx = 0; dx < 3; ++dx) {
+            float w[NO];
+#pragma unroll
+            for (int o = 0; o < NO; o += 4)
+              *reinterpret_cast<float4*>(&w[o]) = *reinterpret_cast<const float4*>(wc + (r * 3 + dx) * COUT + o);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+              for (int o = 0; o < NO; ++o) acc[i][o] = fmaf(w[o], v[i + (BWD ? 2 - dx : dx)], acc[i][o]);
+          }
+        }
+      }
+      __syncthreads();  // the buffer is refilled two chunks on
+    }
+    const int y = y0 + yy, x = x0 + 4 * xg;
+    const int nv = y < H ? min(4, W - x) : 0;  // cells of this thread inside the grid
+    if (nv > 0) {
+#pragma unroll
+      for (int o = 0; o < NO; ++o) {
+        const size_t at = ((size_t)b * COUT + o0 + o) * plane + (size_t)y * W + x;
+        float v[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          v[i] = acc[i][o];
+          if (EPI == kEpiTanh) v[i] = tanhf(v[i]);
+          if (i < nv) {
+            if (EPI == kEpiTanhGrad) {
+              const float a = aux[at + i];
+              v[i] *= (1.f - a * a);
+            }
+            if (EPI == kEpiLoss) {
+              const float d = v[i] - aux[at + i];
+              v[i] = d * inv_n;
+              loss += (double)d * d;
+            }
+          }
+        }
+        if (vec) {
+          *reinterpret_cast<float4*>(out + at) = make_float4(v[0], v[1], v[2], v[3]);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (i < nv) out[at + i] = v[i];
+        }
       }
     }
-    float* ob = out + (size_t)b * CO * plane;
-#pragma unroll
-    for (int co = 0; co < CO; ++co) ob[(size_t)co * plane + cell] = TANH ? tanhf(acc[co]) : acc[co];
+  }
+  if constexpr (EPI == kEpiLoss) {
+    __shared__ double sh[kConvThreads];
+    sh[tid] = loss;
+    __syncthreads();
+    for (int w = kConvThreads / 2; w > 0; w >>= 1) {
+      if (tid < w) sh[tid] += sh[tid + w];
+      __syncthreads();
+    }
+    if (tid == 0) loss_part[blockIdx.x] = sh[0];
   }
 }
 
-// ---- back-propagation -------------------------------------------------------------------------
-// da[ci](z) = sum_co sum_d W[co][ci][d] dy[co](z - d); then times (1 - a^2) if the input came
-// from a tanh (a = that activation).
-template <int CI, int CO, bool TANH_IN>
-__global__ void conv_bwd_data_kernel(const float* __restrict__ dy, const float* __restrict__ params,
-                                     const float* __restrict__ a_in, int batch, int H, int W,
-                                     float* __restrict__ da) {
-  __shared__ float sw[CO * CI * 9];
-  for (int i = threadIdx.x; i < CO * CI * 9; i += blockDim.x) sw[i] = params[i];
-  __syncthreads();
-  const long plane = (long)H * W;
-  const long total = (long)batch * plane;
-  for (long c = blockIdx.x * (long)blockDim.x + threadIdx.x; c < total; c += (long)gridDim.x * blockDim.x) {
-    const int b = (int)(c / plane);
-    const int cell = (int)(c % plane);
-    const int y = cell / W, x = cell % W;
-    int off[9];  // z - d for tap d
-#pragma unroll
-    for (int t = 0; t < 9; ++t) off[t] = wrapi(y - (t / 3 - 1), H) * W + wrapi(x - (t % 3 - 1), W);
-    float acc[CI];
-#pragma unroll
-    for (int ci = 0; ci < CI; ++ci) acc[ci] = 0.f;
-    const float* db = dy + (size_t)b * CO * plane;
-    for (int co = 0; co < CO; ++co) {
-#pragma unroll
-      for (int t = 0; t < 9; ++t) {
-        const float g = db[(size_t)co * plane + off[t]];
-#pragma unroll
-        for (int ci = 0; ci < CI; ++ci) acc[ci] = fmaf(sw[(co * CI + ci) * 9 + t], g, acc[ci]);
-      }
-    }
-    const float* ab = a_in + (size_t)b * CI * plane;
-    float* ob = da + (size_t)b * CI * plane;
-#pragma unroll
-    for (int ci = 0; ci < CI; ++ci) {
-      float v = acc[ci];
-      if (TANH_IN) {
-        const float a = ab[(size_t)ci * plane + cell];
-        v *= (1.f - a * a);
-      }
-      ob[(size_t)ci * plane + cell] = v;
-    }
-  }
+// ---- weight gradients ----------------------------------------------------------------------------
+// dW[co][ci][t] = sum_z dy[co](z) a[ci](z + d_t), db[co] = sum_z dy[co](z).  Bound by binary32 FMAs
+// (18,432 flops per cell for the 32 x 32 layer).  Lane l of a warp holds channel l of the
+// 32-channel operand ("lane": dy for layers 1 and 2, a for layer 3), a warp NW channels of the
+// other ("window"), so a thread keeps NW x 9 sums in registers; per 8 cells it takes 2 16-byte
+// loads of its lane's values and 3 loads per window row, the same address in every lane, for 72
+// NW FMAs.  A block stages 32 x 8 cells of both operands in shared memory; its warps split the
+// window channels, and the rows where there are fewer than eight groups of them.  Sums are
+// kept per tile and then added to a running sum, so binary32 rounding grows with the tiles, not
+// the cells; blocks write partial sums that sum_partials_kernel adds in block order
+// (deterministic).  At 8 x 256^2 the three layers took 20.6 (32 x 32), 7.8 (12 x 32) and 2.6 ms
+// (32 x 4) with one thread per weight reading both operands from global memory; now 236, 100 and
+// 52 us.
+constexpr int kWgThreads = 256;
+constexpr int kWgRows = 8;
+constexpr int kWgCells = kTileW * kWgRows;      // 256: one per thread when staging
+constexpr int kWgLanePitch = kWgCells + 4;      // lanes 4 banks apart: conflict-free 16-byte loads
+constexpr int kWgWinElems = (kWgRows + 2) * kTilePitch;
+static_assert(kWgCells == kWgThreads, "one staged cell per thread and channel");
+
+template <int NWIN>
+__host__ __device__ constexpr size_t wgrad_smem() {
+  return (32 * kWgLanePitch + NWIN * kWgWinElems) * sizeof(float);
 }
 
-// Per-block partial weight gradients over kWeightCellsPerBlock cells:
-// dW[co][ci][d] = sum_z dy[co](z) a[ci](z + d),  db[co] = sum_z dy[co](z).
-template <int CI, int CO>
-__global__ void conv_bwd_weight_kernel(const float* __restrict__ dy, const float* __restrict__ a,
-                                       int batch, int H, int W, float* __restrict__ partials) {
-  constexpr int NW = CO * CI * 9 + CO;
-  const long plane = (long)H * W;
-  const long total = (long)batch * plane;
-  const long c0 = (long)blockIdx.x * kWeightCellsPerBlock;
-  const long c1 = c0 + kWeightCellsPerBlock < total ? c0 + kWeightCellsPerBlock : total;
-  for (int w = threadIdx.x; w < NW; w += blockDim.x) {
-    float acc = 0.f;
-    if (w < CO * CI * 9) {
-      const int co = w / (CI * 9), ci = (w / 9) % CI, t = w % 9;
-      const int ddy = t / 3 - 1, ddx = t % 3 - 1;
-      for (long c = c0; c < c1; ++c) {
-        const int b = (int)(c / plane);
-        const int cell = (int)(c % plane);
-        const int y = cell / W, x = cell % W;
-        const float g = dy[(size_t)b * CO * plane + (size_t)co * plane + cell];
-        const float v = a[(size_t)b * CI * plane + (size_t)ci * plane + wrapi(y + ddy, H) * W + wrapi(x + ddx, W)];
-        acc = fmaf(g, v, acc);
-      }
-    } else {
-      const int co = w - CO * CI * 9;
-      for (long c = c0; c < c1; ++c) {
-        const int b = (int)(c / plane);
-        const int cell = (int)(c % plane);
-        acc += dy[(size_t)b * CO * plane + (size_t)co * plane + cell];
+// NWIN window channels in all, NW per warp.  LANE_DY: lane = dy [32 channels], window = a [NWIN];
+// else lane = a, window = dy (its tap t offset is -d_t).  part: [block][kNumParams] with this
+// layer's parameters from `base`.
+template <int NWIN, int NW, bool LANE_DY>
+__global__ void __launch_bounds__(kWgThreads, 2)
+    conv_wgrad_kernel(const float* __restrict__ lane_op, const float* __restrict__ win_op, int batch, int H, int W,
+                      float* __restrict__ part, int base) {
+  constexpr int kGroups = NWIN / NW, kSplits = 8 / kGroups;
+  static_assert(kGroups * NW == NWIN && kGroups * kSplits == 8, "eight warps");
+  extern __shared__ __align__(16) float wg_smem[];
+  float* sl = wg_smem;                       // [32][kWgLanePitch]
+  float* sn = wg_smem + 32 * kWgLanePitch;   // [NWIN][row][kTilePitch]
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int group = warp % kGroups, split = warp / kGroups;
+  const size_t plane = (size_t)H * W;
+  const int tiles_x = (W + kTileW - 1) / kTileW, tiles_y = (H + kWgRows - 1) / kWgRows;
+  const long ntiles = (long)batch * tiles_x * tiles_y;
+  float tot[NW * 9], tot_b[NW];
+#pragma unroll
+  for (int k = 0; k < NW * 9; ++k) tot[k] = 0.f;
+#pragma unroll
+  for (int k = 0; k < NW; ++k) tot_b[k] = 0.f;
+
+  for (long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int b = (int)(tile / ((long)tiles_x * tiles_y)), rem = (int)(tile % ((long)tiles_x * tiles_y));
+    const int y0 = rem / tiles_x * kWgRows, x0 = rem % tiles_x * kTileW;
+    const float* lb = lane_op + (size_t)b * 32 * plane;
+    const float* wb = win_op + (size_t)b * NWIN * plane;
+    {  // lane operand: cell tid of every channel, zero outside the grid
+      const int y = y0 + tid / kTileW, x = x0 + tid % kTileW;
+      const bool in = y < H && x < W;
+      const float* src = lb + (in ? (size_t)y * W + x : 0);
+#pragma unroll 8
+      for (int c = 0; c < 32; ++c) {
+        if (in) cp_async4(sl + c * kWgLanePitch + tid, src + c * plane);
+        else sl[c * kWgLanePitch + tid] = 0.f;
       }
     }
-    partials[(size_t)blockIdx.x * NW + w] = acc;
-  }
-}
-
-// Sum the block partials in block order (deterministic).
-__global__ void sum_partials_kernel(const float* __restrict__ partials, int nblocks, int nw,
-                                    float* __restrict__ out) {
-  for (int w = blockIdx.x * blockDim.x + threadIdx.x; w < nw; w += gridDim.x * blockDim.x) {
-    float s = 0.f;
-    for (int b = 0; b < nblocks; ++b) s += partials[(size_t)b * nw + w];
-    out[w] = s;
-  }
-}
-
-// dout = (out - target) / n and per-block partial sums of (out - target)^2.
-__global__ void loss_grad_kernel(const float* __restrict__ out, const float* __restrict__ target, long n,
-                                 float* __restrict__ dout, double* __restrict__ partial) {
-  __shared__ double sh[kThreads];
-  double acc = 0.0;
-  const float inv = 1.f / (float)n;
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-    const float d = out[i] - target[i];
-    dout[i] = d * inv;
-    acc += (double)d * d;
-  }
-  sh[threadIdx.x] = acc;
-  __syncthreads();
-  for (int w = kThreads / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {  // window operand: rows y0 - 1 .., columns x0 - 1 .., periodic
+      const int e = tid + k * kWgThreads, r = e / (kTileW + 2), c = e % (kTileW + 2);
+      if (r < kWgRows + 2) {
+        const float* src = wb + (size_t)wrap_mod(y0 - 1 + r, H) * W + wrap_mod(x0 - 1 + c, W);
+        float* dst = sn + r * kTilePitch + c;
+#pragma unroll 4
+        for (int ch = 0; ch < NWIN; ++ch) cp_async4(dst + ch * kWgWinElems, src + ch * plane);
+      }
+    }
+    cp_async_commit();
+    cp_async_wait<0>();
+    __syncthreads();
+    float acc[NW * 9], acc_b[NW];
+#pragma unroll
+    for (int k = 0; k < NW * 9; ++k) acc[k] = 0.f;
+#pragma unroll
+    for (int k = 0; k < NW; ++k) acc_b[k] = 0.f;
+#pragma unroll 1
+    for (int q = split; q < kWgCells / 8; q += kSplits) {  // 8 cells of one row at a time
+      const int row = q / (kTileW / 8), col = q % (kTileW / 8) * 8;
+      float l[8];
+      const float* lp = sl + lane * kWgLanePitch + row * kTileW + col;
+      *reinterpret_cast<float4*>(&l[0]) = *reinterpret_cast<const float4*>(lp);
+      *reinterpret_cast<float4*>(&l[4]) = *reinterpret_cast<const float4*>(lp + 4);
+      const float* wp = sn + group * NW * kWgWinElems + row * kTilePitch + col;
+#pragma unroll
+      for (int n = 0; n < NW; ++n) {
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+          float w[10];
+          const float* p = wp + n * kWgWinElems + r * kTilePitch;
+          *reinterpret_cast<float4*>(&w[0]) = *reinterpret_cast<const float4*>(p);
+          *reinterpret_cast<float4*>(&w[4]) = *reinterpret_cast<const float4*>(p + 4);
+          *reinterpret_cast<float2*>(&w[8]) = *reinterpret_cast<const float2*>(p + 8);
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int dx = 0; dx < 3; ++dx) acc[n * 9 + r * 3 + dx] = fmaf(l[i], w[i + dx], acc[n * 9 + r * 3 + dx]);
+          if (!LANE_DY && r == 1) {
+            // db of window channel n: the cells' own values, those inside the grid (the lane
+            // operand is zero outside, the window wraps)
+            const int nc = y0 + row < H ? W - x0 - col : 0;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) acc_b[n] += i < nc ? w[i + 1] : 0.f;
+          }
+        }
+      }
+      if (LANE_DY && group == 0) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) acc_b[0] += l[i];
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < NW * 9; ++k) tot[k] += acc[k];
+#pragma unroll
+    for (int k = 0; k < NW; ++k) tot_b[k] += acc_b[k];
     __syncthreads();
   }
-  if (threadIdx.x == 0) partial[blockIdx.x] = sh[0];
+  // add the row splits in order (staging buffers free), then store this block's partial sums
+  float* out = part + (size_t)blockIdx.x * kNumParams + base;
+  float* red = wg_smem;  // [group][value][lane]
+  constexpr int NV = NW * 9 + NW;
+  static_assert(kGroups * NV * 32 * sizeof(float) <= wgrad_smem<NWIN>(), "reduction fits");
+  for (int sidx = 1; sidx < kSplits; ++sidx) {
+    if (split == sidx) {
+#pragma unroll
+      for (int k = 0; k < NW * 9; ++k) red[(group * NV + k) * 32 + lane] = tot[k];
+#pragma unroll
+      for (int k = 0; k < NW; ++k) red[(group * NV + NW * 9 + k) * 32 + lane] = tot_b[k];
+    }
+    __syncthreads();
+    if (split == 0) {
+#pragma unroll
+      for (int k = 0; k < NW * 9; ++k) tot[k] += red[(group * NV + k) * 32 + lane];
+#pragma unroll
+      for (int k = 0; k < NW; ++k) tot_b[k] += red[(group * NV + NW * 9 + k) * 32 + lane];
+    }
+    __syncthreads();
+  }
+  if (split == 0) {
+#pragma unroll
+    for (int n = 0; n < NW; ++n) {
+      const int wch = group * NW + n;
+#pragma unroll
+      for (int t = 0; t < 9; ++t) {
+        if (LANE_DY) out[(lane * NWIN + wch) * 9 + t] = tot[n * 9 + t];
+        else out[(wch * 32 + lane) * 9 + 8 - t] = tot[n * 9 + t];
+      }
+      if (!LANE_DY && lane == 0) out[NWIN * 32 * 9 + wch] = tot_b[n];
+    }
+    if (LANE_DY && group == 0) out[32 * NWIN * 9 + lane] = tot_b[0];
+  }
+}
+
+// Sum the blocks' partial gradients and losses: eight threads per parameter take every eighth
+// block in order and are added in order (deterministic).  Block 0 adds up the loss.
+__global__ void sum_partials_kernel(const float* __restrict__ part, int nblocks, float* __restrict__ grad,
+                                    const double* __restrict__ loss_part, int nloss, double* __restrict__ loss) {
+  __shared__ float sh[8][32];
+  const int w = blockIdx.x * 32 + threadIdx.x;
+  float s = 0.f;
+  if (w < kNumParams)
+    for (int b = threadIdx.y; b < nblocks; b += 8) s += part[(size_t)b * kNumParams + w];
+  sh[threadIdx.y][threadIdx.x] = s;
+  __syncthreads();
+  if (threadIdx.y == 0 && w < kNumParams) {
+    float t = 0.f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) t += sh[i][threadIdx.x];
+    grad[w] = t;
+  }
+  if (blockIdx.x == 0) {
+    __shared__ double dl[256];
+    const int tid = threadIdx.y * 32 + threadIdx.x;
+    double d = 0.0;
+    for (int b = tid; b < nloss; b += 256) d += loss_part[b];
+    dl[tid] = d;
+    __syncthreads();
+    for (int h = 128; h > 0; h >>= 1) {
+      if (tid < h) dl[tid] += dl[tid + h];
+      __syncthreads();
+    }
+    if (tid == 0) *loss = dl[0];
+  }
 }
 
 __global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
@@ -292,11 +518,6 @@ __global__ void pack_net_kernel(const float* __restrict__ params, unsigned char*
     const int ci = 16 * kc + k;
     w[i] = __float2bfloat16_rn(n < CO && ci < CI ? params[base + n * CI * 9 + ci * 9 + tap] : 0.f);
   }
-}
-
-__device__ __forceinline__ int wrap_mod(int i, int n) {
-  i %= n;
-  return i < 0 ? i + n : i;
 }
 
 __device__ __forceinline__ float tanh_approx(float x) {
@@ -838,10 +1059,9 @@ struct lbmhd_closure {
   int adam_t = 0;
   // training scratch (grown on demand)
   size_t cap_cells = 0;
-  float *a1 = nullptr, *a2 = nullptr, *out = nullptr, *d3 = nullptr, *d2 = nullptr, *d1 = nullptr;
-  float* wpart = nullptr;
-  size_t wpart_cap = 0;
-  double* lpart = nullptr;
+  float *a1 = nullptr, *a2 = nullptr, *d3 = nullptr, *d2 = nullptr, *d1 = nullptr;
+  float* wpart = nullptr;   // [kMaxConvBlocks][kNumParams] partial weight gradients
+  double* lpart = nullptr;  // kMaxConvBlocks partial losses, then their sum
   cudaStream_t stream = nullptr;
   std::string err;
 };
@@ -869,20 +1089,50 @@ int cfail(lbmhd_closure_t* c, int code, const char* msg) {
 
 int ensure_scratch(lbmhd_closure_t* c, size_t cells) {
   if (cells <= c->cap_cells) return LBMHD_OK;
-  float** bufs[6] = {&c->a1, &c->a2, &c->out, &c->d3, &c->d2, &c->d1};
-  const int ch[6] = {kC1, kC2, kC3, kC3, kC2, kC1};
-  for (int i = 0; i < 6; ++i) {
+  c->cap_cells = 0;  // nothing usable until every buffer below has grown
+  float** bufs[5] = {&c->a1, &c->a2, &c->d3, &c->d2, &c->d1};
+  const int ch[5] = {kC1, kC2, kC3, kC2, kC1};
+  for (int i = 0; i < 5; ++i) {
     if (*bufs[i]) cudaFree(*bufs[i]);
     *bufs[i] = nullptr;
     CL_CUDA(c, cudaMalloc(bufs[i], cells * ch[i] * sizeof(float)));
   }
-  const size_t nblk = (cells + kWeightCellsPerBlock - 1) / kWeightCellsPerBlock;
-  if (c->wpart) cudaFree(c->wpart);
-  c->wpart = nullptr;
-  CL_CUDA(c, cudaMalloc(&c->wpart, nblk * (size_t)kP2 * sizeof(float)));
-  if (!c->lpart) CL_CUDA(c, cudaMalloc(&c->lpart, 152 * 16 * sizeof(double)));
+  if (!c->wpart) CL_CUDA(c, cudaMalloc(&c->wpart, (size_t)kMaxConvBlocks * kNumParams * sizeof(float)));
+  if (!c->lpart) CL_CUDA(c, cudaMalloc(&c->lpart, (kMaxConvBlocks + 1) * sizeof(double)));
   c->cap_cells = cells;
   return LBMHD_OK;
+}
+
+// Blocks for tiles of kTileW x rows cells.
+int conv_grid(int batch, int H, int W, int rows) {
+  const long tiles = (long)batch * ((H + rows - 1) / rows) * ((W + kTileW - 1) / kTileW);
+  return (int)(tiles < kMaxConvBlocks ? tiles : kMaxConvBlocks);
+}
+
+template <int CIN, int COUT, int EPI, bool BWD = false>
+cudaError_t conv(const float* in, const float* params, const float* aux, int batch, int H, int W, float* out,
+                 double* loss_part, cudaStream_t s) {
+  using Sh = ConvShape<CIN, COUT>;
+  auto k = conv_tile_kernel<CIN, COUT, EPI, BWD>;
+  if (Sh::kSmem > 48 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::kSmem);
+    if (e != cudaSuccess) return e;
+  }
+  k<<<conv_grid(batch, H, W, Sh::kRows), kConvThreads, Sh::kSmem, s>>>(in, params, aux, batch, H, W, out, loss_part);
+  return cudaGetLastError();
+}
+
+template <int NWIN, int NW, bool LANE_DY>
+cudaError_t wgrad(const float* lane_op, const float* win_op, int batch, int H, int W, float* part, int base,
+                  cudaStream_t s) {
+  auto k = conv_wgrad_kernel<NWIN, NW, LANE_DY>;
+  constexpr size_t sm = wgrad_smem<NWIN>();
+  if (sm > 48 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+  }
+  k<<<conv_grid(batch, H, W, kWgRows), kWgThreads, sm, s>>>(lane_op, win_op, batch, H, W, part, base);
+  return cudaGetLastError();
 }
 
 // forward (binary32) + loss + back-propagation into c->grad; *loss = mean squared error / 2
@@ -895,32 +1145,24 @@ int forward_backward(lbmhd_closure_t* c, const float* x, const float* t, int bat
   const float* p1 = c->params;
   const float* p2 = c->params + kP1;
   const float* p3 = c->params + kP1 + kP2;
-  const int g = grid_for((long)cells);
-  conv_fwd_kernel<kC0, kC1, true><<<g, kThreads, 0, s>>>(x, p1, batch, h, w, c->a1);
-  conv_fwd_kernel<kC1, kC2, true><<<g, kThreads, 0, s>>>(c->a1, p2, batch, h, w, c->a2);
-  conv_fwd_kernel<kC2, kC3, false><<<g, kThreads, 0, s>>>(c->a2, p3, batch, h, w, c->out);
-  const long nout = (long)cells * kC3;
-  const int lg = grid_for(nout) < 152 * 16 ? grid_for(nout) : 152 * 16;
-  loss_grad_kernel<<<lg, kThreads, 0, s>>>(c->out, t, nout, c->d3, c->lpart);
-  const int nblk = (int)((cells + kWeightCellsPerBlock - 1) / kWeightCellsPerBlock);
-  // layer 3
-  conv_bwd_weight_kernel<kC2, kC3><<<nblk, kThreads, 0, s>>>(c->d3, c->a2, batch, h, w, c->wpart);
-  sum_partials_kernel<<<grid_for(kP3), kThreads, 0, s>>>(c->wpart, nblk, kP3, c->grad + kP1 + kP2);
-  conv_bwd_data_kernel<kC2, kC3, true><<<g, kThreads, 0, s>>>(c->d3, p3, c->a2, batch, h, w, c->d2);
-  // layer 2
-  conv_bwd_weight_kernel<kC1, kC2><<<nblk, kThreads, 0, s>>>(c->d2, c->a1, batch, h, w, c->wpart);
-  sum_partials_kernel<<<grid_for(kP2), kThreads, 0, s>>>(c->wpart, nblk, kP2, c->grad + kP1);
-  conv_bwd_data_kernel<kC1, kC2, true><<<g, kThreads, 0, s>>>(c->d2, p2, c->a1, batch, h, w, c->d1);
-  // layer 1
-  conv_bwd_weight_kernel<kC0, kC1><<<nblk, kThreads, 0, s>>>(c->d1, x, batch, h, w, c->wpart);
-  sum_partials_kernel<<<grid_for(kP1), kThreads, 0, s>>>(c->wpart, nblk, kP1, c->grad);
+  CL_CUDA(c, (conv<kC0, kC1, kEpiTanh>(x, p1, nullptr, batch, h, w, c->a1, nullptr, s)));
+  CL_CUDA(c, (conv<kC1, kC2, kEpiTanh>(c->a1, p2, nullptr, batch, h, w, c->a2, nullptr, s)));
+  CL_CUDA(c, (conv<kC2, kC3, kEpiLoss>(c->a2, p3, t, batch, h, w, c->d3, c->lpart, s)));
+  // data gradients of layers 3 and 2, weight gradients of all three
+  CL_CUDA(c, (wgrad<kC3, 4, false>(c->a2, c->d3, batch, h, w, c->wpart, kP1 + kP2, s)));
+  CL_CUDA(c, (conv<kC3, kC2, kEpiTanhGrad, true>(c->d3, p3, c->a2, batch, h, w, c->d2, nullptr, s)));
+  CL_CUDA(c, (wgrad<kC1, 4, true>(c->d2, c->a1, batch, h, w, c->wpart, kP1, s)));
+  CL_CUDA(c, (conv<kC2, kC1, kEpiTanhGrad, true>(c->d2, p2, c->a1, batch, h, w, c->d1, nullptr, s)));
+  CL_CUDA(c, (wgrad<kC0, 3, true>(c->d1, x, batch, h, w, c->wpart, 0, s)));
+  double* total = c->lpart + kMaxConvBlocks;
+  sum_partials_kernel<<<(kNumParams + 31) / 32, dim3(32, 8), 0, s>>>(
+      c->wpart, conv_grid(batch, h, w, kWgRows), c->grad, c->lpart,
+      conv_grid(batch, h, w, ConvShape<kC2, kC3>::kRows), total);
   CL_CUDA(c, cudaGetLastError());
-  std::vector<double> lp(lg);
-  CL_CUDA(c, cudaMemcpyAsync(lp.data(), c->lpart, lg * sizeof(double), cudaMemcpyDeviceToHost, s));
-  CL_CUDA(c, cudaStreamSynchronize(s));
   double sum = 0.0;
-  for (double v : lp) sum += v;
-  if (loss) *loss = 0.5 * sum / (double)nout;
+  CL_CUDA(c, cudaMemcpyAsync(&sum, total, sizeof sum, cudaMemcpyDeviceToHost, s));
+  CL_CUDA(c, cudaStreamSynchronize(s));
+  if (loss) *loss = 0.5 * sum / (double)(cells * kC3);
   return LBMHD_OK;
 }
 
@@ -934,8 +1176,8 @@ int repack(lbmhd_closure_t* c) {
 void destroy_closure(lbmhd_closure_t* c) {
   if (!c) return;
   if (c->stream) cudaStreamSynchronize(c->stream);
-  float* bufs[] = {c->params, c->grad, c->adam_m, c->adam_v, c->scales, c->a1, c->a2, c->out, c->d3,
-                   c->d2, c->d1, c->wpart};
+  float* bufs[] = {c->params, c->grad, c->adam_m, c->adam_v, c->scales, c->a1, c->a2, c->d3, c->d2,
+                   c->d1, c->wpart};
   for (float* b : bufs)
     if (b) cudaFree(b);
   if (c->lpart) cudaFree(c->lpart);
@@ -1041,20 +1283,16 @@ int lbmhd_closure_forward(lbmhd_closure_t* c, const float* x, int batch, int h, 
                           int tensor_cores) {
   if (!c || !x || !out) return cfail(c, LBMHD_ERR_INVALID, "NULL argument");
   if (batch < 1 || h < 1 || w < 1) return cfail(c, LBMHD_ERR_INVALID, "empty batch");
-  const size_t cells = (size_t)batch * h * w;
-  int rc = ensure_scratch(c, cells);
-  if (rc) return rc;
-  const float* p1 = c->params;
-  const float* p2 = c->params + kP1;
-  const float* p3 = c->params + kP1 + kP2;
   cudaStream_t s = c->stream;
   if (tensor_cores) {
     CL_CUDA(c, launch_net(x, c->packed, nullptr, batch, h, w, out, c->tc_err, c->test_skip_mma, s));
   } else {
-    const int g = grid_for((long)cells);
-    conv_fwd_kernel<kC0, kC1, true><<<g, kThreads, 0, s>>>(x, p1, batch, h, w, c->a1);
-    conv_fwd_kernel<kC1, kC2, true><<<g, kThreads, 0, s>>>(c->a1, p2, batch, h, w, c->a2);
-    conv_fwd_kernel<kC2, kC3, false><<<g, kThreads, 0, s>>>(c->a2, p3, batch, h, w, out);
+    int rc = ensure_scratch(c, (size_t)batch * h * w);
+    if (rc) return rc;
+    const float* p = c->params;
+    CL_CUDA(c, (conv<kC0, kC1, kEpiTanh>(x, p, nullptr, batch, h, w, c->a1, nullptr, s)));
+    CL_CUDA(c, (conv<kC1, kC2, kEpiTanh>(c->a1, p + kP1, nullptr, batch, h, w, c->a2, nullptr, s)));
+    CL_CUDA(c, (conv<kC2, kC3, kEpiNone>(c->a2, p + kP1 + kP2, nullptr, batch, h, w, out, nullptr, s)));
   }
   CL_CUDA(c, cudaGetLastError());
   CL_CUDA(c, cudaStreamSynchronize(s));
