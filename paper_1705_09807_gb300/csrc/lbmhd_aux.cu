@@ -140,34 +140,125 @@ __device__ __forceinline__ void pull_cell(const T* __restrict__ pops, const Step
   }
 }
 
+// Exact binary64 value of a binary32 number by integer operations: GB300 converts binary32 to
+// binary64 at its binary64 rate (1/74 of its integer rate).  Subnormals, infinities and NaN take
+// the conversion instruction.
+__device__ __forceinline__ double widen(float f) {
+  const uint32_t b = __float_as_uint(f), a = b & 0x7fffffffu;
+  if (a - 0x00800000u >= 0x7f000000u && a != 0u) return (double)f;
+  const uint32_t hi = a == 0u ? 0u : (a >> 3) + 0x38000000u;
+  return __hiloint2double((int)((b & 0x80000000u) | hi), (int)(a << 29));
+}
+
 // Sum of binary32 values kept exactly as the unevaluated pair hi + lo (Knuth's TwoSum: the
 // rounding error of each binary32 addition is itself a binary32 value).  Nine stored binary32 or
 // binary16 values sum to the binary64 result up to one rounding of lo, with binary32 arithmetic
-// only: GB300's binary64 rate (about 1/60 of binary32) made the binary64 sums of the moments
-// read-out take 0.55 ms at 2048^2, four times the kernel's memory time.
+// only.  EXACT: the caller knows that hi + v never rounds, so lo stays zero.
 struct PairSum {
   float hi = 0.f, lo = 0.f;
+  template <bool EXACT = false>
   __device__ __forceinline__ void add(float v) {
-    const float s = hi + v, bv = s - hi;
-    lo += (hi - (s - bv)) + (v - bv);
+    const float s = hi + v;
+    if constexpr (!EXACT) {
+      const float bv = s - hi;
+      lo += (hi - (s - bv)) + (v - bv);
+    }
     hi = s;
   }
-  __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+  template <bool EXACT = false>
+  __device__ __forceinline__ double value() const {
+    return EXACT ? widen(hi) : widen(hi) + widen(lo);
+  }
+  __device__ __forceinline__ float rounded() const { return hi + lo; }
+  // hi + lo + n / 12 rounded to binary32 (n a pair): quotient and remainder, then one TwoSum
+  __device__ __forceinline__ float plus_twelfth(const PairSum& n) const {
+    const float r12 = 1.f / 12.f, q = __fmul_rn(n.hi, r12);  // rounded: TwoSum needs the value
+    const float ql = (fmaf(-12.f, q, n.hi) + n.lo) * r12;
+    PairSum t = *this;
+    t.add(q);
+    return t.hi + (t.lo + ql);
+  }
 };
 
+// rho, u, B of one cell from its 27 pulled binary32 values (f as stored deviations; REL: relative
+// to w_i (1 + 3 c_i . U), with U[k] = {U_x, U_y} of the source cell of f_(k+1)).
+template <bool EXACT, bool REL>
+__device__ __forceinline__ void moments_of(const float (&v)[27], const float (&U)[8][2], double (&out)[5]) {
+  PairSum r, px, py, qx, qy;
+#pragma unroll
+  for (int i = 0; i < 9; ++i) {
+    r.add<EXACT>(v[i]);
+    if (vx(i)) px.add<EXACT>(vx(i) > 0 ? v[i] : -v[i]);
+    if (vy(i)) py.add<EXACT>(vy(i) > 0 ? v[i] : -v[i]);
+    qx.add<EXACT>(v[9 + i]);
+    qy.add<EXACT>(v[18 + i]);
+  }
+  float jx, jy;
+  if constexpr (REL) {
+    // sum_i (1, c_i) 3 w_i c_i . U(x - c_i) = n / 12 with integer coefficients: 3 w_i is 4/12 on
+    // the axes and 1/12 on the diagonals
+    PairSum nr, nx, ny;
+#pragma unroll
+    for (int i = 1; i < 9; ++i) {
+      const float k = i < 5 ? 4.f : 1.f;
+#pragma unroll
+      for (int comp = 0; comp < 2; ++comp) {
+        const int c = comp ? vy(i) : vx(i);
+        if (c == 0) continue;
+        const float t = k * (c > 0 ? U[i - 1][comp] : -U[i - 1][comp]);
+        nr.add(t);
+        if (vx(i)) nx.add(vx(i) > 0 ? t : -t);
+        if (vy(i)) ny.add(vy(i) > 0 ? t : -t);
+      }
+    }
+    out[0] = 1.0 + fma(nr.value(), 1.0 / 12.0, r.value<EXACT>());
+    jx = px.plus_twelfth(nx);
+    jy = py.plus_twelfth(ny);
+    const float q = __fmul_rn(nr.hi, 1.f / 12.f);  // for the binary32 division below
+    r.add(q);
+    r.lo += (fmaf(-12.f, q, nr.hi) + nr.lo) * (1.f / 12.f);
+  } else {
+    out[0] = 1.0 + r.value<EXACT>();
+    jx = px.rounded();
+    jy = py.rounded();
+  }
+  PairSum rr;
+  rr.hi = 1.f;
+  rr.add(r.hi);
+  rr.lo += r.lo;
+  const float ir = 1.f / rr.rounded();  // binary32: GB300's binary64 divide is slow
+  out[1] = widen(jx * ir);
+  out[2] = widen(jy * ir);
+  out[3] = qx.value<EXACT>();
+  out[4] = qy.value<EXACT>();
+}
+
+// Macroscopic fields.  One cell per thread, rows of a block's columns; the ghost columns hold the
+// periodic x-neighbours, so a cell's 27 values are at fixed offsets from its three rows.  For
+// binary32 and binary16 storage the sums are exact binary32 pairs, and only what a result
+// cannot do without is binary64 (four additions per cell, one for binary16): with conversions and
+// additions of every sum in binary64 the binary64 units set the time.  Binary16 values are
+// multiples of 2^-24, so while a sum's magnitudes add up to at most 1 (|f_i - w_i|, |g_i| ~ 0.1
+// in any flow this model is valid for) plain binary32 additions are exact and the pairs are not
+// needed; other cells take them.  @@MOM@@
 template <typename T, bool REL = false>
-__global__ void moments_kernel(const T* __restrict__ pops, StepGeom g, double* __restrict__ rho,
-                               double* __restrict__ ux, double* __restrict__ uy,
-                               double* __restrict__ bx, double* __restrict__ by) {
-  const long n = (long)g.nx * g.ny;
-  for (long c = blockIdx.x * (long)blockDim.x + threadIdx.x; c < n; c += (long)gridDim.x * blockDim.x) {
-    const int x = (int)(c % g.nx), y = (int)(c / g.nx);
-    double rr, jx, jy, sbx, sby;
-    if constexpr (sizeof(T) == 8 || REL) {  // binary64 sums (REL: the decoded values are binary64)
+__global__ void __launch_bounds__(128)
+    moments_kernel(const T* __restrict__ pops, StepGeom g, double* __restrict__ rho, double* __restrict__ ux,
+                   double* __restrict__ uy, double* __restrict__ bx, double* __restrict__ by) {
+  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  if (x >= g.nx) return;
+  for (int y = blockIdx.y; y < g.ny; y += gridDim.y) {
+    const T* rows[3];  // rows y - 1, y, y + 1 (sources of c_y = 1, 0, -1) at column x
+#pragma unroll
+    for (int k = 0; k < 3; ++k) rows[k] = pops + (size_t)wrapi(y - 1 + k, g.ny) * g.pitch + kXOff + x;
+    auto at = [&](int plane, int i) { return rows[1 - vy(i)][(size_t)plane * g.plane - vx(i)]; };
+    const size_t c = (size_t)y * g.nx + x;
+    double out[5];
+    if constexpr (sizeof(T) == 8) {
       double v[27];
-      pull_cell<T, REL>(pops, g, x, y, v);
-      double r = 0;
-      jx = jy = sbx = sby = 0;
+#pragma unroll
+      for (int q = 0; q < 27; ++q) v[q] = at(plane_of(q), q % 9);
+      double r = 0, jx = 0, jy = 0, sbx = 0, sby = 0;
 #pragma unroll
       for (int i = 0; i < 9; ++i) {
         r += v[i];
@@ -176,41 +267,37 @@ __global__ void moments_kernel(const T* __restrict__ pops, StepGeom g, double* _
         sbx += v[9 + i];
         sby += v[18 + i];
       }
-      rr = 1.0 + r;
-    } else {  // binary32 / binary16 storage: exact binary32 pair sums of the pulled values
-      PairSum r, px, py, qx, qy;
+      out[0] = 1.0 + r;
+      out[1] = jx / out[0];
+      out[2] = jy / out[0];
+      out[3] = sbx;
+      out[4] = sby;
+    } else {
+      float v[27], U[8][2] = {};
 #pragma unroll
-      for (int q = 0; q < 27; ++q) {
-        const int i = q % 9;
-        const int sx = wrapi(x - vx(i), g.nx), sy = wrapi(y - vy(i), g.ny);
-        const float v = load_as<float>(pops[(size_t)plane_of(q) * g.plane + (size_t)sy * g.pitch + kXOff + sx]);
-        if (q < 9) {
-          r.add(v);
-          if (vx(i)) px.add(vx(i) > 0 ? v : -v);
-          if (vy(i)) py.add(vy(i) > 0 ? v : -v);
-        } else if (q < 18) {
-          qx.add(v);
-        } else {
-          qy.add(v);
+      for (int q = 0; q < 27; ++q) v[q] = load_as<float>(at(plane_of(q), q % 9));
+      if constexpr (REL) {
+#pragma unroll
+        for (int i = 1; i < 9; ++i) {
+          if (vx(i)) U[i - 1][0] = load_as<float>(at(kQ, i));
+          if (vy(i)) U[i - 1][1] = load_as<float>(at(kQ + 1, i));
         }
       }
-      rr = 1.0 + r.value();
-      jx = px.value();
-      jy = py.value();
-      sbx = qx.value();
-      sby = qy.value();
+      if constexpr (sizeof(T) == 2) {
+        float a[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+        for (int q = 0; q < 27; ++q) a[q / 9] += fabsf(v[q]);
+        if (a[0] <= 1.f && a[1] <= 1.f && a[2] <= 1.f) moments_of<true, REL>(v, U, out);
+        else moments_of<false, REL>(v, U, out);
+      } else {
+        moments_of<false, REL>(v, U, out);
+      }
     }
-    rho[c] = rr;
-    if (sizeof(T) == 8) {
-      ux[c] = jx / rr;
-      uy[c] = jy / rr;
-    } else {  // binary32 / binary16 storage: a binary32 division (GB300's binary64 divide is slow)
-      const float ir = 1.f / (float)rr;
-      ux[c] = (double)((float)jx * ir);
-      uy[c] = (double)((float)jy * ir);
-    }
-    bx[c] = sbx;
-    by[c] = sby;
+    rho[c] = out[0];
+    ux[c] = out[1];
+    uy[c] = out[2];
+    bx[c] = out[3];
+    by[c] = out[4];
   }
 }
 
@@ -365,15 +452,16 @@ cudaError_t launch_zero_pads(void* pops0, void* pops1, const StepGeom& g, int np
 
 cudaError_t launch_moments(int precision, const void* pops, const StepGeom& g, double* rho,
                            double* ux, double* uy, double* bx, double* by, cudaStream_t s) {
-  const int grid = grid_for((long)g.nx * g.ny, 256);
+  const int nt = std::min(128, (g.nx + 31) / 32 * 32);
+  const dim3 grid((g.nx + nt - 1) / nt, (unsigned)std::min(g.ny, 65535));
   if (precision == 0)
-    moments_kernel<double><<<grid, 256, 0, s>>>((const double*)pops, g, rho, ux, uy, bx, by);
+    moments_kernel<double><<<grid, nt, 0, s>>>((const double*)pops, g, rho, ux, uy, bx, by);
   else if (precision == 1)
-    moments_kernel<float><<<grid, 256, 0, s>>>((const float*)pops, g, rho, ux, uy, bx, by);
+    moments_kernel<float><<<grid, nt, 0, s>>>((const float*)pops, g, rho, ux, uy, bx, by);
   else if (precision == LBMHD_FP16)
-    moments_kernel<__half><<<grid, 256, 0, s>>>((const __half*)pops, g, rho, ux, uy, bx, by);
+    moments_kernel<__half><<<grid, nt, 0, s>>>((const __half*)pops, g, rho, ux, uy, bx, by);
   else
-    moments_kernel<__half, true><<<grid, 256, 0, s>>>((const __half*)pops, g, rho, ux, uy, bx, by);
+    moments_kernel<__half, true><<<grid, nt, 0, s>>>((const __half*)pops, g, rho, ux, uy, bx, by);
   return cudaGetLastError();
 }
 
