@@ -311,8 +311,8 @@ int64_t lbmhd_step_count(const lbmhd_t* h);
  * lbmhd_diagnostics, then 1.0 if any cell has NaN/Inf, rho <= 0 or |u| > 0.4, else 0.0.
  * Enqueued on `stream` (a cudaStream_t; NULL = the legacy default stream); no synchronisation.
  *
- * It calls no cudaMalloc/cudaFree or other allocating routine: its scratch (one partial record
- * per 4096 cells) is a fixed 352 KiB device array of the library, resident on every GPU that
+ * It calls no cudaMalloc/cudaFree or other allocating routine: its scratch (4096 partial
+ * records) is a fixed 352 KiB device array of the library, resident on every GPU that
  * loads the library until the process exits.  Hence at most 4096 x 4096 = 16,777,216 cells;
  * larger grids, sides < 3 and NULL pointers return LBMHD_ERR_INVALID (see lbmhd_last_error(NULL)).
  * The first call in a device's context looks up that array's device address (with the device

@@ -3,6 +3,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "lbmhd_diag.cuh"
 #include "lbmhd_internal.cuh"
 
 namespace lbmhd_gpu {
@@ -313,85 +314,6 @@ __global__ void populations_kernel(const T* __restrict__ pops, StepGeom g, doubl
   }
 }
 
-// ---- diagnostics ----------------------------------------------------------------------
-constexpr int kDiagThreads = 256;
-
-__device__ __forceinline__ double iso_d(const double* a, int nx, int ny, int x, int y, int axis) {
-  double s = 0.0;
-#pragma unroll
-  for (int i = 1; i < 9; ++i) {
-    const int c = axis == 0 ? vx(i) : vy(i);
-    if (c == 0) continue;
-    s += 3.0 * wt(i) * c * a[(size_t)wrapi(y + vy(i), ny) * nx + wrapi(x + vx(i), nx)];
-  }
-  return s;
-}
-
-// Slots: 0 sum rho, 1 sum Jx, 2 sum Jy, 3 sum Bx, 4 sum By, 5 sum rho|u|^2/2, 6 sum |B|^2/2,
-// 7 max|div B| isotropic, 8 max|div B| central, 9 max|dB| isotropic, 10 instability flag.
-__global__ void diag_partial_kernel(const double* __restrict__ f, int nx, int ny,
-                                    double* __restrict__ partials) {
-  const long n = (long)nx * ny;
-  const double* rho = f;
-  const double* ux = f + n;
-  const double* uy = f + 2 * n;
-  const double* bx = f + 3 * n;
-  const double* by = f + 4 * n;
-  double acc[kDiagSlots];
-#pragma unroll
-  for (int k = 0; k < kDiagSlots; ++k) acc[k] = 0.0;
-  for (long c = blockIdx.x * (long)blockDim.x + threadIdx.x; c < n; c += (long)gridDim.x * blockDim.x) {
-    const int x = (int)(c % nx), y = (int)(c / nx);
-    const double r = rho[c], u = ux[c], v = uy[c], b = bx[c], d = by[c];
-    acc[0] += r;
-    acc[1] += r * u;
-    acc[2] += r * v;
-    acc[3] += b;
-    acc[4] += d;
-    acc[5] += 0.5 * r * (u * u + v * v);
-    acc[6] += 0.5 * (b * b + d * d);
-    const double dxbx = iso_d(bx, nx, ny, x, y, 0), dybx = iso_d(bx, nx, ny, x, y, 1);
-    const double dxby = iso_d(by, nx, ny, x, y, 0), dyby = iso_d(by, nx, ny, x, y, 1);
-    acc[7] = fmax(acc[7], fabs(dxbx + dyby));
-    const int xp = x + 1 == nx ? 0 : x + 1, xm = x == 0 ? nx - 1 : x - 1;
-    const int yp = y + 1 == ny ? 0 : y + 1, ym = y == 0 ? ny - 1 : y - 1;
-    const double cdiv = 0.5 * (bx[(size_t)y * nx + xp] - bx[(size_t)y * nx + xm] +
-                               by[(size_t)yp * nx + x] - by[(size_t)ym * nx + x]);
-    acc[8] = fmax(acc[8], fabs(cdiv));
-    acc[9] = fmax(acc[9], fmax(fmax(fabs(dxbx), fabs(dybx)), fmax(fabs(dxby), fabs(dyby))));
-    const bool bad = !(isfinite(r) && isfinite(u) && isfinite(v) && isfinite(b) && isfinite(d)) ||
-                     !(r > 0.0) || !(u * u + v * v <= 0.16);
-    if (bad) acc[10] = 1.0;
-  }
-  __shared__ double sh[kDiagSlots][kDiagThreads];
-#pragma unroll
-  for (int k = 0; k < kDiagSlots; ++k) sh[k][threadIdx.x] = acc[k];
-  __syncthreads();
-  for (int w = kDiagThreads / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) {
-#pragma unroll
-      for (int k = 0; k < kDiagSlots; ++k) {
-        const double a = sh[k][threadIdx.x], b = sh[k][threadIdx.x + w];
-        sh[k][threadIdx.x] = (k <= 6) ? a + b : fmax(a, b);
-      }
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x < kDiagSlots) partials[(size_t)blockIdx.x * kDiagSlots + threadIdx.x] = sh[threadIdx.x][0];
-}
-
-__global__ void diag_final_kernel(const double* __restrict__ partials, int nblocks,
-                                  double* __restrict__ out) {
-  const int k = threadIdx.x;
-  if (k >= kDiagSlots) return;
-  double a = 0.0;
-  for (int b = 0; b < nblocks; ++b) {
-    const double v = partials[(size_t)b * kDiagSlots + k];
-    a = (k <= 6) ? a + v : fmax(a, v);
-  }
-  out[k] = a;
-}
-
 int grid_for(long n, int threads) {
   long b = (n + threads - 1) / threads;
   if (b > 152L * 16) b = 152L * 16;
@@ -481,10 +403,13 @@ cudaError_t launch_populations(int precision, const void* pops, const StepGeom& 
 
 cudaError_t launch_diagnostics(const double* fields, int nx, int ny, double* partials, double* out,
                                cudaStream_t s) {
-  diag_partial_kernel<<<kDiagBlocks, kDiagThreads, 0, s>>>(fields, nx, ny, partials);
+  const size_t n = (size_t)nx * ny;
+  const DiagTiles t = diag_tiles(nx, ny, kDiagBlocks);
+  diag_partial_kernel<<<t.blocks, kDiagThreads, 0, s>>>(fields, fields + n, fields + 2 * n, fields + 3 * n,
+                                                         fields + 4 * n, nx, ny, t, partials);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  diag_final_kernel<<<1, 32, 0, s>>>(partials, kDiagBlocks, out);
+  diag_final_kernel<<<1, 32 * kDiagSlots, 0, s>>>(partials, t.blocks, out);
   return cudaGetLastError();
 }
 

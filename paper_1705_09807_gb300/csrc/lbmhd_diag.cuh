@@ -1,0 +1,151 @@
+// Diagnostics reduction over five device moment fields rho, ux, uy, bx, by [ny][nx] (periodic),
+// shared by lbmhd_diagnostics (moment fields of a handle) and lbmhd_diagnostics_fields_noalloc.
+//
+// Slots of a record: 0 sum rho, 1 sum Jx, 2 sum Jy, 3 sum Bx, 4 sum By, 5 sum rho |u|^2 / 2,
+// 6 sum |B|^2 / 2, 7 max |div B| (isotropic), 8 max |div B| (central), 9 max |d_beta B_alpha|
+// (isotropic), 10 instability flag.  Maxima skip NaN (the flag reports it), as fmax does.
+//
+// Bound by GB300's binary64 rate (528 G instructions/s; the 40 bytes per cell would take 25 us at
+// 2048^2), so the work is arranged for few binary64 instructions, 25 per cell against about 60
+// with each derivative summed from its six neighbours: a thread marches down one column of a
+// 128-column tile and forms each row's x-difference D = a(x+1) - a(x-1) and weighted sum
+// S = a(x) + (a(x-1) + a(x+1)) / 4 once, from which the isotropic derivatives of row y are
+// 3 d_x = D(y) + (D(y-1) + D(y+1)) / 4 and 3 d_y = S(y+1) - S(y-1); scales are applied once at the
+// end; maxima and the stability tests compare bit patterns with integer instructions.
+// 2048^2, cold caches: 444 us and 42 us for the final record before, 279 and 13 us now.
+#pragma once
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "lbmhd_internal.cuh"
+
+namespace lbmhd_gpu {
+
+constexpr int kDiagThreads = 128;  // columns of a tile
+constexpr int kDiagMinRows = 4;    // rows of a tile, at least (halo rows are formed twice)
+
+// Tiles of kDiagThreads columns x `rows` rows: as few rows as keep the tiles within max_blocks.
+struct DiagTiles {
+  int strips, rows, blocks;
+  long tiles;
+};
+inline DiagTiles diag_tiles(int nx, int ny, int max_blocks) {
+  DiagTiles t;
+  t.strips = (nx + kDiagThreads - 1) / kDiagThreads;
+  const long rows = ((long)t.strips * ny + max_blocks - 1) / max_blocks;
+  t.rows = (int)(rows < kDiagMinRows ? kDiagMinRows : (rows > ny ? ny : rows));
+  t.tiles = (long)t.strips * ((ny + t.rows - 1) / t.rows);
+  t.blocks = (int)(t.tiles < max_blocks ? t.tiles : max_blocks);
+  return t;
+}
+
+namespace {
+
+// Bits of |v|, ordered like the values; NaN as 0.
+__device__ __forceinline__ unsigned long long abs_bits(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+  return b > 0x7ff0000000000000ull ? 0ull : b;
+}
+__device__ __forceinline__ bool not_finite(double v) { return (__double2hiint(v) & 0x7ff00000) == 0x7ff00000; }
+
+// Combine two records' slot k (max for the non-negative maxima and the flag).
+__device__ __forceinline__ double diag_combine(int k, double a, double b) { return k <= 6 ? a + b : (b > a ? b : a); }
+
+// One record per block into partials[blockIdx.x].
+__global__ void __launch_bounds__(kDiagThreads)
+    diag_partial_kernel(const double* __restrict__ rho, const double* __restrict__ ux, const double* __restrict__ uy,
+                        const double* __restrict__ bx, const double* __restrict__ by, int nx, int ny, DiagTiles t,
+                        double* __restrict__ partials) {
+  double sum[7];
+  unsigned long long mx[3] = {0, 0, 0};
+  bool bad = false;
+#pragma unroll
+  for (int k = 0; k < 7; ++k) sum[k] = 0.0;
+  for (long tile = blockIdx.x; tile < t.tiles; tile += gridDim.x) {
+    const int x = (int)(tile % t.strips) * kDiagThreads + threadIdx.x;
+    const int y0 = (int)(tile / t.strips) * t.rows, y1 = min(y0 + t.rows, ny);
+    if (x >= nx) continue;
+    const int xe = x + 1 == nx ? 0 : x + 1, xw = x == 0 ? nx - 1 : x - 1;
+    // rows y - 1, y, y + 1 in slots 0, 1, 2: value, D and S of B_x and B_y
+    double a[2][3], D[2][3], S[2][3];
+    auto row = [&](int y, int k) {
+      const size_t o = (size_t)(y < 0 ? y + ny : (y >= ny ? y - ny : y)) * nx;
+#pragma unroll
+      for (int f = 0; f < 2; ++f) {
+        const double* p = (f ? by : bx) + o;
+        const double e = p[xe], w = p[xw];
+        a[f][k] = p[x];
+        D[f][k] = e - w;
+        S[f][k] = fma(0.25, e + w, a[f][k]);
+      }
+    };
+    row(y0 - 1, 0);
+    row(y0, 1);
+    for (int y = y0; y < y1; ++y) {
+      row(y + 1, 2);
+      const size_t c = (size_t)y * nx + x;
+      const double r = rho[c], u = ux[c], v = uy[c], b = a[0][1], d = a[1][1];
+      const double q = fma(u, u, v * v);
+      sum[0] += r;
+      sum[1] = fma(r, u, sum[1]);
+      sum[2] = fma(r, v, sum[2]);
+      sum[3] += b;
+      sum[4] += d;
+      sum[5] = fma(r, q, sum[5]);
+      sum[6] = fma(b, b, fma(d, d, sum[6]));
+      double dx[2], dy[2];  // three times the isotropic derivatives
+#pragma unroll
+      for (int f = 0; f < 2; ++f) {
+        dx[f] = fma(0.25, D[f][0] + D[f][2], D[f][1]);
+        dy[f] = S[f][2] - S[f][0];
+      }
+      mx[0] = max(mx[0], abs_bits(dx[0] + dy[1]));
+      mx[1] = max(mx[1], abs_bits(D[0][1] + (a[1][2] - a[1][0])));
+      mx[2] = max(max(mx[2], max(abs_bits(dx[0]), abs_bits(dy[0]))), max(abs_bits(dx[1]), abs_bits(dy[1])));
+      // not (rho > 0 and |u|^2 <= 0.16), or anything not finite
+      bad = bad || not_finite(r) || not_finite(u) || not_finite(v) || not_finite(b) || not_finite(d) ||
+            __double_as_longlong(r) <= 0 || __double_as_longlong(q) > __double_as_longlong(0.16);
+#pragma unroll
+      for (int f = 0; f < 2; ++f)
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          a[f][k] = a[f][k + 1];
+          D[f][k] = D[f][k + 1];
+          S[f][k] = S[f][k + 1];
+        }
+    }
+  }
+  __shared__ double sh[kDiagSlots][kDiagThreads];
+#pragma unroll
+  for (int k = 0; k < 7; ++k) sh[k][threadIdx.x] = (k >= 5 ? 0.5 : 1.0) * sum[k];
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+    sh[7 + k][threadIdx.x] = (k == 1 ? 0.5 : 1.0 / 3.0) * __longlong_as_double((long long)mx[k]);
+  sh[10][threadIdx.x] = bad ? 1.0 : 0.0;
+  __syncthreads();
+  for (int w = kDiagThreads / 2; w > 0; w >>= 1) {
+    if ((int)threadIdx.x < w) {
+#pragma unroll
+      for (int k = 0; k < kDiagSlots; ++k)
+        sh[k][threadIdx.x] = diag_combine(k, sh[k][threadIdx.x], sh[k][threadIdx.x + w]);
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x < kDiagSlots) partials[(size_t)blockIdx.x * kDiagSlots + threadIdx.x] = sh[threadIdx.x][0];
+}
+
+// out[k] = records combined in a fixed order: warp k takes slot k, each lane every 32nd record,
+// then the lanes by halves.  (One thread per slot took 42 us for 304 records.)
+__global__ void __launch_bounds__(32 * kDiagSlots)
+    diag_final_kernel(const double* __restrict__ partials, int nblocks, double* __restrict__ out) {
+  const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double a = 0.0;
+#pragma unroll 4
+  for (int b = lane; b < nblocks; b += 32) a = diag_combine(k, a, partials[(size_t)b * kDiagSlots + k]);
+  for (int w = 16; w > 0; w >>= 1) a = diag_combine(k, a, __shfl_down_sync(0xffffffffu, a, w));
+  if (lane == 0) out[k] = a;
+}
+
+}  // namespace
+}  // namespace lbmhd_gpu

@@ -150,10 +150,10 @@ cudaError_t launch_moments(int precision, const void* pops, const StepGeom& g, d
 cudaError_t launch_populations(int precision, const void* pops, const StepGeom& g, double* out,
                                cudaStream_t s);
 // Diagnostics over the five moment fields (rho, ux, uy, bx, by, each nx*ny, contiguous):
-// block partials into `partials` (kDiagBlocks x kDiagSlots doubles), then a single-block
-// fixed-order reduction into out[kDiagSlots] (device).
-constexpr int kDiagBlocks = 304;
-constexpr int kDiagSlots = 11;  // 10 public values + instability flag
+// block partials into `partials` (kDiagBlocks x kDiagSlots doubles, lbmhd_diag.cuh), then a
+// single-block fixed-order reduction into out[kDiagSlots] (device).
+constexpr int kDiagBlocks = 1024;
+constexpr int kDiagSlots = LBMHD_NDIAG + 1;  // the public values and the instability flag
 cudaError_t launch_diagnostics(const double* fields, int nx, int ny, double* partials,
                                double* out, cudaStream_t s);
 
