@@ -913,107 +913,158 @@ cudaError_t launch_net(const float* in, const unsigned char* packed, const float
 // Coarse moments of a fine state by r x r box filter, including the filtered nonlinear products:
 // out planes [0..4] = rho, Jx, Jy, Bx, By; [5] JxJy/rho - BxBy; [6] (Jx^2-Jy^2)/rho - (Bx^2-By^2);
 // [7] (Jx^2+Jy^2)/rho; [8] (Jx By - Jy Bx)/rho.
-__global__ void filter_products_kernel(const double* __restrict__ fine, int n, int r,
-                                       double* __restrict__ coarse) {
+//
+// Bound by GB300's binary64 rate, not by the 40 bytes per fine cell: with J = rho u the quotients
+// are products (J_x J_y / rho = J_x u_y, ...), 17 binary64 instructions per fine cell instead of
+// about 57 with four divisions.  A thread adds up one fine column of a coarse row, so the loads
+// are coalesced and a coarse cell occupies r threads; the r columns are then added in order.
+// 2048^2, r = 8, cold caches: 481 -> 147 us.
+constexpr int kFilterThreads = 128;
+__global__ void __launch_bounds__(kFilterThreads)
+    filter_products_kernel(const double* __restrict__ fine, int n, int r, double* __restrict__ coarse) {
+  __shared__ double sh[9][kFilterThreads];
   const int m = n / r;
-  const long mm = (long)m * m, nn = (long)n * n;
+  const size_t mm = (size_t)m * m, nn = (size_t)n * n;
   const double inv = 1.0 / ((double)r * r);
-  for (long c = blockIdx.x * (long)blockDim.x + threadIdx.x; c < mm; c += (long)gridDim.x * blockDim.x) {
-    const int i = (int)(c % m), j = (int)(c / m);
-    double s[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-    for (int yy = 0; yy < r; ++yy)
-      for (int xx = 0; xx < r; ++xx) {
-        const size_t f = (size_t)(j * r + yy) * n + (size_t)(i * r + xx);
-        const double rho = fine[f], ux = fine[nn + f], uy = fine[2 * nn + f], bx = fine[3 * nn + f],
-                     by = fine[4 * nn + f];
-        const double jx = rho * ux, jy = rho * uy;
-        s[0] += rho;
-        s[1] += jx;
-        s[2] += jy;
-        s[3] += bx;
-        s[4] += by;
-        s[5] += jx * jy / rho - bx * by;
-        s[6] += (jx * jx - jy * jy) / rho - (bx * bx - by * by);
-        s[7] += (jx * jx + jy * jy) / rho;
-        s[8] += (jx * by - jy * bx) / rho;
+  // whole coarse cells per block; filters wider than the block take several passes of columns
+  const int cells = r <= kFilterThreads ? kFilterThreads / r : 1;
+  for (int j = blockIdx.y; j < m; j += gridDim.y) {
+    const int i0 = blockIdx.x * cells;
+    const int cols = min(cells, m - i0) * r;
+    double tot[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+    for (int c0 = 0; c0 < cols; c0 += kFilterThreads) {
+      const int x = c0 + (int)threadIdx.x, w = min(kFilterThreads, cols - c0);
+      double s[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0}, a = 0, b = 0, c = 0, d = 0;
+      if (x < cols) {
+        const double* p = fine + (size_t)j * r * n + (size_t)i0 * r + x;
+        for (int yy = 0; yy < r; ++yy, p += n) {
+          const double rho = p[0], ux = p[nn], uy = p[2 * nn], bx = p[3 * nn], by = p[4 * nn];
+          const double jx = rho * ux, jy = rho * uy;
+          s[0] += rho;
+          s[1] += jx;
+          s[2] += jy;
+          s[3] += bx;
+          s[4] += by;
+          s[5] = fma(jx, uy, fma(-bx, by, s[5]));
+          a = fma(jx, ux, a);
+          b = fma(jy, uy, b);
+          c = fma(bx, bx, c);
+          d = fma(by, by, d);
+          s[8] = fma(ux, by, fma(-uy, bx, s[8]));
+        }
+        s[6] = (a - b) - (c - d);
+        s[7] = a + b;
       }
-    for (int k = 0; k < 9; ++k) coarse[(size_t)k * mm + c] = s[k] * inv;
+#pragma unroll
+      for (int k = 0; k < 9; ++k) sh[k][threadIdx.x] = s[k];
+      __syncthreads();
+      // coarse cell t of the block (one when r exceeds the block): its columns of this pass
+      const int first = r <= kFilterThreads ? threadIdx.x * r : 0, num = r <= kFilterThreads ? r : w;
+      if ((int)threadIdx.x < (r <= kFilterThreads ? cols / r : 1)) {
+        for (int q = 0; q < num; ++q)
+#pragma unroll
+          for (int k = 0; k < 9; ++k) tot[k] += sh[k][first + q];
+      }
+      __syncthreads();
+    }
+    if ((int)threadIdx.x < cols / r) {
+#pragma unroll
+      for (int k = 0; k < 9; ++k) coarse[k * mm + (size_t)j * m + i0 + threadIdx.x] = tot[k] * inv;
+    }
   }
-}
-
-__device__ __forceinline__ double cdiff(const double* a, int m, int x, int y, int axis) {
-  return axis == 0 ? 0.5 * (a[(size_t)y * m + wrapi(x + 1, m)] - a[(size_t)y * m + wrapi(x - 1, m)])
-                   : 0.5 * (a[(size_t)wrapi(y + 1, m) * m + x] - a[(size_t)wrapi(y - 1, m) * m + x]);
 }
 
 // Features (12 channels: u, B and their central differences, each over its scale) of a coarse
-// state given as rho, Jx, Jy, Bx, By planes (J = rho u); optionally the analytic closure a0..a3
-// (k = delta^2/12) into `analytic` (4 planes), and, when `products` is given (planes 5..8 of
-// filter_products_kernel), the training target (c - a)/out_scale into `target`.
-__global__ void features_kernel(const double* __restrict__ st, int m, int velocity,
-                                const float* __restrict__ in_scale, const float* __restrict__ out_scale,
-                                double kd, float* __restrict__ x, float* __restrict__ analytic,
-                                const double* __restrict__ products, float* __restrict__ target) {
-  const long mm = (long)m * m;
-  const double* rho = st;
-  const double* p1 = st + mm;  // J_x, or u_x when `velocity`
-  const double* p2 = st + 2 * mm;
-  const double* bx = st + 3 * mm;
-  const double* by = st + 4 * mm;
-  auto jval = [&](int f, size_t o) -> double {  // J_x (f = 0) or J_y (f = 1) at cell o
-    const double v = f == 0 ? p1[o] : p2[o];
-    return velocity ? rho[o] * v : v;
-  };
-  auto uval = [&](int f, size_t o) -> double {  // u_x, u_y, B_x, B_y at cell o
-    if (f >= 2) return f == 2 ? bx[o] : by[o];
-    const double v = f == 0 ? p1[o] : p2[o];
-    return velocity ? v : v / rho[o];
-  };
-  for (long c = blockIdx.x * (long)blockDim.x + threadIdx.x; c < mm; c += (long)gridDim.x * blockDim.x) {
-    const int i = (int)(c % m), j = (int)(c / m);
-    const size_t xe = (size_t)j * m + wrapi(i + 1, m), xw = (size_t)j * m + wrapi(i - 1, m);
-    const size_t yn = (size_t)wrapi(j + 1, m) * m + i, ys = (size_t)wrapi(j - 1, m) * m + i;
-    // gradients of u and B for the features; of J and B for the closure
-    double u[4], du[8], gj[4], gb[4];
-    const double r0 = rho[c];
-    for (int f = 0; f < 4; ++f) {
-      u[f] = uval(f, c);
-      du[2 * f] = 0.5 * (uval(f, xe) - uval(f, xw));
-      du[2 * f + 1] = 0.5 * (uval(f, yn) - uval(f, ys));
-    }
-    gj[0] = 0.5 * (jval(0, xe) - jval(0, xw));
-    gj[1] = 0.5 * (jval(0, yn) - jval(0, ys));
-    gj[2] = 0.5 * (jval(1, xe) - jval(1, xw));
-    gj[3] = 0.5 * (jval(1, yn) - jval(1, ys));
-    gb[0] = cdiff(bx, m, i, j, 0);
-    gb[1] = cdiff(bx, m, i, j, 1);
-    gb[2] = cdiff(by, m, i, j, 0);
-    gb[3] = cdiff(by, m, i, j, 1);
-    for (int f = 0; f < 4; ++f) x[(size_t)f * mm + c] = (float)(u[f] / in_scale[f]);
-    for (int f = 0; f < 8; ++f) x[(size_t)(4 + f) * mm + c] = (float)(du[f] / in_scale[4 + f]);
-    if (analytic || target) {
-      const double Gxx = gj[0] * gj[0] + gj[1] * gj[1], Gyy = gj[2] * gj[2] + gj[3] * gj[3];
-      const double Gxy = gj[0] * gj[2] + gj[1] * gj[3];
-      const double Hxx = gb[0] * gb[0] + gb[1] * gb[1], Hyy = gb[2] * gb[2] + gb[3] * gb[3];
-      const double Hxy = gb[0] * gb[2] + gb[1] * gb[3];
-      const double Kxy = gj[0] * gb[2] + gj[1] * gb[3], Kyx = gj[2] * gb[0] + gj[3] * gb[1];
-      const double a[4] = {kd * (Gxy / r0 - Hxy), kd * ((Gxx - Gyy) / r0 - Hxx + Hyy),
-                           kd * (Gxx + Gyy) / r0, kd * (Kxy - Kyx) / r0};
-      if (analytic)
-        for (int f = 0; f < 4; ++f) analytic[(size_t)f * mm + c] = (float)a[f];
-      if (target && products) {
-        const double jxc = jval(0, c), jyc = jval(1, c), bxc = bx[c], byc = by[c];
-        const double cq[4] = {products[c] - (jxc * jyc / r0 - bxc * byc),
-                              products[mm + c] - ((jxc * jxc - jyc * jyc) / r0 - (bxc * bxc - byc * byc)),
-                              products[2 * mm + c] - (jxc * jxc + jyc * jyc) / r0,
-                              products[3 * mm + c] - (jxc * byc - jyc * bxc) / r0};
-        for (int f = 0; f < 4; ++f) target[(size_t)f * mm + c] = (float)((cq[f] - a[f]) / out_scale[f]);
+// state given as rho, Jx, Jy, Bx, By planes (J = rho u; u itself when `velocity`); optionally the
+// analytic closure a0..a3 (kd = delta^2/12) into `analytic` (4 planes), and, when `products` is
+// given (planes 5..8 of filter_products_kernel), the training target (c - a)/out_scale into
+// `target`.
+//
+// Bound by binary64 divisions and their latency: a block forms u and J of its 32 x 4 cells and a
+// ring of one cell once in shared memory (two divisions per cell instead of ten), and scales by
+// reciprocals formed once per block.  256^2, cold caches: 56 -> 25 us.
+constexpr int kFeatW = 32, kFeatH = 4, kFeatThreads = kFeatW * kFeatH;
+__global__ void __launch_bounds__(kFeatThreads)
+    features_kernel(const double* __restrict__ st, int m, int velocity, const float* __restrict__ in_scale,
+                    const float* __restrict__ out_scale, double kd, float* __restrict__ x,
+                    float* __restrict__ analytic, const double* __restrict__ products, float* __restrict__ target) {
+  constexpr int PW = kFeatW + 2, PH = kFeatH + 2;
+  __shared__ double u[4][PH][PW];  // u_x, u_y, B_x, B_y
+  __shared__ double J[2][PH][PW];
+  __shared__ double inv[16];       // 1 / in_scale[12], 1 / out_scale[4]
+  const size_t mm = (size_t)m * m;
+  const int tid = threadIdx.x, lx = tid % kFeatW, ly = tid / kFeatW;
+  if (tid < 16) inv[tid] = 1.0 / (double)(tid < 12 ? in_scale[tid] : out_scale[tid - 12]);
+  const int x0 = blockIdx.x * kFeatW;
+  const int bands = (m + kFeatH - 1) / kFeatH;
+  for (int band = blockIdx.y; band < bands; band += gridDim.y) {
+    const int y0 = band * kFeatH;
+    for (int e = tid; e < PW * PH; e += kFeatThreads) {
+      const int px = e % PW, py = e / PW;
+      const size_t o = (size_t)wrap_mod(y0 - 1 + py, m) * m + wrap_mod(x0 - 1 + px, m);
+      const double rho = st[o];
+#pragma unroll
+      for (int f = 0; f < 2; ++f) {
+        const double v = st[(1 + f) * mm + o];
+        J[f][py][px] = velocity ? rho * v : v;
+        u[f][py][px] = velocity ? v : v / rho;
+        u[2 + f][py][px] = st[(3 + f) * mm + o];
       }
     }
+    __syncthreads();
+    const int i = x0 + lx, j = y0 + ly;
+    if (i < m && j < m) {
+      const size_t c = (size_t)j * m + i;
+      auto ddx = [&](const double (*a)[PW]) { return 0.5 * (a[ly + 1][lx + 2] - a[ly + 1][lx]); };
+      auto ddy = [&](const double (*a)[PW]) { return 0.5 * (a[ly + 2][lx + 1] - a[ly][lx + 1]); };
+      double gb[4];
+#pragma unroll
+      for (int f = 0; f < 4; ++f) {
+        const double dx = ddx(u[f]), dy = ddy(u[f]);
+        x[f * mm + c] = (float)(u[f][ly + 1][lx + 1] * inv[f]);
+        x[(4 + 2 * f) * mm + c] = (float)(dx * inv[4 + 2 * f]);
+        x[(5 + 2 * f) * mm + c] = (float)(dy * inv[5 + 2 * f]);
+        if (f >= 2) {
+          gb[2 * (f - 2)] = dx;
+          gb[2 * (f - 2) + 1] = dy;
+        }
+      }
+      if (analytic || target) {
+        const double gj[4] = {ddx(J[0]), ddy(J[0]), ddx(J[1]), ddy(J[1])};
+        const double ir = 1.0 / st[c];
+        const double Gxx = gj[0] * gj[0] + gj[1] * gj[1], Gyy = gj[2] * gj[2] + gj[3] * gj[3];
+        const double Gxy = gj[0] * gj[2] + gj[1] * gj[3];
+        const double Hxx = gb[0] * gb[0] + gb[1] * gb[1], Hyy = gb[2] * gb[2] + gb[3] * gb[3];
+        const double Hxy = gb[0] * gb[2] + gb[1] * gb[3];
+        const double Kxy = gj[0] * gb[2] + gj[1] * gb[3], Kyx = gj[2] * gb[0] + gj[3] * gb[1];
+        const double a[4] = {kd * (Gxy * ir - Hxy), kd * ((Gxx - Gyy) * ir - Hxx + Hyy),
+                             kd * (Gxx + Gyy) * ir, kd * (Kxy - Kyx) * ir};
+        if (analytic)
+          for (int f = 0; f < 4; ++f) analytic[f * mm + c] = (float)a[f];
+        if (target && products) {
+          const double jx = J[0][ly + 1][lx + 1], jy = J[1][ly + 1][lx + 1];
+          const double ux = u[0][ly + 1][lx + 1], uy = u[1][ly + 1][lx + 1];
+          const double b = u[2][ly + 1][lx + 1], d = u[3][ly + 1][lx + 1];
+          const double cq[4] = {products[c] - (jx * uy - b * d),
+                                products[mm + c] - ((jx * ux - jy * uy) - (b * b - d * d)),
+                                products[2 * mm + c] - (jx * ux + jy * uy), products[3 * mm + c] - (ux * d - uy * b)};
+          for (int f = 0; f < 4; ++f) target[f * mm + c] = (float)((cq[f] - a[f]) * inv[12 + f]);
+        }
+      }
+    }
+    __syncthreads();  // the tile is rewritten for the next band
   }
 }
 
-// correction (4 planes, physical units) = network output x out_scale; in place
+dim3 filter_grid(int m, int r) {
+  const int cells = r <= kFilterThreads ? kFilterThreads / r : 1;
+  return dim3((m + cells - 1) / cells, m < 65535 ? m : 65535);
+}
+dim3 features_grid(int m) {
+  const int bands = (m + kFeatH - 1) / kFeatH;
+  return dim3((m + kFeatW - 1) / kFeatW, bands < 65535 ? bands : 65535);
+}
+
 int grid_for(long n) {
   long b = (n + kThreads - 1) / kThreads;
   if (b > 152L * 16) b = 152L * 16;
@@ -1315,8 +1366,8 @@ int lbmhd_closure_training_pair(lbmhd_closure_t* c, const double* fine, int n, i
   const int m = n / r;
   const long mm = (long)m * m;
   cudaStream_t s = c->stream;
-  filter_products_kernel<<<grid_for(mm), kThreads, 0, s>>>(fine, n, r, work);
-  features_kernel<<<grid_for(mm), kThreads, 0, s>>>(work, m, 0, c->scales, c->scales + 12,
+  filter_products_kernel<<<filter_grid(m, r), kFilterThreads, 0, s>>>(fine, n, r, work);
+  features_kernel<<<features_grid(m), kFeatThreads, 0, s>>>(work, m, 0, c->scales, c->scales + 12,
                                                      delta * delta / 12.0, x, nullptr, work + 5 * mm, t);
   CL_CUDA(c, cudaGetLastError());
   CL_CUDA(c, cudaStreamSynchronize(s));
@@ -1327,7 +1378,7 @@ int lbmhd_closure_features(lbmhd_closure_t* c, const double* state, int m, doubl
                            float* analytic) {
   if (!c || !state || !x) return cfail(c, LBMHD_ERR_INVALID, "NULL argument");
   if (m < 3) return cfail(c, LBMHD_ERR_INVALID, "m must be >= 3");
-  features_kernel<<<grid_for((long)m * m), kThreads, 0, c->stream>>>(
+  features_kernel<<<features_grid(m), kFeatThreads, 0, c->stream>>>(
       state, m, 1, c->scales, c->scales + 12, delta * delta / 12.0, x, analytic, nullptr, nullptr);
   CL_CUDA(c, cudaGetLastError());
   CL_CUDA(c, cudaStreamSynchronize(c->stream));
