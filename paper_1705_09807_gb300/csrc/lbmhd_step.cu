@@ -64,6 +64,15 @@ template <typename T>
 struct KCoef {
   T r3, r4, r5, r6, r7, r8, sm, kq;
 };
+// Binary64: the products of the rates with the integers of T and with the weights that collide64
+// takes, formed once on the host.
+template <>
+struct KCoef<double> {
+  double r3, r4, kq;
+  double r5, r6, r7x4, r7x9, r7x3;  // s_j' = s_j / |T_j|^2, 4 s_7', ...
+  double r8x5, r8, r8x8_3, r8x3;
+  double sm;
+};
 
 // Collision of one cell; p[] holds the pulled (current) populations with f as deviations
 // f_i - w_i, and receives the post-collision values.  rho1 = rho - 1.  dJ = undivided
@@ -165,6 +174,122 @@ __device__ __forceinline__ void collide(T p[kQ], T rho1, T jx, T jy, T bx, T by,
   }
 }
 
+
+// ---- binary64 collision ---------------------------------------------------------------------------
+// The binary64 step is bound by GB300's binary64 rate (528 G instructions/s, every kind alike), so
+// it is written for few instructions: 173 per cell of an LES step against 216 for the form that
+// `collide` spells out, the same algebra otherwise.
+//  - Moments and non-equilibrium parts share their sums: the sums and differences of opposite
+//    populations that give rho and J (moments64) are kept until the cell is collided, and
+//    n_5 = 2 e_x - (f_1 - f_3) with e_x the diagonals' part of J_x, n_7 = 4 rho - 9 (f_1+..+f_4) + 3 q and
+//    n_8 = 5 f_0 + (f_1+..+f_4) - 8/3 rho + 3 q (rho as its deviation) replace the sums over all
+//    populations; in n_7 and n_8 the rates are folded into the coefficients.
+//  - The magnetic equilibria share w B and 3 w E, and the rest population takes B minus five times
+//    the axis ones' w B.  The update stays g + s_m (g^eq - g): (1 - s_m) g + s_m g^eq in one FMA would
+//    save 18 more (1024^2: 342 instead of 372 us per step), but it rounds g itself at every step: the
+//    errors of g grew by 20% and those of B by up to 1.5 (s_m = 0.71).
+//  - 1/rho: hardware estimate (20 bits) and one step of Halley's cubic iteration.
+// Each value added to a population of size O(u) or O(B) is formed first, so that a population is
+// rounded once at its own size, as in `collide`: against 80-bit arithmetic (64^2, SRT and MRT, 20
+// steps) the errors of f, g, rho, J and B are 0.93 to 1.00 of those of the 216-instruction form.
+// 1024^2, Delta = 2: 453 -> 372 us per step.
+struct Fluid64 {  // of one cell, from its f (deviations)
+  double c1, c2;  // f_1 - f_3, f_2 - f_4
+  double e1, e2;  // f_5 - f_6 - f_7 + f_8, f_5 + f_6 - f_7 - f_8
+  double ab;      // (f_1 + f_3) - (f_2 + f_4)
+  double pm;      // (f_5 + f_7) - (f_6 + f_8)
+  double s1;      // f_1 + f_2 + f_3 + f_4
+};
+
+template <typename V>
+__device__ __forceinline__ void moments64(V v, double& rho1, double& jx, double& jy, double& bx, double& by,
+                                          Fluid64& k) {
+  const double f1 = v(1), f2 = v(2), f3 = v(3), f4 = v(4), f5 = v(5), f6 = v(6), f7 = v(7), f8 = v(8);
+  const double a = f1 + f3, b = f2 + f4, p = f5 + f7, m = f6 + f8;
+  const double m1 = f5 - f7, m2 = f6 - f8;
+  k.c1 = f1 - f3;
+  k.c2 = f2 - f4;
+  k.ab = a - b;
+  k.pm = p - m;
+  k.s1 = a + b;
+  rho1 = (v(0) + k.s1) + (p + m);
+  k.e1 = m1 - m2;
+  k.e2 = m1 + m2;
+  jx = k.c1 + k.e1;
+  jy = k.c2 + k.e2;
+  bx = ((v(9) + v(10)) + (v(11) + v(12))) + ((v(13) + v(14)) + (v(15) + v(16))) + v(17);
+  by = ((v(18) + v(19)) + (v(20) + v(21))) + ((v(22) + v(23)) + (v(24) + v(25))) + v(26);
+}
+
+__device__ __forceinline__ double reciprocal(double r) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(r));
+  const double e = fma(-r, y, 1.0);  // y (1 + e + e^2): relative error e^3 < 2^-57
+  return fma(y, fma(e, e, e), y);
+}
+
+// One magnetic component toward b w_i -+ 3 w_i E (t = 3 w E on the axis, u on the diagonals):
+// populations of p in the order rest; the two axis ones without E; minus and plus E on the axis;
+// minus, minus, plus, plus on the diagonals.
+__device__ __forceinline__ void relax64(double* p0, double* pa, double* pb, double* pm, double* pp, double* pd0,
+                                        double* pd1, double* pu0, double* pu1, double b, double t, double u,
+                                        double sm) {
+  const double ea = (1.0 / 9.0) * b;  // = 4 w_diag b as well
+  const double em = ea - t, ep = ea + t, dm = fma(0.25, ea, -u), dp = fma(0.25, ea, u);
+  const double e0 = fma(-5.0, ea, b);
+  *p0 = fma(sm, e0 - *p0, *p0);
+  *pa = fma(sm, ea - *pa, *pa);
+  *pb = fma(sm, ea - *pb, *pb);
+  *pm = fma(sm, em - *pm, *pm);
+  *pp = fma(sm, ep - *pp, *pp);
+  *pd0 = fma(sm, dm - *pd0, *pd0);
+  *pd1 = fma(sm, dm - *pd1, *pd1);
+  *pu0 = fma(sm, dp - *pu0, *pu0);
+  *pu1 = fma(sm, dp - *pu1, *pu1);
+}
+
+template <bool CORR>
+__device__ __forceinline__ void collide64(double p[kQ], double rho1, double jx, double jy, double bx, double by,
+                                          const Fluid64& m, const double dJ[4], const double dB[4],
+                                          const KCoef<double>& c, const double* cq) {
+  const double ir = reciprocal(1.0 + rho1), k = c.kq;
+  const double gxx = fma(dJ[1], dJ[1], dJ[0] * dJ[0]), gyy = fma(dJ[3], dJ[3], dJ[2] * dJ[2]);
+  const double gxy = fma(dJ[1], dJ[3], dJ[0] * dJ[2]);
+  const double hd = fma(-dB[3], dB[3], fma(-dB[2], dB[2], fma(dB[1], dB[1], dB[0] * dB[0])));  // H_xx - H_yy
+  const double hxy = fma(dB[1], dB[3], dB[0] * dB[2]);
+  const double kk = fma(-dJ[3], dB[1], fma(-dJ[2], dB[0], fma(dJ[1], dB[3], dJ[0] * dB[2])));  // K_xy - K_yx
+  const double qxx = fma(k, gxx, jx * jx) * ir, qyy = fma(k, gyy, jy * jy) * ir;
+  double sxy = fma(fma(k, gxy, jx * jy), ir, -fma(k, hxy, bx * by));        // Q_xy - R_xy
+  double sd = (qxx - qyy) - fma(k, hd, fma(-by, by, bx * bx));              // (Q_xx - Q_yy) - (R_xx - R_yy)
+  double qq = qxx + qyy;
+  double E = fma(k, kk, fma(-jy, bx, jx * by)) * ir;
+  if (CORR) {
+    sxy += cq[0];
+    sd += cq[1];
+    qq += cq[2];
+    E += cq[3];
+  }
+  const double d3 = c.r3 * (m.pm - sxy), d4 = c.r4 * (m.ab - sd);
+  const double d5 = c.r5 * fma(2.0, m.e1, -m.c1), d6 = c.r6 * fma(2.0, m.e2, -m.c2);
+  const double d7 = fma(c.r7x3, qq, fma(-c.r7x9, m.s1, c.r7x4 * rho1));
+  const double d8 = fma(c.r8x3, qq, fma(c.r8x5, p[0], fma(c.r8, m.s1, -c.r8x8_3 * rho1)));
+  // f* = f - T^T d
+  const double u = fma(5.0, d7, -d4), w = fma(5.0, d7, d4), e78 = fma(-4.0, d7, d8);
+  const double g = e78 - d3, h = e78 + d3, a = d5 + d6, b = d5 - d6;
+  p[0] = fma(-4.0, d7 + d8, p[0]);
+  p[1] += fma(2.0, d5, u);
+  p[2] += fma(2.0, d6, w);
+  p[3] += fma(-2.0, d5, u);
+  p[4] += fma(-2.0, d6, w);
+  p[5] += g - a;
+  p[6] += h + b;
+  p[7] += g + a;
+  p[8] += h - b;
+  // g^eq_x,i = w_i (B_x - 3 c_iy E), g^eq_y,i = w_i (B_y + 3 c_ix E)
+  const double t = (1.0 / 3.0) * E, v = (1.0 / 12.0) * E;
+  relax64(p + 9, p + 10, p + 12, p + 11, p + 13, p + 14, p + 15, p + 16, p + 17, bx, t, v, c.sm);
+  relax64(p + 18, p + 20, p + 22, p + 21, p + 19, p + 24, p + 25, p + 23, p + 26, by, t, v, c.sm);
+}
 
 // ---- packed binary32 pairs (two cells per thread, binary16 storage) ---------------------------
 // Blackwell executes add / sub / mul / fma on two binary32 lanes held in a 64-bit register pair
@@ -458,14 +583,19 @@ __device__ __forceinline__ bool run_tile(const CUtensorMap* srcp, S* __restrict_
     return mbar_wait_bounded(&S_.full[K % NST], (K / NST) & 1u, kWaitLimitNs);
   };
   // moments of staged row k into ring slot k & 3 (own column and the strip's halo columns)
+  constexpr bool F64 = sizeof(T) == 8;
   T rho_next = T(0);
+  Fluid64 kept_next{};  // binary64: sums of the cell's f that its collision takes
   auto ring_moments = [&](int k) {
     const S* st = S_.stage[slot(k)];
     T* rg = &S_.ring[k & (kRing - 1)][0][0];
     constexpr int RS = SM::kRingW;
     T r1, jx, jy, bx, by;
     if (active) {
-      moments_from<T, S, BW>(st, GE, t + LEAD, r1, jx, jy, bx, by);
+      if constexpr (F64)
+        moments64([&](int q) { return staged<T, S, BW>(st, GE, q, t + LEAD); }, r1, jx, jy, bx, by, kept_next);
+      else
+        moments_from<T, S, BW>(st, GE, t + LEAD, r1, jx, jy, bx, by);
       rg[0 * RS + t + 1] = jx;
       rg[1 * RS + t + 1] = jy;
       rg[2 * RS + t + 1] = bx;
@@ -504,6 +634,7 @@ __device__ __forceinline__ bool run_tile(const CUtensorMap* srcp, S* __restrict_
   if (wait_row(0)) ring_moments(0); else S_.abort_flag[1] = 1;
   if (wait_row(1)) ring_moments(1); else S_.abort_flag[1] = 1;
   T rho_cur = rho_next;
+  Fluid64 kept = kept_next;
 
   const size_t pitch = (size_t)g.pitch;
   for (int m = 1; m <= L - 2; ++m) {
@@ -566,9 +697,11 @@ __device__ __forceinline__ bool run_tile(const CUtensorMap* srcp, S* __restrict_
         const size_t cell = (size_t)y * nx + x, cplane = (size_t)nx * ny;
         const T cq[4] = {(T)corr[cell], (T)corr[cplane + cell], (T)corr[2 * cplane + cell],
                          (T)corr[3 * cplane + cell]};
-        collide<T, true>(p, rho_cur, jx, jy, bx, by, dJ, dB, c, cq);
+        if constexpr (F64) collide64<true>(p, rho_cur, jx, jy, bx, by, kept, dJ, dB, c, cq);
+        else collide<T, true>(p, rho_cur, jx, jy, bx, by, dJ, dB, c, cq);
       } else {
-        collide(p, rho_cur, jx, jy, bx, by, dJ, dB, c);
+        if constexpr (F64) collide64<false>(p, rho_cur, jx, jy, bx, by, kept, dJ, dB, c, nullptr);
+        else collide(p, rho_cur, jx, jy, bx, by, dJ, dB, c);
       }
       S* o = dst + (size_t)y * pitch + kXOff + x;
       const S* end = dst + (size_t)g.pitch * ny;  // one past the copy (checking build)
@@ -589,6 +722,7 @@ __device__ __forceinline__ bool run_tile(const CUtensorMap* srcp, S* __restrict_
       }
     }
     rho_cur = rho_next;
+    if constexpr (F64) kept = kept_next;
   }
   kbase = kb + (uint32_t)L;
   return true;
@@ -1075,6 +1209,22 @@ __global__ void __launch_bounds__(step_threads<S>(), MINB)
 template <typename T>
 KCoef<T> cast_coef(const StepCoef& c) {
   KCoef<T> k;
+  if constexpr (sizeof(T) == 8) {
+    k.r3 = c.r[3];
+    k.r4 = c.r[4];
+    k.kq = c.kq;
+    k.r5 = c.r[5];
+    k.r6 = c.r[6];
+    k.r7x4 = 4 * c.r[7];
+    k.r7x9 = 9 * c.r[7];
+    k.r7x3 = 3 * c.r[7];
+    k.r8x5 = 5 * c.r[8];
+    k.r8 = c.r[8];
+    k.r8x8_3 = 8 * c.r[8] / 3;
+    k.r8x3 = 3 * c.r[8];
+    k.sm = c.s_m;
+    return k;
+  } else {
   k.r3 = (T)c.r[3];
   k.r4 = (T)c.r[4];
   k.r5 = (T)c.r[5];
@@ -1084,6 +1234,7 @@ KCoef<T> cast_coef(const StepCoef& c) {
   k.sm = (T)c.s_m;
   k.kq = (T)c.kq;
   return k;
+  }
 }
 
 // Pipeline depth and residency per storage type (at least 3 stages: iteration m waits for row
