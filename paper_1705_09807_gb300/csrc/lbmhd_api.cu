@@ -238,7 +238,6 @@ int create(lbmhd_t** out, const lbmhd_params* p) {
   g.ny = p->ny;
   g.plane = (p->nx + kXOff + 2 + 31) / 32 * 32;  // one row of one plane
   g.pitch = (int)(h->nplanes * g.plane);          // one row of all 27 (29) planes
-  g.band = step_band_rows(p->nx, p->ny, p->precision, sms);
   // rates scaled by the diagonal of T T^T = (9, 6, 6, 4, 4, 12, 12, 180, 20) (Eq. FluidTMatrix)
   const double norm[9] = {9, 6, 6, 4, 4, 12, 12, 180, 20};
   for (int j = 0; j < 9; ++j) h->coef.r[j] = j < 3 ? 0.0 : p->s[j] / norm[j];
@@ -247,6 +246,8 @@ int create(lbmhd_t** out, const lbmhd_params* p) {
   // undivided differences: central a(+1)-a(-1) = 2 d; isotropic 12 d
   h->coef.kq = p->grad_stencil == LBMHD_GRAD_ISOTROPIC ? kd / 144.0 : kd / 4.0;
   h->state_bytes = (size_t)g.pitch * p->ny * h->elem;
+  g.plain = plain_step_pays(p->precision, h->coef.kq, h->state_bytes) ? 1 : 0;
+  g.band = step_band_rows(p->nx, p->ny, p->precision, sms, g.plain != 0);
 #define LB_INIT(call)                 \
   do {                                \
     cudaError_t e_ = (call);          \

@@ -93,6 +93,7 @@ struct StepGeom {
   int nx, ny, pitch;  // grid; elements from one row to the next (all 27 planes of a row)
   size_t plane;       // elements from one plane to the next within a row
   int band;           // rows per block
+  int plain;          // 1: steps without correction planes take the plain form (Delta = 0)
   int skip_copy;      // test hook: 1 = block (0, 0) never issues its third row copy, so its
                       // bounded wait runs out and the step reports a timeout (no fault)
 };
@@ -119,8 +120,11 @@ cudaError_t launch_step_f16(const CUtensorMap& src, __half* dst, const StepGeom&
 constexpr int kQRel = kQ + 2;
 cudaError_t launch_step_f16rel(const CUtensorMap& src, const CUtensorMap& usrc, __half* dst, const StepGeom& g,
                                const StepCoef& c, int stencil, unsigned* err, cudaStream_t s);
-// Rows per block for the grid and precision (one wave of resident blocks when possible).
-int step_band_rows(int nx, int ny, int precision, int num_sms);
+// Whether a single grid's steps without correction planes take the plain form (no moments of other
+// cells; needs kq == 0), and the rows per block of its step (one wave of resident blocks when
+// possible).
+bool plain_step_pays(int precision, double kq, size_t state_bytes);
+int step_band_rows(int nx, int ny, int precision, int num_sms, bool plain = false);
 // Opt the step kernels in to their dynamic shared memory (once per process and device).
 cudaError_t prepare_step_kernels();
 #ifdef LBMHD_BOUNDS_CHECK

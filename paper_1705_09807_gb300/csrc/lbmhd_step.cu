@@ -36,6 +36,7 @@
 //   G_ab = d_b'J_a d_b'J_b, H_ab = d_b'B_a d_b'B_b, K_ab = d_b'J_a d_b'B_b (sum over b').
 #include <cstdlib>
 #include <mutex>
+#include <type_traits>
 
 #include "lbmhd_internal.cuh"
 #include "lbmhd_ptx.cuh"
@@ -248,21 +249,28 @@ __device__ __forceinline__ void relax64(double* p0, double* pa, double* pb, doub
   *pu1 = fma(sm, dp - *pu1, *pu1);
 }
 
-template <bool CORR>
+template <bool CORR, bool LES = true>
 __device__ __forceinline__ void collide64(double p[kQ], double rho1, double jx, double jy, double bx, double by,
                                           const Fluid64& m, const double dJ[4], const double dB[4],
                                           const KCoef<double>& c, const double* cq) {
-  const double ir = reciprocal(1.0 + rho1), k = c.kq;
-  const double gxx = fma(dJ[1], dJ[1], dJ[0] * dJ[0]), gyy = fma(dJ[3], dJ[3], dJ[2] * dJ[2]);
-  const double gxy = fma(dJ[1], dJ[3], dJ[0] * dJ[2]);
-  const double hd = fma(-dB[3], dB[3], fma(-dB[2], dB[2], fma(dB[1], dB[1], dB[0] * dB[0])));  // H_xx - H_yy
-  const double hxy = fma(dB[1], dB[3], dB[0] * dB[2]);
-  const double kk = fma(-dJ[3], dB[1], fma(-dJ[2], dB[0], fma(dJ[1], dB[3], dJ[0] * dB[2])));  // K_xy - K_yx
-  const double qxx = fma(k, gxx, jx * jx) * ir, qyy = fma(k, gyy, jy * jy) * ir;
-  double sxy = fma(fma(k, gxy, jx * jy), ir, -fma(k, hxy, bx * by));        // Q_xy - R_xy
-  double sd = (qxx - qyy) - fma(k, hd, fma(-by, by, bx * bx));              // (Q_xx - Q_yy) - (R_xx - R_yy)
+  const double ir = reciprocal(1.0 + rho1);
+  // J_a J_b, B_x^2 - B_y^2, B_x B_y and J_x B_y - J_y B_x, each with its gradient products
+  double nxx = jx * jx, nyy = jy * jy, nxy = jx * jy;
+  double bd = fma(-by, by, bx * bx), bxy = bx * by, ne = fma(-jy, bx, jx * by);
+  if constexpr (LES) {
+    const double k = c.kq;
+    nxx = fma(k, fma(dJ[1], dJ[1], dJ[0] * dJ[0]), nxx);
+    nyy = fma(k, fma(dJ[3], dJ[3], dJ[2] * dJ[2]), nyy);
+    nxy = fma(k, fma(dJ[1], dJ[3], dJ[0] * dJ[2]), nxy);
+    bd = fma(k, fma(-dB[3], dB[3], fma(-dB[2], dB[2], fma(dB[1], dB[1], dB[0] * dB[0]))), bd);
+    bxy = fma(k, fma(dB[1], dB[3], dB[0] * dB[2]), bxy);
+    ne = fma(k, fma(-dJ[3], dB[1], fma(-dJ[2], dB[0], fma(dJ[1], dB[3], dJ[0] * dB[2]))), ne);
+  }
+  const double qxx = nxx * ir, qyy = nyy * ir;
+  double sxy = fma(nxy, ir, -bxy);     // Q_xy - R_xy
+  double sd = (qxx - qyy) - bd;        // (Q_xx - Q_yy) - (R_xx - R_yy)
   double qq = qxx + qyy;
-  double E = fma(k, kk, fma(-jy, bx, jx * by)) * ir;
+  double E = ne * ir;
   if (CORR) {
     sxy += cq[0];
     sd += cq[1];
@@ -455,6 +463,21 @@ struct StepSmem : URingSmem<REL, box_width((int)sizeof(S))> {
   int abort_flag[2];
 };
 
+// The same for plain steps (Delta = 0), which need no moments of other cells and hence no ring.
+template <typename S, int NST, bool REL = false>
+struct PlainSmem : URingSmem<REL, box_width((int)sizeof(S))> {
+  using C = typename ArithOf<S>::type;
+  static constexpr int kNst = NST;
+  static constexpr int kLead = box_lead((int)sizeof(S));
+  static constexpr int kBoxW = box_width((int)sizeof(S));
+  static constexpr int kGroupElems = ((9 * kBoxW * (int)sizeof(S) + 127) / 128 * 128) / (int)sizeof(S);
+  static constexpr int kStageElems = 3 * kGroupElems;
+  static constexpr uint32_t kTxBytes = 3u * 9u * kBoxW * sizeof(S);
+  S stage[NST][kStageElems];
+  uint64_t full[NST];
+  int abort_flag[2];
+};
+
 // Store the 27 post-collision values of one cell, planes in address order through one advancing
 // pointer (fewer address instructions than 27 independent 64-bit plane offsets).
 template <typename S, typename T, int PL>
@@ -463,6 +486,28 @@ __device__ __forceinline__ void store_planes(S* op, const T* p, size_t plane, co
     constexpr int q = q_of_plane(PL);
     if (LB_IN(op >= lo && op < hi, 2)) *op = store_as<S>(p[q]);
     store_planes<S, T, PL + 1>(op + plane, p, plane, lo, hi);
+  }
+}
+
+// Store a collided cell and its ghost copies (columns 0, 1 at nx, nx + 1; nx - 2, nx - 1 at -2, -1).
+template <typename S, typename T>
+__device__ __forceinline__ void store_cell(S* __restrict__ dst, const StepGeom& g, int x, int y, const T* p) {
+  S* o = dst + (size_t)y * g.pitch + kXOff + x;
+  const S* end = dst + (size_t)g.pitch * g.ny;  // one past the copy (checking build)
+  store_planes<S, T, 0>(o, p, g.plane, dst, end);
+  if (x < 2) {
+#pragma unroll
+    for (int q = 0; q < kQ; ++q) {
+      S* a = o + (size_t)plane_of(q) * g.plane + g.nx;
+      if (LB_IN(a >= dst && a < end, 2)) *a = store_as<S>(p[q]);
+    }
+  }
+  if (x >= g.nx - 2) {
+#pragma unroll
+    for (int q = 0; q < kQ; ++q) {
+      S* a = o + (size_t)plane_of(q) * g.plane - g.nx;
+      if (LB_IN(a >= dst && a < end, 2)) *a = store_as<S>(p[q]);
+    }
   }
 }
 
@@ -475,10 +520,9 @@ __device__ __forceinline__ C staged(const S* st, int ge, int q, int col) {
   return load_as<C>(st[group_of(i) * ge + (3 * (q / 9) + index_in_group(i)) * BW + c]);
 }
 
-template <typename C, typename S, int BW>
-__device__ __forceinline__ void moments_from(const S* st, int ge, int col, C& rho1, C& jx, C& jy,
-                                             C& bx, C& by) {
-  auto v = [&](int q) -> C { return staged<C, S, BW>(st, ge, q, col); };
+// rho - 1, J and B of a cell whose pulled populations are v(q).
+template <typename C, typename V>
+__device__ __forceinline__ void moments_of(V v, C& rho1, C& jx, C& jy, C& bx, C& by) {
   const C f0 = v(0), f1 = v(1), f2 = v(2), f3 = v(3), f4 = v(4), f5 = v(5), f6 = v(6), f7 = v(7),
           f8 = v(8);
   rho1 = ((f0 + f1) + (f2 + f3)) + ((f4 + f5) + (f6 + f7)) + f8;
@@ -488,11 +532,21 @@ __device__ __forceinline__ void moments_from(const S* st, int ge, int col, C& rh
   by = ((v(18) + v(19)) + (v(20) + v(21))) + ((v(22) + v(23)) + (v(24) + v(25))) + v(26);
 }
 
+template <typename C, typename S, int BW>
+__device__ __forceinline__ void moments_from(const S* st, int ge, int col, C& rho1, C& jx, C& jy,
+                                             C& bx, C& by) {
+  moments_of([&](int q) -> C { return staged<C, S, BW>(st, ge, q, col); }, rho1, jx, jy, bx, by);
+}
+
 // Dynamic shared memory of a step block, rounded up to the 128-byte alignment TMA needs.
+template <typename SM>
+__device__ __forceinline__ SM& block_smem() {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  return *reinterpret_cast<SM*>(smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u));
+}
 template <typename S, int NST, bool REL = false>
 __device__ __forceinline__ StepSmem<S, NST, REL>& step_smem() {
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  return *reinterpret_cast<StepSmem<S, NST, REL>*>(smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u));
+  return block_smem<StepSmem<S, NST, REL>>();
 }
 
 template <typename SM>
@@ -636,7 +690,6 @@ __device__ __forceinline__ bool run_tile(const CUtensorMap* srcp, S* __restrict_
   T rho_cur = rho_next;
   Fluid64 kept = kept_next;
 
-  const size_t pitch = (size_t)g.pitch;
   for (int m = 1; m <= L - 2; ++m) {
     // A: moments of the next row
     if (wait_row(m + 1)) ring_moments(m + 1); else S_.abort_flag[m & 1] = 1;
@@ -703,23 +756,7 @@ __device__ __forceinline__ bool run_tile(const CUtensorMap* srcp, S* __restrict_
         if constexpr (F64) collide64<false>(p, rho_cur, jx, jy, bx, by, kept, dJ, dB, c, nullptr);
         else collide(p, rho_cur, jx, jy, bx, by, dJ, dB, c);
       }
-      S* o = dst + (size_t)y * pitch + kXOff + x;
-      const S* end = dst + (size_t)g.pitch * ny;  // one past the copy (checking build)
-      store_planes<S, T, 0>(o, p, g.plane, dst, end);
-      if (x < 2) {  // right ghosts: logical columns nx, nx + 1
-#pragma unroll
-        for (int q = 0; q < kQ; ++q) {
-          S* a = o + (size_t)plane_of(q) * g.plane + nx;
-          if (LB_IN(a >= dst && a < end, 2)) *a = store_as<S>(p[q]);
-        }
-      }
-      if (x >= nx - 2) {  // left ghosts: logical columns -2, -1
-#pragma unroll
-        for (int q = 0; q < kQ; ++q) {
-          S* a = o + (size_t)plane_of(q) * g.plane - nx;
-          if (LB_IN(a >= dst && a < end, 2)) *a = store_as<S>(p[q]);
-        }
-      }
+      store_cell(dst, g, x, y, p);
     }
     rho_cur = rho_next;
     if constexpr (F64) kept = kept_next;
@@ -826,6 +863,66 @@ __device__ __forceinline__ void store_planes_pair(__half* op, const F2* p, size_
         *op = __float2half_rn(lo(p[q]));
     }
     store_planes_pair<PL + 1>(op + plane, p, plane, both, lo_end, hi_end);
+  }
+}
+
+// Store two collided cells, columns x and x + 1 (only x unless `both`), and their ghost copies.
+// REL: ux, uy are the cells' velocities J / rho (collision invariants); rounded to binary16 they
+// become the cells' velocity reference U, and the f values are stored relative to w_i (1 + 3 c_i . U).
+template <bool REL>
+__device__ __forceinline__ void store_cell_pair(__half* __restrict__ dst, const StepGeom& g, int x, int y, bool both,
+                                                F2* p, F2 ux, F2 uy) {
+  __half* o = dst + (size_t)y * g.pitch + kXOff + x;
+  const __half* end = dst + (size_t)g.pitch * g.ny;  // one past the copy (checking build)
+  __half2 uh[2];
+  if constexpr (REL) {
+    // f_1 -= U_x / 3, f_3 += U_x / 3, f_2 -= U_y / 3, f_4 += U_y / 3, f_5 -= (U_x + U_y) / 12,
+    // f_7 += (U_x + U_y) / 12, f_6 -= (U_y - U_x) / 12, f_8 += (U_y - U_x) / 12
+    uh[0] = __floats2half2_rn(lo(ux), hi(ux));
+    uh[1] = __floats2half2_rn(lo(uy), hi(uy));
+    const float2 fx = __half22float2(uh[0]), fy = __half22float2(uh[1]);
+    const F2 Ux = f2(fx.x, fx.y), Uy = f2(fy.x, fy.y);
+    const F2 a = f2(1.f / 3.f) * Ux, b = f2(1.f / 3.f) * Uy;
+    const F2 d1 = f2(1.f / 12.f) * (Ux + Uy), d2 = f2(1.f / 12.f) * (Uy - Ux);
+    p[1] = p[1] - a;
+    p[3] = p[3] + a;
+    p[2] = p[2] - b;
+    p[4] = p[4] + b;
+    p[5] = p[5] - d1;
+    p[7] = p[7] + d1;
+    p[6] = p[6] - d2;
+    p[8] = p[8] + d2;
+  }
+  store_planes_pair<0>(o, p, g.plane, both, dst, end);
+  if constexpr (REL) {
+#pragma unroll
+    for (int comp = 0; comp < 2; ++comp) {
+      __half* a = o + (size_t)(kQ + comp) * g.plane;
+      if (LB_IN(a >= dst && a + (both ? 2 : 1) <= end, 2)) {
+        if (both) *reinterpret_cast<__half2*>(a) = uh[comp];
+        else *a = __low2half(uh[comp]);
+      }
+    }
+  }
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int xh = x + h;
+    if (h == 1 && !both) break;
+    if (xh < 2 || xh >= g.nx - 2) {  // ghosts: logical nx, nx + 1 and -2, -1
+      __half* gp = o + h + (xh < 2 ? g.nx : -g.nx);
+#pragma unroll
+      for (int q = 0; q < kQ; ++q) {
+        __half* a = gp + (size_t)plane_of(q) * g.plane;
+        if (LB_IN(a >= dst && a < end, 2)) *a = __float2half_rn(h ? hi(p[q]) : lo(p[q]));
+      }
+      if constexpr (REL) {
+#pragma unroll
+        for (int comp = 0; comp < 2; ++comp) {
+          __half* a = gp + (size_t)(kQ + comp) * g.plane;
+          if (LB_IN(a >= dst && a < end, 2)) *a = h ? __high2half(uh[comp]) : __low2half(uh[comp]);
+        }
+      }
+    }
   }
 }
 
@@ -957,7 +1054,6 @@ __device__ __forceinline__ bool run_tile_pair(const CUtensorMap* srcp, __half* _
   if (wait_row(1)) ring_moments(1); else S_.abort_flag[1] = 1;
   F2 rho_cur = rho_next;
 
-  const size_t pitch = (size_t)g.pitch;
   for (int m = 1; m <= L - 2; ++m) {
     if (wait_row(m + 1)) ring_moments(m + 1); else S_.abort_flag[m & 1] = 1;
     __syncthreads();
@@ -1021,67 +1117,139 @@ __device__ __forceinline__ bool run_tile_pair(const CUtensorMap* srcp, __half* _
       for (int q = 0; q < kQ; ++q) p[q] = staged_pair_rel<BW, REL>(st, GE, q, c0 + LEAD, ur);
       F2 ir;
       collide_pair(p, rho_cur, own[0], own[1], own[2], own[3], dJ, dB, c, &ir);
-      const int y = row_of(m);
-      const int x = x0 + c0;
-      __half* o = dst + (size_t)y * pitch + kXOff + x;
-      const __half* end = dst + (size_t)g.pitch * ny;  // one past the copy (checking build)
-      __half2 uh[2];  // this cell pair's velocity reference U_x, U_y (binary16)
-      if constexpr (REL) {
-        // u = J / rho of the cells (collision invariants), rounded to binary16; the f values are
-        // stored relative to w_i (1 + 3 c_i . U): f_1 -= U_x / 3, f_3 += U_x / 3, f_2 -= U_y / 3,
-        // f_4 += U_y / 3, f_5 -= (U_x + U_y) / 12, f_7 += (U_x + U_y) / 12, f_6 -= (U_y - U_x) / 12,
-        // f_8 += (U_y - U_x) / 12
-        const F2 ux = own[0] * ir, uy = own[1] * ir;
-        uh[0] = __floats2half2_rn(lo(ux), hi(ux));
-        uh[1] = __floats2half2_rn(lo(uy), hi(uy));
-        const float2 fx = __half22float2(uh[0]), fy = __half22float2(uh[1]);
-        const F2 Ux = f2(fx.x, fx.y), Uy = f2(fy.x, fy.y);
-        const F2 a = f2(1.f / 3.f) * Ux, b = f2(1.f / 3.f) * Uy;
-        const F2 d1 = f2(1.f / 12.f) * (Ux + Uy), d2 = f2(1.f / 12.f) * (Uy - Ux);
-        p[1] = p[1] - a;
-        p[3] = p[3] + a;
-        p[2] = p[2] - b;
-        p[4] = p[4] + b;
-        p[5] = p[5] - d1;
-        p[7] = p[7] + d1;
-        p[6] = p[6] - d2;
-        p[8] = p[8] + d2;
-      }
-      store_planes_pair<0>(o, p, g.plane, c0 + 1 < ncol, dst, end);
-      if constexpr (REL) {
-#pragma unroll
-        for (int comp = 0; comp < 2; ++comp) {
-          __half* a = o + (size_t)(kQ + comp) * g.plane;
-          if (LB_IN(a >= dst && a + (c0 + 1 < ncol ? 2 : 1) <= end, 2)) {
-            if (c0 + 1 < ncol) *reinterpret_cast<__half2*>(a) = uh[comp];
-            else *a = __low2half(uh[comp]);
-          }
-        }
-      }
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int xh = x + h;
-        if (h == 1 && c0 + 1 >= ncol) break;
-        if (xh < 2 || xh >= nx - 2) {  // ghosts: logical nx, nx + 1 and -2, -1
-          __half* gp = o + h + (xh < 2 ? nx : -nx);
-#pragma unroll
-          for (int q = 0; q < kQ; ++q) {
-            __half* a = gp + (size_t)plane_of(q) * g.plane;
-            if (LB_IN(a >= dst && a < end, 2)) *a = __float2half_rn(h ? hi(p[q]) : lo(p[q]));
-          }
-          if constexpr (REL) {
-#pragma unroll
-            for (int comp = 0; comp < 2; ++comp) {
-              __half* a = gp + (size_t)(kQ + comp) * g.plane;
-              if (LB_IN(a >= dst && a < end, 2)) *a = h ? __high2half(uh[comp]) : __low2half(uh[comp]);
-            }
-          }
-        }
-      }
+      store_cell_pair<REL>(dst, g, x0 + c0, row_of(m), c0 + 1 < ncol, p, own[0] * ir, own[1] * ir);
     }
     rho_cur = rho_next;
   }
   kbase = kb + (uint32_t)L;
+  return true;
+}
+
+// ---- plain steps (Delta = 0) ----------------------------------------------------------------------
+// Without the filter's gradient products a cell's collision needs its own moments only: no moment
+// ring, no halo columns, and a band stages exactly its own rows.  Each thread takes its 27 values
+// out of the stage, one CTA barrier frees the stage for the row NST further on, and moments,
+// collision and stores run from registers, so all NST rows are in flight (the LES form keeps a row
+// staged from its moments to its collision).  The state is bitwise that of the LES form with k = 0
+// (zero gradients go through the same operations, so the compiler contracts them alike).
+// us per step against the LES form: binary64 64^2 14.7 -> 6.3, 512^2 127 -> 81, 2048^2 1811 -> 1159
+// (140 instead of 173 binary64 instructions per cell); binary32 128^2 2.76 -> 1.86, 512^2 9.7 -> 6.6,
+// 1024^2 36.4 -> 34.6; binary16 512^2 9.3 -> 5.7, 1024^2 22.5 -> 19.2, its relative form 256^2 5.4 -> 3.3.
+// Larger grids of the memory-bound forms lose (plain_step_pays).
+// Returns false if a wait timed out (the block must stop; *err is set).
+template <typename S, int NST, bool REL>
+__device__ __forceinline__ bool run_tile_plain(const CUtensorMap* srcp, S* __restrict__ dst, const StepGeom& g,
+                                               const KCoef<typename ArithOf<S>::type>& c1, int x0, int y0,
+                                               int band_parity, unsigned* __restrict__ err,
+                                               const CUtensorMap* usrcp = nullptr) {
+  using SM = PlainSmem<S, NST, REL>;
+  using T = typename SM::C;
+  constexpr bool PAIR = sizeof(S) == 2;  // two cells per thread
+  constexpr int GE = SM::kGroupElems, LEAD = SM::kLead, BW = SM::kBoxW;
+  SM& S_ = block_smem<SM>();
+  const int t = threadIdx.x;
+  const int c0 = PAIR ? 2 * t : t;  // first strip column of this thread
+  const int nx = g.nx, ny = g.ny;
+  const int ncol = min(kStepThreads, nx - x0);
+  const bool active = c0 < ncol;
+  const int y1 = min(y0 + g.band, ny), L = y1 - y0;
+  const int dir = (band_parity & 1) ? -1 : 1;
+  auto row_of = [&](int k) -> int {  // k = -1 and L: the neighbouring rows (U rows only)
+    int r = dir > 0 ? y0 + k : y1 - 1 - k;
+    if (r < 0) r += ny;
+    if (r >= ny) r -= ny;
+    return r;
+  };
+  auto issue = [&](int k) {
+    if (g.skip_copy && k == 0 && blockIdx.x == 0 && blockIdx.y == 0) return;  // test hook
+    const int s = k % NST;
+    const int r = row_of(k);
+    const int ra = r == 0 ? ny - 1 : r - 1;  // c_y = +1 group is pulled from row r - 1
+    const int rc = r == ny - 1 ? 0 : r + 1;  // c_y = -1 group from row r + 1
+    const int cx = x0 + kXOff - LEAD;
+    const bool in = LB_IN(ra >= 0 && ra < ny && r >= 0 && r < ny && rc >= 0 && rc < ny && cx >= 0, 3);
+    constexpr uint32_t kUBytes = 2u * BW * 2u;  // one U row
+    const uint32_t ubytes = REL ? (k == 0 ? 3u : 1u) * kUBytes : 0u;
+    mbar_arrive_expect_tx(&S_.full[s], in ? SM::kTxBytes + ubytes : 0u);  // 0: the phase completes empty
+    if (in) {
+      copy_row_boxes(S_.stage[s], GE, srcp, cx, ra, r, rc, &S_.full[s], false);
+      if constexpr (REL) {  // U rows of march indices k + 1 (and k - 1, k for the first row)
+        for (int j = (k == 0 ? -1 : k + 1); j <= k + 1; ++j)
+          tma_load_3d(&S_.uring[(j + kURing) % kURing][0], usrcp, cx, kQ, row_of(j), &S_.full[s]);
+      }
+    }
+  };
+  auto wait_row = [&](int k) -> bool {
+    return mbar_wait_bounded(&S_.full[k % NST], (uint32_t)(k / NST) & 1u, kWaitLimitNs);
+  };
+  if (t == 0) {
+    S_.abort_flag[0] = 0;
+    S_.abort_flag[1] = 0;
+  }
+  __syncthreads();  // barriers initialised
+  const int first = NST < L ? NST : L;
+  if (t == 0) {
+    fence_proxy_async_smem();
+    for (int k = 0; k < first; ++k) issue(k);
+  }
+  int issued = first;  // meaningful in thread 0 only
+
+  using V = typename std::conditional<PAIR, F2, T>::type;
+  for (int m = 0; m < L; ++m) {
+    if (!wait_row(m)) S_.abort_flag[m & 1] = 1;
+    V p[kQ];
+    if (active) {
+      const S* st = S_.stage[m % NST];
+      if constexpr (PAIR) {
+        const __half* ur[3] = {nullptr, nullptr, nullptr};
+        if constexpr (REL) {  // groups 0, 1, 2 are pulled from rows y - 1, y, y + 1
+          ur[0] = &S_.uring[(m - dir + kURing) % kURing][0];
+          ur[1] = &S_.uring[(m + kURing) % kURing][0];
+          ur[2] = &S_.uring[(m + dir + kURing) % kURing][0];
+        }
+#pragma unroll
+        for (int q = 0; q < kQ; ++q) p[q] = staged_pair_rel<BW, REL>(st, GE, q, c0 + LEAD, ur);
+      } else {
+#pragma unroll
+        for (int q = 0; q < kQ; ++q) p[q] = staged<T, S, BW>(st, GE, q, c0 + LEAD);
+      }
+    }
+    __syncthreads();
+    if (S_.abort_flag[m & 1]) {
+      if (t == 0) {
+        atomicOr(err, 1u);
+        for (int k = m; k < issued; ++k) wait_row(k);  // drain copies still in flight
+      }
+      return false;
+    }
+    if (t == 0 && m + NST < L) {
+      fence_proxy_async_smem();
+      issue(m + NST);
+      ++issued;
+    }
+    if (active) {
+      V rho1, jx, jy, bx, by;
+      auto v = [&](int q) -> V { return p[q]; };
+      const int y = row_of(m), x = x0 + c0;
+      if constexpr (PAIR) {
+        moments_of<V>(v, rho1, jx, jy, bx, by);
+        F2 ir;
+        const F2 zero[4] = {f2(0.f), f2(0.f), f2(0.f), f2(0.f)};
+        collide_pair(p, rho1, jx, jy, bx, by, zero, zero, pair_coef(c1), &ir);
+        store_cell_pair<REL>(dst, g, x, y, c0 + 1 < ncol, p, jx * ir, jy * ir);
+      } else if constexpr (sizeof(T) == 8) {
+        Fluid64 kept;
+        moments64(v, rho1, jx, jy, bx, by, kept);
+        collide64<false, false>(p, rho1, jx, jy, bx, by, kept, nullptr, nullptr, c1, nullptr);
+        store_cell(dst, g, x, y, p);
+      } else {
+        moments_of<V>(v, rho1, jx, jy, bx, by);
+        const T zero[4] = {T(0), T(0), T(0), T(0)};
+        collide(p, rho1, jx, jy, bx, by, zero, zero, c1);
+        store_cell(dst, g, x, y, p);
+      }
+    }
+  }
   return true;
 }
 
@@ -1144,6 +1312,20 @@ __global__ void __launch_bounds__(step_threads<S>(), MINB)
   uint32_t kbase = 0;
   run_any_tile<S, ISO, NST, CORR>(&src, dst, g, c, strip * kStepThreads, band * g.band, band + flip, kbase,
                                   err, corr);
+}
+
+// Plain step of one grid (Delta = 0); REL: with the U planes' tensor map.
+template <typename S, int NST, int MINB, bool REL>
+__global__ void __launch_bounds__(step_threads<S>(), MINB)
+    plain_step_kernel(const __grid_constant__ CUtensorMap src, const __grid_constant__ CUtensorMap usrc,
+                      S* __restrict__ dst, StepGeom g, KCoef<typename ArithOf<S>::type> c, unsigned* __restrict__ err,
+                      int flip) {
+  int strip, band;
+  tile_of_block(strip, band);
+  if (band * g.band >= g.ny) return;  // uniform per block
+  init_stage_barriers(block_smem<PlainSmem<S, NST, REL>>(), &src, REL ? &usrc : nullptr);
+  grid_dependency_wait();
+  run_tile_plain<S, NST, REL>(&src, dst, g, c, strip * kStepThreads, band * g.band, band + flip, err, &usrc);
 }
 
 // Relative binary16 storage (LBMHD_FP16_REL; single grids): fused_step_kernel's binary16 step
@@ -1285,6 +1467,47 @@ template <> struct StepConfig<__half> {
   static constexpr int kStages = LBMHD_F16_STAGES, kMinBlocks = LBMHD_F16_BLOCKS;
 };
 
+// The same for plain steps, whose blocks need no moment ring.  Measured (us per step): binary32 3 x 5
+// 6.60 / 35.1 at 512^2 / 1024^2 (3 x 4: 7.05 / 35.0, 4 x 3: 7.11 / 34.6, 2 x 6: 6.56 / 35.2);
+// binary64 2 x 3 81.5 / 284 at 512^2 / 1024^2 (3 x 2: 298 at 1024^2; 1 x 4: 85.8 at 512^2); binary16
+// 3 x 8 19.2 at 1024^2 (3 x 6: 19.8, 3 x 7: 20.7, 4 x 5: 21.1).
+#ifndef LBMHD_P32_STAGES
+#define LBMHD_P32_STAGES 3
+#endif
+#ifndef LBMHD_P32_BLOCKS
+#define LBMHD_P32_BLOCKS 5
+#endif
+#ifndef LBMHD_P64_STAGES
+#define LBMHD_P64_STAGES 2
+#endif
+#ifndef LBMHD_P64_BLOCKS
+#define LBMHD_P64_BLOCKS 3
+#endif
+#ifndef LBMHD_P16_STAGES
+#define LBMHD_P16_STAGES 3
+#endif
+#ifndef LBMHD_P16_BLOCKS
+#define LBMHD_P16_BLOCKS 8
+#endif
+template <typename S> struct PlainConfig;
+template <> struct PlainConfig<float> {
+  static constexpr int kStages = LBMHD_P32_STAGES, kMinBlocks = LBMHD_P32_BLOCKS;
+};
+template <> struct PlainConfig<double> {
+  static constexpr int kStages = LBMHD_P64_STAGES, kMinBlocks = LBMHD_P64_BLOCKS;
+};
+template <> struct PlainConfig<__half> {
+  static constexpr int kStages = LBMHD_P16_STAGES, kMinBlocks = LBMHD_P16_BLOCKS;
+};
+template <typename S, bool REL = false>
+constexpr auto plain_kernel_ptr() {
+  return &plain_step_kernel<S, PlainConfig<S>::kStages, PlainConfig<S>::kMinBlocks, REL>;
+}
+template <typename S, bool REL = false>
+constexpr size_t plain_smem_bytes() {
+  return sizeof(PlainSmem<S, PlainConfig<S>::kStages, REL>) + 128;
+}
+
 template <typename S, int ISO, bool CORR = false>
 constexpr auto kernel_ptr() {
   return &fused_step_kernel<S, ISO, StepConfig<S>::kStages, StepConfig<S>::kMinBlocks, CORR>;
@@ -1323,6 +1546,8 @@ cudaError_t launch_step(const CUtensorMap& src, S* dst, const StepGeom& g, const
       return stencil == 1 ? launch_programmatic(kernel_ptr<S, 1, true>(), grid, nt, sm, s, src, dst, g, k, err, corr, flip)
                           : launch_programmatic(kernel_ptr<S, 0, true>(), grid, nt, sm, s, src, dst, g, k, err, corr, flip);
   }
+  if (g.plain)
+    return launch_programmatic(plain_kernel_ptr<S>(), grid, nt, plain_smem_bytes<S>(), s, src, src, dst, g, k, err, flip);
   const float* none = nullptr;
   return stencil == 1 ? launch_programmatic(kernel_ptr<S, 1>(), grid, nt, sm, s, src, dst, g, k, err, none, flip)
                       : launch_programmatic(kernel_ptr<S, 0>(), grid, nt, sm, s, src, dst, g, k, err, none, flip);
@@ -1333,6 +1558,9 @@ cudaError_t launch_step_rel(const CUtensorMap& src, const CUtensorMap& usrc, __h
   dim3 grid((g.nx + kStepThreads - 1) / kStepThreads, (g.ny + g.band - 1) / g.band);
   const KCoef<float> k = cast_coef<float>(c);
   const int nt = kStepThreads / 2;
+  if (g.plain)
+    return launch_programmatic(plain_kernel_ptr<__half, true>(), grid, nt, plain_smem_bytes<__half, true>(), s, src, usrc,
+                               dst, g, k, err, 0);
   const size_t sm = rel_smem_bytes();
   return stencil == 1 ? launch_programmatic(rel_kernel_ptr<1>(), grid, nt, sm, s, src, usrc, dst, g, k, err)
                       : launch_programmatic(rel_kernel_ptr<0>(), grid, nt, sm, s, src, usrc, dst, g, k, err);
@@ -1349,6 +1577,14 @@ cudaError_t set_smem_attr() {
   cudaError_t e = cudaFuncSetAttribute(kernel_ptr<S, 0>(), cudaFuncAttributeMaxDynamicSharedMemorySize, b);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(kernel_ptr<S, 1>(), cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(plain_kernel_ptr<S>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)plain_smem_bytes<S>());
+  if constexpr (sizeof(S) == 2) {
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(plain_kernel_ptr<S, true>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)plain_smem_bytes<S, true>());
+  }
   if constexpr (sizeof(S) != 2) {
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(kernel_ptr<S, 0, true>(), cudaFuncAttributeMaxDynamicSharedMemorySize, b);
@@ -1471,14 +1707,29 @@ int resident_step_blocks(int precision, int num_sms) {
   return num_sms * per_sm;
 }
 
+// Whether a grid's steps without filter and correction (kq == 0) take the plain form.  Binary64,
+// bound by arithmetic: always.  The others only while one copy of the state fits the 129 MB L2: with
+// NST rows in flight per block, neighbouring strips drift apart by more than the L2 holds of larger
+// grids, and the box columns that two strips share are then read from DRAM twice (2048^2 binary32:
+// 507 instead of 470 MB read per step, 158 instead of 142 us; 1448^2, 235 MB a copy: 79.5 against
+// 73.1; 1150^2, 147 MB: 45.7 against 45.9; 1024^2, 120 MB: 34.6 against 36.4; binary16 1700^2, 161
+// MB: 63.4 against 62.0; 1448^2, 118 MB: 43.7 against 46.9).
+bool plain_step_pays(int precision, double kq, size_t state_bytes) {
+  return kq == 0.0 && (precision == 0 || state_bytes <= (size_t)128 << 20);
+}
+
 // Rows per block: with the blocks that fit on the GPU at once (`resident`), give every strip
 // floor(resident / strips) bands so the whole grid runs in one wave; never fewer than
 // LBMHD_MIN_BAND rows.
-int step_band_rows(int nx, int ny, int precision, int num_sms) {
+int step_band_rows(int nx, int ny, int precision, int num_sms, bool plain) {
   const int strips = (nx + kStepThreads - 1) / kStepThreads;
-  const int per_sm = precision == 0   ? StepConfig<double>::kMinBlocks
-                     : precision == 1 ? StepConfig<float>::kMinBlocks
-                                      : StepConfig<__half>::kMinBlocks;  // binary16, both forms
+  int per_sm = precision == 0   ? StepConfig<double>::kMinBlocks
+               : precision == 1 ? StepConfig<float>::kMinBlocks
+                                : StepConfig<__half>::kMinBlocks;  // binary16, both forms
+  if (plain)
+    per_sm = precision == 0   ? PlainConfig<double>::kMinBlocks
+             : precision == 1 ? PlainConfig<float>::kMinBlocks
+                              : PlainConfig<__half>::kMinBlocks;
   const long resident = (long)num_sms * per_sm * LBMHD_WAVES;
   long bands = resident / strips;
   if (bands < 1) bands = 1;
