@@ -19,7 +19,8 @@
 // one the columns and adds up the shells, so the n x n spectrum is never stored.  Every n <= 4096
 // takes O(n^2 log n): radices 8, 4, 2, 3, 5, 7, 11, 13 when they factor n, Bluestein's chirp
 // convolution of power-of-two length >= 2n - 1 otherwise.  Four fields at n = 1024 took 60.1 ms with
-// direct O(n^3) sums; now rows 178, columns and shells 286, shell totals 19 us.
+// direct O(n^3) sums; now rows 178 (151 of
+// them its 2.5 M binary64 warp instructions), columns and shells 210, shell totals 7 us.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -31,21 +32,35 @@
 namespace lbmhd_gpu {
 namespace {
 
-constexpr int kThreads = 256;
-
-__global__ void block_mean_kernel(const double* __restrict__ in, int nx, int ny, int r,
-                                  double* __restrict__ out) {
-  const int mx = nx / r, my = ny / r;
-  const long m = (long)mx * my;
-  const double inv = 1.0 / ((double)r * r);
-  for (long c = blockIdx.x * (long)blockDim.x + threadIdx.x; c < m; c += (long)gridDim.x * blockDim.x) {
-    const int i = (int)(c % mx), j = (int)(c / mx);
+// Memory-bound (8 bytes in per cell), so what matters is loads in flight: a thread adds up one
+// coarse cell, row by row from the left, with the loads of a row independent of one another; a
+// warp reads whole rows of the fine field.  VEC: 16-byte loads (r even, rows and field on 16-byte
+// boundaries).  2048^2, r = 2, cold caches: 24.5 us with 64-bit divisions per cell and a grid-stride
+// loop (a division by r^2 in every thread cost another binary64 dozen); now 14.8 us.
+template <bool VEC>
+__global__ void __launch_bounds__(128)
+    block_mean_kernel(const double* __restrict__ in, int nx, int mx, int my, int r, double inv,
+                      double* __restrict__ out) {
+  const int i = blockIdx.x * 128 + threadIdx.x;
+  if (i >= mx) return;
+  for (int j = blockIdx.y; j < my; j += gridDim.y) {
+    const double* row = in + (size_t)j * r * nx + (size_t)i * r;
     double s = 0.0;
-    for (int yy = 0; yy < r; ++yy) {
-      const double* row = in + (size_t)(j * r + yy) * nx + (size_t)i * r;
-      for (int xx = 0; xx < r; ++xx) s += row[xx];
+#pragma unroll 2
+    for (int yy = 0; yy < r; ++yy, row += nx) {
+      if constexpr (VEC) {
+#pragma unroll 4
+        for (int xx = 0; xx < r; xx += 2) {
+          const double2 v = *reinterpret_cast<const double2*>(row + xx);
+          s += v.x;
+          s += v.y;
+        }
+      } else {
+#pragma unroll 4
+        for (int xx = 0; xx < r; ++xx) s += row[xx];
+      }
     }
-    out[c] = s * inv;
+    out[(size_t)j * mx + i] = s * inv;
   }
 }
 
@@ -347,6 +362,15 @@ __global__ void __launch_bounds__(256)
   }
   __syncthreads();
   transform_lines(fft_buf, p, t);
+  // |Z|^2 in natural order first: the runs below are then consecutive (a thread that added up to 45
+  // digit-reversed cells of its run held its block up)
+  double* power = reinterpret_cast<double*>(fft_buf + (size_t)lines * len);  // [lines][n]
+  for (int q = threadIdx.x; q < lines * n; q += blockDim.x) {
+    const int c = q / n, k = q - c * n;
+    const double2 z = fft_result(fft_buf + (size_t)c * len, p, t, k, false);
+    power[q] = z.x * z.x + z.y * z.y;
+  }
+  __syncthreads();
   for (int s = threadIdx.x; s < nbins; s += blockDim.x) {
     const int lo4 = (2 * s - 1) * (2 * s - 1), hi4 = (2 * s + 1) * (2 * s + 1);
     double sum = 0.0;
@@ -358,36 +382,34 @@ __global__ void __launch_bounds__(256)
       // Shell 0 holds the zero wavevector only.
       const int a = s == 0 || k4 > lo4 ? 0 : half_isqrt(lo4 - k4) + 1;
       const int b = half_isqrt(hi4 - k4);
-      const double2* line = fft_buf + (size_t)c * len;
-      for (int k = a; k <= min(b, kpos); ++k) {
-        const double2 z = fft_result(line, p, t, k, false);
-        sum += z.x * z.x + z.y * z.y;
-      }
-      for (int k = max(a, 1); k <= min(b, kneg); ++k) {
-        const double2 z = fft_result(line, p, t, n - k, false);
-        sum += z.x * z.x + z.y * z.y;
-      }
+      const double* line = power + (size_t)c * n;
+      for (int k = a; k <= min(b, kpos); ++k) sum += line[k];
+      for (int k = max(a, 1); k <= min(b, kneg); ++k) sum += line[n - k];
     }
     out[s] = sum;
   }
 }
 
-// E[s] = norm * sum over the column groups of part[pair][group][s]: 8 threads per shell take
-// every eighth group in order, then are added in order.
-__global__ void shell_total_kernel(const double* __restrict__ part, int groups, int nbins, double norm,
-                                   double* __restrict__ ek, double* __restrict__ em) {
-  __shared__ double sh[8][32];
-  const int s = blockIdx.x * 32 + threadIdx.x;
+// E[s] = norm * sum over the column groups of part[pair][group][s]: 32 threads per shell take every
+// 32nd group in order, then are added in order.
+constexpr int kTotalShells = 8;
+__global__ void __launch_bounds__(32 * kTotalShells)
+    shell_total_kernel(const double* __restrict__ part, int groups, int nbins, double norm, double* __restrict__ ek,
+                       double* __restrict__ em) {
+  __shared__ double sh[32][kTotalShells + 1];
+  const int s = blockIdx.x * kTotalShells + threadIdx.x;
   const double* p = part + (size_t)blockIdx.y * groups * nbins;
   double sum = 0.0;
-  if (s < nbins)
-    for (int g = threadIdx.y; g < groups; g += 8) sum += p[(size_t)g * nbins + s];
+  if (s < nbins) {
+#pragma unroll 4
+    for (int g = threadIdx.y; g < groups; g += 32) sum += p[(size_t)g * nbins + s];
+  }
   sh[threadIdx.y][threadIdx.x] = sum;
   __syncthreads();
   if (threadIdx.y == 0 && s < nbins) {
     double tot = 0.0;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) tot += sh[i][threadIdx.x];
+    for (int i = 0; i < 32; ++i) tot += sh[i][threadIdx.x];
     (blockIdx.y ? em : ek)[s] = norm * tot;
   }
 }
@@ -418,12 +440,6 @@ FftPlan make_plan(int n) {
   return p;
 }
 
-int grid_for(long n) {
-  long b = (n + kThreads - 1) / kThreads;
-  if (b > 152L * 16) b = 152L * 16;
-  return b < 1 ? 1 : (int)b;
-}
-
 }  // namespace
 
 size_t spectrum_work_bytes(int n) {
@@ -448,11 +464,12 @@ cudaError_t launch_energy_spectrum(const double* ux, const double* uy, const dou
   }
   double* part = reinterpret_cast<double*>(G + 2 * nn);
   const size_t smem = (size_t)p.lines * p.len * sizeof(double2);
+  const size_t smem_cols = smem + (size_t)p.lines * n * sizeof(double);  // and the power of the lines
   cudaError_t e = cudaSuccess;
-  if (smem > 48 * 1024) {
-    const int b = (int)smem;
+  if (smem_cols > 48 * 1024) {
+    const int b = (int)smem, bc = (int)smem_cols;
     e = cudaFuncSetAttribute(fft_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fft_cols_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fft_cols_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bc);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fft_filter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
     if (e != cudaSuccess) return e;
   }
@@ -460,14 +477,20 @@ cudaError_t launch_energy_spectrum(const double* ux, const double* uy, const dou
   fft_tables_kernel<<<(p.len + n + 127) / 128, 128, 0, s>>>(p, t);
   if (p.chirp()) fft_filter_kernel<<<1, 256, p.len * sizeof(double2), s>>>(p, t);
   fft_rows_kernel<<<dim3(groups, 2), p.threads, smem, s>>>(ux, uy, bx, by, p, t, G);
-  fft_cols_kernel<<<dim3(groups, 2), p.threads, smem, s>>>(G, p, t, nbins, part);
-  shell_total_kernel<<<dim3((nbins + 31) / 32, 2), dim3(32, 8), 0, s>>>(part, groups, nbins,
+  fft_cols_kernel<<<dim3(groups, 2), p.threads, smem_cols, s>>>(G, p, t, nbins, part);
+  shell_total_kernel<<<dim3((nbins + kTotalShells - 1) / kTotalShells, 2), dim3(kTotalShells, 32), 0, s>>>(part, groups, nbins,
                                                                        0.5 / ((double)nn * (double)nn), ek, em);
   return cudaGetLastError();
 }
 
 cudaError_t launch_block_mean(const double* in, int nx, int ny, int r, double* out, cudaStream_t s) {
-  block_mean_kernel<<<grid_for((long)(nx / r) * (ny / r)), kThreads, 0, s>>>(in, nx, ny, r, out);
+  const int mx = nx / r, my = ny / r;
+  const double inv = 1.0 / ((double)r * r);  // a binary64 division per thread would outweigh the sums
+  const dim3 grid((mx + 127) / 128, my < 65535 ? my : 65535);
+  if (r % 2 == 0 && nx % 2 == 0 && reinterpret_cast<uintptr_t>(in) % 16 == 0)
+    block_mean_kernel<true><<<grid, 128, 0, s>>>(in, nx, mx, my, r, inv, out);
+  else
+    block_mean_kernel<false><<<grid, 128, 0, s>>>(in, nx, mx, my, r, inv, out);
   return cudaGetLastError();
 }
 

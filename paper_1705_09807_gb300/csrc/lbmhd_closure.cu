@@ -918,14 +918,13 @@ cudaError_t launch_net(const float* in, const unsigned char* packed, const float
 // are products (J_x J_y / rho = J_x u_y, ...), 17 binary64 instructions per fine cell instead of
 // about 57 with four divisions.  A thread adds up one fine column of a coarse row, so the loads
 // are coalesced and a coarse cell occupies r threads; the r columns are then added in order.
-// 2048^2, r = 8, cold caches: 481 -> 147 us.
+// 2048^2, r = 8, cold caches: 481 -> 142 us.
 constexpr int kFilterThreads = 128;
 __global__ void __launch_bounds__(kFilterThreads)
-    filter_products_kernel(const double* __restrict__ fine, int n, int r, double* __restrict__ coarse) {
+    filter_products_kernel(const double* __restrict__ fine, int n, int r, double inv, double* __restrict__ coarse) {
   __shared__ double sh[9][kFilterThreads];
   const int m = n / r;
   const size_t mm = (size_t)m * m, nn = (size_t)n * n;
-  const double inv = 1.0 / ((double)r * r);
   // whole coarse cells per block; filters wider than the block take several passes of columns
   const int cells = r <= kFilterThreads ? kFilterThreads / r : 1;
   for (int j = blockIdx.y; j < m; j += gridDim.y) {
@@ -1366,7 +1365,7 @@ int lbmhd_closure_training_pair(lbmhd_closure_t* c, const double* fine, int n, i
   const int m = n / r;
   const long mm = (long)m * m;
   cudaStream_t s = c->stream;
-  filter_products_kernel<<<filter_grid(m, r), kFilterThreads, 0, s>>>(fine, n, r, work);
+  filter_products_kernel<<<filter_grid(m, r), kFilterThreads, 0, s>>>(fine, n, r, 1.0 / ((double)r * r), work);
   features_kernel<<<features_grid(m), kFeatThreads, 0, s>>>(work, m, 0, c->scales, c->scales + 12,
                                                      delta * delta / 12.0, x, nullptr, work + 5 * mm, t);
   CL_CUDA(c, cudaGetLastError());

@@ -41,3 +41,20 @@ def test_spectrum_of_every_transform_form(n, nbins):
     rk, rm = osp.energy_spectrum(*f, nbins=nbins)
     np.testing.assert_allclose(ek.cpu().numpy(), rk, rtol=1e-11, atol=1e-20)
     np.testing.assert_allclose(em.cpu().numpy(), rm, rtol=1e-11, atol=1e-20)
+
+
+@pytest.mark.parametrize("nx,ny,r,offset", [(6, 4, 2, 0), (258, 6, 2, 0), (258, 6, 2, 1), (9, 6, 3, 0), (600, 12, 6, 1),
+                                            (129, 129, 1, 0), (130, 130, 130, 0), (256, 300, 4, 0)])
+def test_block_mean_of_every_width_and_alignment(nx, ny, r, offset):
+    """Even and odd widths, fields on 16-byte boundaries and 8 bytes off them; r^2 additions of
+    values of order one in binary64."""
+    import torch
+    a = np.random.default_rng(nx + r).normal(size=(ny, nx))
+    buf = torch.empty(nx * ny + offset, dtype=torch.float64, device="cuda")
+    t = buf[offset:].view(ny, nx)
+    t.copy_(torch.tensor(a))
+    out = torch.full((ny // r + 1, nx // r), 9.0, dtype=torch.float64, device="cuda")
+    lbmhd.lbmhd_block_mean_device(t, r, out[:ny // r])
+    torch.cuda.synchronize()
+    np.testing.assert_allclose(out[:-1].cpu().numpy(), a.reshape(ny // r, r, nx // r, r).mean((1, 3)), rtol=0, atol=1e-14)
+    assert bool((out[-1] == 9.0).all())
