@@ -340,8 +340,14 @@ int lbmhd_probe_fp64_fma_rate(int iters, int repeats, double* dfma_per_second);
  * h is NULL.  Never NULL; valid until the next call on the same handle / thread. */
 const char* lbmhd_last_error(const lbmhd_t* h);
 
-/* Release the handle and its device memory (waits for its stream).  NULL is a no-op. */
+/* Release the handle and its device memory (waits for its stream).  NULL is a no-op.  The library
+ * keeps up to 1 GiB of device memory of freed handles for later ones (of the same grid size and
+ * precision); it is returned to the device when an allocation of the library fails, or by
+ * lbmhd_release_cached_memory. */
 void lbmhd_free(lbmhd_t* h);
+
+/* Return the device memory kept from freed handles to the device. */
+void lbmhd_release_cached_memory(void);
 
 #ifdef __cplusplus
 }

@@ -87,17 +87,20 @@ int check_params(const lbmhd_params* p) {
 
 void free_all(lbmhd_t* h) {
   if (!h) return;
-  if (h->stream) cudaStreamSynchronize(h->stream);
+  // blocks of an idle handle are kept for later ones; where its stream cannot be waited for (a
+  // caller's stream that is gone), its work may still run: wait for the device and free them
+  const bool idle = !h->stream || cudaStreamSynchronize(h->stream) == cudaSuccess;
+  if (!idle) {
+    cudaGetLastError();
+    cudaDeviceSynchronize();
+  }
   for (int i = 0; i < 2; ++i)
     if (h->graph[i]) cudaGraphExecDestroy(h->graph[i]);
-  for (int i = 0; i < 2; ++i)
-    if (h->pops[i]) cudaFree(h->pops[i]);
-  if (h->fields) cudaFree(h->fields);
-  if (h->partials) cudaFree(h->partials);
-  if (h->diag_out) cudaFree(h->diag_out);
-  if (h->err_flag) cudaFree(h->err_flag);
-  if (h->spec_work) cudaFree(h->spec_work);
-  if (h->cl_buf) cudaFree(h->cl_buf);
+  for (int i = 0; i < 2; ++i) device_free(h->pops[i], idle);
+  device_free(h->fields, idle);
+  device_free(h->partials, idle);  // and diag_out, err_flag
+  device_free(h->spec_work, idle);
+  device_free(h->cl_buf, idle);
   if (h->ev_a) cudaEventDestroy(h->ev_a);
   if (h->ev_b) cudaEventDestroy(h->ev_b);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
@@ -193,7 +196,7 @@ void* mapped_host_array(const void* ptr, size_t bytes) {
 // through it: page-locked host arrays and the device entry points never need it.
 int ensure_fields(lbmhd_t* h) {
   if (!h->fields) {
-    cudaError_t e = cudaMalloc(&h->fields, 5 * (size_t)h->p.nx * h->p.ny * sizeof(double));
+    cudaError_t e = device_alloc((void**)&h->fields, 5 * (size_t)h->p.nx * h->p.ny * sizeof(double));
     if (e != cudaSuccess) {
       h->fields = nullptr;
       return cuda_fail(h, e, "allocating the moment-field buffer");
@@ -265,10 +268,12 @@ int create(lbmhd_t** out, const lbmhd_params* p) {
   }
   LB_INIT(cudaEventCreateWithFlags(&h->ev_a, cudaEventDisableTiming));
   LB_INIT(cudaEventCreateWithFlags(&h->ev_b, cudaEventDisableTiming));
-  for (int i = 0; i < 2; ++i) LB_INIT(cudaMalloc(&h->pops[i], h->state_bytes));
-  LB_INIT(cudaMalloc(&h->partials, (size_t)kDiagBlocks * kDiagSlots * sizeof(double)));
-  LB_INIT(cudaMalloc(&h->diag_out, kDiagSlots * sizeof(double)));
-  LB_INIT(cudaMalloc(&h->err_flag, sizeof(unsigned)));
+  for (int i = 0; i < 2; ++i) LB_INIT(device_alloc(&h->pops[i], h->state_bytes));
+  // one block: diagnostics partials, their result, the pipeline status word
+  const size_t npart = (size_t)kDiagBlocks * kDiagSlots;
+  LB_INIT(device_alloc((void**)&h->partials, (npart + kDiagSlots + 1) * sizeof(double)));
+  h->diag_out = h->partials + npart;
+  h->err_flag = reinterpret_cast<unsigned*>(h->diag_out + kDiagSlots);
   LB_INIT(cudaMemsetAsync(h->err_flag, 0, sizeof(unsigned), h->stream));
   LB_INIT(prepare_step_kernels());
   for (int i = 0; i < 2; ++i) {
@@ -600,7 +605,7 @@ int lbmhd_energy_spectrum(lbmhd_t* h, int nbins, double* e_kin, double* e_mag) {
   if (n > 4096) return fail(h, LBMHD_ERR_INVALID, "spectra are limited to n <= 4096");
   if (nbins < 1 || nbins > n) return fail(h, LBMHD_ERR_INVALID, "nbins must be in [1, n]");
   const size_t wb = spectrum_work_bytes(n);
-  if (!h->spec_work) LB_CUDA(h, cudaMalloc(&h->spec_work, wb + 2 * (size_t)n * sizeof(double)));
+  if (!h->spec_work) LB_CUDA(h, device_alloc(&h->spec_work, wb + 2 * (size_t)n * sizeof(double)));
   double* dk = reinterpret_cast<double*>(static_cast<char*>(h->spec_work) + wb);
   double* dm = dk + n;
   const size_t ncell = (size_t)n * n;
@@ -645,7 +650,7 @@ int lbmhd_set_closure(lbmhd_t* h, lbmhd_closure_t* c) {
     if (h->corr_static) return fail(h, LBMHD_ERR_INVALID, "detach the static correction first");
     if (!h->cl_buf) {
       const size_t mm = (size_t)h->p.nx * h->p.ny;
-      LB_CUDA(h, cudaMalloc(&h->cl_buf, 4 * mm * sizeof(float)));
+      LB_CUDA(h, device_alloc((void**)&h->cl_buf, 4 * mm * sizeof(float)));
     }
     // the closure's parameters must be in place before this handle's stream reads them
     LB_CUDA(h, cudaStreamSynchronize(closure_stream(c)));

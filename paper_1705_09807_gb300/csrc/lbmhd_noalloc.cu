@@ -60,10 +60,12 @@ F driver_fn(const char* name, int version) {
   return reinterpret_cast<F>(f);
 }
 
+}  // namespace
+
 // Identifier of the calling thread's current context; false if it cannot be had (no current
 // context yet, or a driver without cuCtxGetId), in which case the caller looks the address up
 // afresh.
-bool current_context_id(unsigned long long* id) {
+bool lbmhd_gpu::current_context_id(unsigned long long* id) {
   static const CtxGetCurrentFn get_current = driver_fn<CtxGetCurrentFn>("cuCtxGetCurrent", 4000);
   static const CtxGetIdFn get_id = driver_fn<CtxGetIdFn>("cuCtxGetId", 12000);
   if (!get_current || !get_id) return false;
@@ -71,6 +73,8 @@ bool current_context_id(unsigned long long* id) {
   if (get_current(&ctx) != CUDA_SUCCESS || !ctx) return false;
   return get_id(ctx, id) == CUDA_SUCCESS;
 }
+
+namespace {
 
 struct PartialsAddr {
   double* ptr = nullptr;

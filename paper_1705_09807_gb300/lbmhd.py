@@ -138,6 +138,7 @@ def load_library(path: str | None = None):
             "lbmhd_step_count": (ctypes.c_int64, [_H]),
             "lbmhd_last_error": (ctypes.c_char_p, [_H]),
             "lbmhd_free": (None, [_H]),
+            "lbmhd_release_cached_memory": (None, []),
         }
         for name, (res, args) in sig.items():
             fn = getattr(lib, name)
@@ -345,6 +346,11 @@ def lbmhd_last_error(h=None) -> str:
 def lbmhd_free(h) -> None:
     if h is not None and h.value:
         load_library().lbmhd_free(h)
+
+
+def lbmhd_release_cached_memory() -> None:
+    """Return the device memory kept from freed handles (at most 1 GiB) to the device."""
+    load_library().lbmhd_release_cached_memory()
 
 
 # ---------------------------------------------------------------- convenience wrapper
