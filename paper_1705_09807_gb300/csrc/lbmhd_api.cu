@@ -577,14 +577,12 @@ int lbmhd_get_populations(lbmhd_t* h, double* pops) {
 int lbmhd_diagnostics(lbmhd_t* h, double* out) {
   if (!h) return fail(nullptr, LBMHD_ERR_INVALID, "handle is NULL");
   if (!out) return fail(h, LBMHD_ERR_INVALID, "out is NULL");
-  const size_t ncell = (size_t)h->p.nx * h->p.ny;
-  int frc = ensure_fields(h);
+  const bool through_fields = h->precision == LBMHD_FP64;
+  int frc = through_fields ? ensure_fields(h) : LBMHD_OK;
   if (frc) return frc;
-  double* f = h->fields;
-  LB_CUDA(h, launch_moments(h->precision, h->pops[h->cur], h->geom, f, f + ncell, f + 2 * ncell,
-                            f + 3 * ncell, f + 4 * ncell, h->stream));
-  LB_CUDA(h, launch_diagnostics(f, h->p.nx, h->p.ny, h->partials, h->diag_out, h->stream));
-  h->launches += 3;
+  LB_CUDA(h, launch_diagnostics(h->precision, h->pops[h->cur], h->geom, h->fields, h->partials, h->diag_out,
+                                h->stream));
+  h->launches += through_fields ? 3 : 2;
   double res[kDiagSlots];
   LB_CUDA(h, cudaMemcpyAsync(res, h->diag_out, sizeof res, cudaMemcpyDeviceToHost, h->stream));
   LB_CUDA(h, cudaStreamSynchronize(h->stream));

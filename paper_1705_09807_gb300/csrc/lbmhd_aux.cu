@@ -141,14 +141,25 @@ __device__ __forceinline__ void pull_cell(const T* __restrict__ pops, const Step
   }
 }
 
-// Exact binary64 value of a binary32 number by integer operations: GB300 converts binary32 to
-// binary64 at its binary64 rate (1/74 of its integer rate).  Subnormals, infinities and NaN take
-// the conversion instruction.
+// Exact binary64 value of a binary32 number, by integer operations alone: GB300 converts binary32
+// to binary64 at its binary64 rate (1/74 of its integer rate), and a conversion kept for the rare
+// forms is predicated, not branched around, and so takes its time on the binary64 pipe all the same.
 __device__ __forceinline__ double widen(float f) {
   const uint32_t b = __float_as_uint(f), a = b & 0x7fffffffu;
-  if (a - 0x00800000u >= 0x7f000000u && a != 0u) return (double)f;
-  const uint32_t hi = a == 0u ? 0u : (a >> 3) + 0x38000000u;
-  return __hiloint2double((int)((b & 0x80000000u) | hi), (int)(a << 29));
+  uint32_t m = a, e = 0x38000000u;  // significand with its exponent field, exponent offset
+  if (a - 0x00800000u >= 0x7f000000u) {
+    if (a >= 0x7f800000u) {  // infinity, NaN (made quiet)
+      e = 0x70000000u;
+      m = a > 0x7f800000u ? a | 0x00400000u : a;
+    } else if (a != 0u) {  // subnormal: normalise
+      const int shift = __clz(a) - 8;
+      m = a << shift;
+      e = 0x38000000u - (uint32_t)(shift << 20);
+    } else {
+      e = 0u;
+    }
+  }
+  return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + e)), (int)(m << 29));
 }
 
 // Sum of binary32 values kept exactly as the unevaluated pair hi + lo (Knuth's TwoSum: the
@@ -241,24 +252,30 @@ __device__ __forceinline__ void moments_of(const float (&v)[27], const float (&U
 // additions of every sum in binary64 the binary64 units set the time.  Binary16 values are
 // multiples of 2^-24, so while a sum's magnitudes add up to at most 1 (|f_i - w_i|, |g_i| ~ 0.1
 // in any flow this model is valid for) plain binary32 additions are exact and the pairs are not
-// needed; other cells take them.  @@MOM@@
-template <typename T, bool REL = false>
-__global__ void __launch_bounds__(128)
-    moments_kernel(const T* __restrict__ pops, StepGeom g, double* __restrict__ rho, double* __restrict__ ux,
-                   double* __restrict__ uy, double* __restrict__ bx, double* __restrict__ by) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= g.nx) return;
-  for (int y = blockIdx.y; y < g.ny; y += gridDim.y) {
+// needed; other cells take them.  Cold caches, conversions and sums in binary64 -> now: binary32
+// 2048^2 125 -> 91 us (memory: 92), binary16 4096^2 436 -> 268, relative binary16 2048^2 844 -> 88.
+// The values that a cell pulls, as stored.
+template <typename T, bool REL>
+struct CellValues {
+  T v[27];
+  T U[REL ? 8 : 1][2];  // of the source cell of f_(k+1): U_x where c_x != 0, U_y where c_y != 0
+  __device__ __forceinline__ void load(const T* __restrict__ pops, const StepGeom& g, int x, int y) {
     const T* rows[3];  // rows y - 1, y, y + 1 (sources of c_y = 1, 0, -1) at column x
 #pragma unroll
     for (int k = 0; k < 3; ++k) rows[k] = pops + (size_t)wrapi(y - 1 + k, g.ny) * g.pitch + kXOff + x;
     auto at = [&](int plane, int i) { return rows[1 - vy(i)][(size_t)plane * g.plane - vx(i)]; };
-    const size_t c = (size_t)y * g.nx + x;
-    double out[5];
-    if constexpr (sizeof(T) == 8) {
-      double v[27];
 #pragma unroll
-      for (int q = 0; q < 27; ++q) v[q] = at(plane_of(q), q % 9);
+    for (int q = 0; q < 27; ++q) v[q] = at(plane_of(q), q % 9);
+    if constexpr (REL) {
+#pragma unroll
+      for (int i = 1; i < 9; ++i) {
+        if (vx(i)) U[i - 1][0] = at(kQ, i);
+        if (vy(i)) U[i - 1][1] = at(kQ + 1, i);
+      }
+    }
+  }
+  __device__ __forceinline__ void moments(double (&out)[5]) const {
+    if constexpr (sizeof(T) == 8) {
       double r = 0, jx = 0, jy = 0, sbx = 0, sby = 0;
 #pragma unroll
       for (int i = 0; i < 9; ++i) {
@@ -274,32 +291,131 @@ __global__ void __launch_bounds__(128)
       out[3] = sbx;
       out[4] = sby;
     } else {
-      float v[27], U[8][2] = {};
+      float w[27], W[8][2] = {};
 #pragma unroll
-      for (int q = 0; q < 27; ++q) v[q] = load_as<float>(at(plane_of(q), q % 9));
+      for (int q = 0; q < 27; ++q) w[q] = load_as<float>(v[q]);
       if constexpr (REL) {
 #pragma unroll
         for (int i = 1; i < 9; ++i) {
-          if (vx(i)) U[i - 1][0] = load_as<float>(at(kQ, i));
-          if (vy(i)) U[i - 1][1] = load_as<float>(at(kQ + 1, i));
+          if (vx(i)) W[i - 1][0] = load_as<float>(U[i - 1][0]);
+          if (vy(i)) W[i - 1][1] = load_as<float>(U[i - 1][1]);
         }
       }
       if constexpr (sizeof(T) == 2) {
         float a[3] = {0.f, 0.f, 0.f};
 #pragma unroll
-        for (int q = 0; q < 27; ++q) a[q / 9] += fabsf(v[q]);
-        if (a[0] <= 1.f && a[1] <= 1.f && a[2] <= 1.f) moments_of<true, REL>(v, U, out);
-        else moments_of<false, REL>(v, U, out);
+        for (int q = 0; q < 27; ++q) a[q / 9] += fabsf(w[q]);
+        if (a[0] <= 1.f && a[1] <= 1.f && a[2] <= 1.f) moments_of<true, REL>(w, W, out);
+        else moments_of<false, REL>(w, W, out);
       } else {
-        moments_of<false, REL>(v, U, out);
+        moments_of<false, REL>(w, W, out);
       }
     }
+  }
+};
+
+template <typename T, bool REL = false>
+__global__ void __launch_bounds__(128)
+    moments_kernel(const T* __restrict__ pops, StepGeom g, double* __restrict__ rho, double* __restrict__ ux,
+                   double* __restrict__ uy, double* __restrict__ bx, double* __restrict__ by) {
+  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  if (x >= g.nx) return;
+  for (int y = blockIdx.y; y < g.ny; y += gridDim.y) {
+    const size_t c = (size_t)y * g.nx + x;
+    double out[5];
+    CellValues<T, REL> cell;
+    cell.load(pops, g, x, y);
+    cell.moments(out);
     rho[c] = out[0];
     ux[c] = out[1];
     uy[c] = out[2];
     bx[c] = out[3];
     by[c] = out[4];
   }
+}
+
+// Diagnostics of a binary32 or binary16 state, one record per block (lbmhd_diag.cuh has the slots and
+// the reduction's parts): the moments of a row are formed as moments_kernel forms them and used
+// at once, so that reading the populations runs under the reduction's binary64 instructions,
+// which bound it (30 per cell), and the moment fields are neither written nor read.  A block
+// marches a 128-column tile down its rows.  B of a row passes through shared memory to the
+// neighbouring columns; the columns beside the tile come in as single stored values, one per
+// thread and two rows ahead, which four lanes of one warp, another one each row, add up.  One
+// tile per block, four blocks per SM, tiles of at least one row: a small grid takes the time of
+// three rows.  The next row's populations are loaded before this row's binary64 work where the
+// registers allow it (not with REL's eight more values).
+// Kernels at 2048^2 binary32: moments 98 + reduction 224 -> 268 us.
+// Call of lbmhd_diagnostics with moments and reduction apart -> now: binary32 64^2 57 -> 48, 256^2 59
+// -> 58, 1024^2 146 -> 123, 2048^2 369 -> 307 us; binary16 2048^2 341 -> 281, relative 358 -> 330.
+// Three, five or six blocks per SM: 439, 343, 383 (binary32, 2048^2); REL with the early loads 396.
+constexpr int kDiagPopsBlocks = 4 * 152;
+static_assert(kDiagPopsBlocks <= kDiagBlocks, "one record per block");
+template <typename T, bool REL = false>
+__global__ void __launch_bounds__(kDiagThreads, 4)
+    diag_pops_kernel(const T* __restrict__ pops, StepGeom g, DiagTiles t, double* __restrict__ partials) {
+  static_assert(sizeof(T) <= 4, "binary32 sums");
+  constexpr bool kAhead = !REL;
+  __shared__ double sh[kDiagSlots][kDiagThreads];
+  __shared__ double sb[2][2][kDiagThreads + 2];  // [row parity][B_x, B_y][column x0 - 1 + .]
+  __shared__ T hs[2][2][18];  // [row parity][west, east][stored g value]
+  const int nx = g.nx, ny = g.ny, tid = threadIdx.x;
+  DiagAcc acc;
+  acc.clear();
+  for (long tile = blockIdx.x; tile < t.tiles; tile += gridDim.x) {
+    const int x0 = (int)(tile % t.strips) * kDiagThreads, cols = min(kDiagThreads, nx - x0);
+    const int y0 = (int)(tile / t.strips) * t.rows, y1 = min(y0 + t.rows, ny);
+    // threads 0 .. 35: one stored g value of the column west (0 .. 17) or east of the tile
+    const bool halo = tid < 36;
+    const int side = tid / 18, q = 9 + tid % 18, i = q % 9;
+    const int hx = side ? (x0 + cols == nx ? 0 : x0 + cols) : (x0 == 0 ? nx - 1 : x0 - 1);
+    auto load_halo = [&](int y) {  // y <= y1 + 2
+      int yy = y - vel_y(i);
+      yy = yy < 0 ? yy + ny : yy % ny;
+      return pops[(size_t)yy * g.pitch + (size_t)plane_of(q) * g.plane + kXOff + hx - vel_x(i)];
+    };
+    T hv = T(0);
+    if (halo) {
+      hs[1][side][q - 9] = load_halo(y0 - 1);
+      hv = load_halo(y0);
+    }
+    DiagRows rows;
+    CellValues<T, REL> cell;
+    if (kAhead && tid < cols) cell.load(pops, g, x0 + tid, wrapi(y0 - 1, ny));
+    __syncthreads();
+    for (int y = y0 - 1; y <= y1; ++y) {  // row y arrives in slot 2
+      const int par = (y - y0) & 1;
+      double m[5];
+      if (halo) {
+        hs[par ^ 1][side][q - 9] = hv;  // row y + 1
+        if (y < y1) hv = load_halo(y + 2);
+      }
+      if (tid < cols) {
+        if (!kAhead) cell.load(pops, g, x0 + tid, wrapi(y, ny));
+        cell.moments(m);
+        if (kAhead && y < y1) cell.load(pops, g, x0 + tid, wrapi(y + 1, ny));
+        sb[par][0][tid + 1] = m[3];
+        sb[par][1][tid + 1] = m[4];
+        if (y >= y0 && y < y1) acc.add_cell(m[0], m[1], m[2], m[3], m[4]);
+      }
+      const int lane = tid - (((y - y0) & 3) << 5);
+      if (lane >= 0 && lane < 4) {  // B_x, B_y beside the tile, summed as CellValues::moments does
+        const T* h = hs[par][lane >> 1] + 9 * (lane & 1);
+        PairSum p;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) p.add(load_as<float>(h[k]));
+        sb[par][lane & 1][lane >> 1 ? cols + 1 : 0] = p.value();
+      }
+      __syncthreads();  // the buffers of this parity are rewritten after the next row's barrier
+      if (tid < cols) {
+#pragma unroll
+        for (int f = 0; f < 2; ++f) rows.set(f, 2, m[3 + f], sb[par][f][tid + 2], sb[par][f][tid]);
+        if (y > y0) rows.add_to(acc);
+        rows.advance();
+      }
+    }
+    __syncthreads();
+  }
+  diag_record(acc, sh, partials + (size_t)blockIdx.x * kDiagSlots);
 }
 
 template <typename T, bool REL = false>
@@ -401,12 +517,27 @@ cudaError_t launch_populations(int precision, const void* pops, const StepGeom& 
   return cudaGetLastError();
 }
 
-cudaError_t launch_diagnostics(const double* fields, int nx, int ny, double* partials, double* out,
-                               cudaStream_t s) {
-  const size_t n = (size_t)nx * ny;
-  const DiagTiles t = diag_tiles(nx, ny, kDiagBlocks);
-  diag_partial_kernel<<<t.blocks, kDiagThreads, 0, s>>>(fields, fields + n, fields + 2 * n, fields + 3 * n,
-                                                         fields + 4 * n, nx, ny, t, partials);
+cudaError_t launch_diagnostics(int precision, const void* pops, const StepGeom& g, double* fields, double* partials,
+                               double* out, cudaStream_t s) {
+  // binary64 moments take about 50 binary64 instructions a cell, too many to form them again in
+  // the tiles' halo rows: lbmhd_diagnostics at 256^2 60 us through the fields, 80 straight from the
+  // populations; 2048^2 751 and 777
+  const bool through_fields = precision == 0;
+  const DiagTiles t = through_fields ? diag_tiles(g.nx, g.ny, kDiagBlocks) : diag_tiles(g.nx, g.ny, kDiagPopsBlocks, 1);
+  if (through_fields) {
+    const size_t n = (size_t)g.nx * g.ny;
+    cudaError_t e = launch_moments(precision, pops, g, fields, fields + n, fields + 2 * n, fields + 3 * n,
+                                   fields + 4 * n, s);
+    if (e != cudaSuccess) return e;
+    diag_partial_kernel<<<t.blocks, kDiagThreads, 0, s>>>(fields, fields + n, fields + 2 * n, fields + 3 * n,
+                                                           fields + 4 * n, g.nx, g.ny, t, partials);
+  } else if (precision == 1) {
+    diag_pops_kernel<float><<<t.blocks, kDiagThreads, 0, s>>>((const float*)pops, g, t, partials);
+  } else if (precision == LBMHD_FP16) {
+    diag_pops_kernel<__half><<<t.blocks, kDiagThreads, 0, s>>>((const __half*)pops, g, t, partials);
+  } else {
+    diag_pops_kernel<__half, true><<<t.blocks, kDiagThreads, 0, s>>>((const __half*)pops, g, t, partials);
+  }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   diag_final_kernel<<<1, 32 * kDiagSlots, 0, s>>>(partials, t.blocks, out);

@@ -1,5 +1,6 @@
-// Diagnostics reduction over five device moment fields rho, ux, uy, bx, by [ny][nx] (periodic),
-// shared by lbmhd_diagnostics (moment fields of a handle) and lbmhd_diagnostics_fields_noalloc.
+// Diagnostics reduction over five device moment fields rho, ux, uy, bx, by [ny][nx] (periodic), for
+// lbmhd_diagnostics_fields_noalloc and binary64 states, and its parts, which binary32 and binary16
+// states apply to moments taken straight from the populations (diag_pops_kernel, lbmhd_aux.cu).
 //
 // Slots of a record: 0 sum rho, 1 sum Jx, 2 sum Jy, 3 sum Bx, 4 sum By, 5 sum rho |u|^2 / 2,
 // 6 sum |B|^2 / 2, 7 max |div B| (isotropic), 8 max |div B| (central), 9 max |d_beta B_alpha|
@@ -30,11 +31,11 @@ struct DiagTiles {
   int strips, rows, blocks;
   long tiles;
 };
-inline DiagTiles diag_tiles(int nx, int ny, int max_blocks) {
+inline DiagTiles diag_tiles(int nx, int ny, int max_blocks, int min_rows = kDiagMinRows) {
   DiagTiles t;
   t.strips = (nx + kDiagThreads - 1) / kDiagThreads;
   const long rows = ((long)t.strips * ny + max_blocks - 1) / max_blocks;
-  t.rows = (int)(rows < kDiagMinRows ? kDiagMinRows : (rows > ny ? ny : rows));
+  t.rows = (int)(rows < min_rows ? min_rows : (rows > ny ? ny : rows));
   t.tiles = (long)t.strips * ((ny + t.rows - 1) / t.rows);
   t.blocks = (int)(t.tiles < max_blocks ? t.tiles : max_blocks);
   return t;
@@ -53,77 +54,75 @@ __device__ __forceinline__ bool not_finite(double v) { return (__double2hiint(v)
 // Combine two records' slot k (max for the non-negative maxima and the flag).
 __device__ __forceinline__ double diag_combine(int k, double a, double b) { return k <= 6 ? a + b : (b > a ? b : a); }
 
-// One record per block into partials[blockIdx.x].
-__global__ void __launch_bounds__(kDiagThreads)
-    diag_partial_kernel(const double* __restrict__ rho, const double* __restrict__ ux, const double* __restrict__ uy,
-                        const double* __restrict__ bx, const double* __restrict__ by, int nx, int ny, DiagTiles t,
-                        double* __restrict__ partials) {
+// A thread's part of a record: sums of its cells, maxima (bits) and flag.
+struct DiagAcc {
   double sum[7];
-  unsigned long long mx[3] = {0, 0, 0};
-  bool bad = false;
+  unsigned long long mx[3];
+  bool bad;
+  __device__ __forceinline__ void clear() {
 #pragma unroll
-  for (int k = 0; k < 7; ++k) sum[k] = 0.0;
-  for (long tile = blockIdx.x; tile < t.tiles; tile += gridDim.x) {
-    const int x = (int)(tile % t.strips) * kDiagThreads + threadIdx.x;
-    const int y0 = (int)(tile / t.strips) * t.rows, y1 = min(y0 + t.rows, ny);
-    if (x >= nx) continue;
-    const int xe = x + 1 == nx ? 0 : x + 1, xw = x == 0 ? nx - 1 : x - 1;
-    // rows y - 1, y, y + 1 in slots 0, 1, 2: value, D and S of B_x and B_y
-    double a[2][3], D[2][3], S[2][3];
-    auto row = [&](int y, int k) {
-      const size_t o = (size_t)(y < 0 ? y + ny : (y >= ny ? y - ny : y)) * nx;
+    for (int k = 0; k < 7; ++k) sum[k] = 0.0;
 #pragma unroll
-      for (int f = 0; f < 2; ++f) {
-        const double* p = (f ? by : bx) + o;
-        const double e = p[xe], w = p[xw];
-        a[f][k] = p[x];
-        D[f][k] = e - w;
-        S[f][k] = fma(0.25, e + w, a[f][k]);
-      }
-    };
-    row(y0 - 1, 0);
-    row(y0, 1);
-    for (int y = y0; y < y1; ++y) {
-      row(y + 1, 2);
-      const size_t c = (size_t)y * nx + x;
-      const double r = rho[c], u = ux[c], v = uy[c], b = a[0][1], d = a[1][1];
-      const double q = fma(u, u, v * v);
-      sum[0] += r;
-      sum[1] = fma(r, u, sum[1]);
-      sum[2] = fma(r, v, sum[2]);
-      sum[3] += b;
-      sum[4] += d;
-      sum[5] = fma(r, q, sum[5]);
-      sum[6] = fma(b, b, fma(d, d, sum[6]));
-      double dx[2], dy[2];  // three times the isotropic derivatives
-#pragma unroll
-      for (int f = 0; f < 2; ++f) {
-        dx[f] = fma(0.25, D[f][0] + D[f][2], D[f][1]);
-        dy[f] = S[f][2] - S[f][0];
-      }
-      mx[0] = max(mx[0], abs_bits(dx[0] + dy[1]));
-      mx[1] = max(mx[1], abs_bits(D[0][1] + (a[1][2] - a[1][0])));
-      mx[2] = max(max(mx[2], max(abs_bits(dx[0]), abs_bits(dy[0]))), max(abs_bits(dx[1]), abs_bits(dy[1])));
-      // not (rho > 0 and |u|^2 <= 0.16), or anything not finite
-      bad = bad || not_finite(r) || not_finite(u) || not_finite(v) || not_finite(b) || not_finite(d) ||
-            __double_as_longlong(r) <= 0 || __double_as_longlong(q) > __double_as_longlong(0.16);
-#pragma unroll
-      for (int f = 0; f < 2; ++f)
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-          a[f][k] = a[f][k + 1];
-          D[f][k] = D[f][k + 1];
-          S[f][k] = S[f][k + 1];
-        }
-    }
+    for (int k = 0; k < 3; ++k) mx[k] = 0;
+    bad = false;
   }
-  __shared__ double sh[kDiagSlots][kDiagThreads];
+  __device__ __forceinline__ void add_cell(double r, double u, double v, double b, double d) {
+    const double q = fma(u, u, v * v);
+    sum[0] += r;
+    sum[1] = fma(r, u, sum[1]);
+    sum[2] = fma(r, v, sum[2]);
+    sum[3] += b;
+    sum[4] += d;
+    sum[5] = fma(r, q, sum[5]);
+    sum[6] = fma(b, b, fma(d, d, sum[6]));
+    // not (rho > 0 and |u|^2 <= 0.16), or anything not finite
+    bad = bad || not_finite(r) || not_finite(u) || not_finite(v) || not_finite(b) || not_finite(d) ||
+          __double_as_longlong(r) <= 0 || __double_as_longlong(q) > __double_as_longlong(0.16);
+  }
+};
+
+// Rows y - 1, y, y + 1 of one column in slots 0, 1, 2: value, D and S of B_x and B_y.
+struct DiagRows {
+  double a[2][3], D[2][3], S[2][3];
+  __device__ __forceinline__ void set(int f, int k, double v, double e, double w) {
+    a[f][k] = v;
+    D[f][k] = e - w;
+    S[f][k] = fma(0.25, e + w, v);
+  }
+  // the derivatives of row y
+  __device__ __forceinline__ void add_to(DiagAcc& acc) const {
+    double dx[2], dy[2];  // three times the isotropic derivatives
 #pragma unroll
-  for (int k = 0; k < 7; ++k) sh[k][threadIdx.x] = (k >= 5 ? 0.5 : 1.0) * sum[k];
+    for (int f = 0; f < 2; ++f) {
+      dx[f] = fma(0.25, D[f][0] + D[f][2], D[f][1]);
+      dy[f] = S[f][2] - S[f][0];
+    }
+    acc.mx[0] = max(acc.mx[0], abs_bits(dx[0] + dy[1]));
+    acc.mx[1] = max(acc.mx[1], abs_bits(D[0][1] + (a[1][2] - a[1][0])));
+    acc.mx[2] =
+        max(max(acc.mx[2], max(abs_bits(dx[0]), abs_bits(dy[0]))), max(abs_bits(dx[1]), abs_bits(dy[1])));
+  }
+  __device__ __forceinline__ void advance() {
+#pragma unroll
+    for (int f = 0; f < 2; ++f)
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        a[f][k] = a[f][k + 1];
+        D[f][k] = D[f][k + 1];
+        S[f][k] = S[f][k + 1];
+      }
+  }
+};
+
+// The block's record: its threads' parts by halves.
+__device__ __forceinline__ void diag_record(const DiagAcc& acc, double (&sh)[kDiagSlots][kDiagThreads],
+                                            double* __restrict__ rec) {
+#pragma unroll
+  for (int k = 0; k < 7; ++k) sh[k][threadIdx.x] = (k >= 5 ? 0.5 : 1.0) * acc.sum[k];
 #pragma unroll
   for (int k = 0; k < 3; ++k)
-    sh[7 + k][threadIdx.x] = (k == 1 ? 0.5 : 1.0 / 3.0) * __longlong_as_double((long long)mx[k]);
-  sh[10][threadIdx.x] = bad ? 1.0 : 0.0;
+    sh[7 + k][threadIdx.x] = (k == 1 ? 0.5 : 1.0 / 3.0) * __longlong_as_double((long long)acc.mx[k]);
+  sh[10][threadIdx.x] = acc.bad ? 1.0 : 0.0;
   __syncthreads();
   for (int w = kDiagThreads / 2; w > 0; w >>= 1) {
     if ((int)threadIdx.x < w) {
@@ -133,7 +132,42 @@ __global__ void __launch_bounds__(kDiagThreads)
     }
     __syncthreads();
   }
-  if (threadIdx.x < kDiagSlots) partials[(size_t)blockIdx.x * kDiagSlots + threadIdx.x] = sh[threadIdx.x][0];
+  if (threadIdx.x < kDiagSlots) rec[threadIdx.x] = sh[threadIdx.x][0];
+}
+
+// One record per block into partials[blockIdx.x].
+__global__ void __launch_bounds__(kDiagThreads)
+    diag_partial_kernel(const double* __restrict__ rho, const double* __restrict__ ux, const double* __restrict__ uy,
+                        const double* __restrict__ bx, const double* __restrict__ by, int nx, int ny, DiagTiles t,
+                        double* __restrict__ partials) {
+  DiagAcc acc;
+  acc.clear();
+  for (long tile = blockIdx.x; tile < t.tiles; tile += gridDim.x) {
+    const int x = (int)(tile % t.strips) * kDiagThreads + threadIdx.x;
+    const int y0 = (int)(tile / t.strips) * t.rows, y1 = min(y0 + t.rows, ny);
+    if (x >= nx) continue;
+    const int xe = x + 1 == nx ? 0 : x + 1, xw = x == 0 ? nx - 1 : x - 1;
+    DiagRows rows;
+    auto row = [&](int y, int k) {
+      const size_t o = (size_t)(y < 0 ? y + ny : (y >= ny ? y - ny : y)) * nx;
+#pragma unroll
+      for (int f = 0; f < 2; ++f) {
+        const double* p = (f ? by : bx) + o;
+        rows.set(f, k, p[x], p[xe], p[xw]);
+      }
+    };
+    row(y0 - 1, 0);
+    row(y0, 1);
+    for (int y = y0; y < y1; ++y) {
+      row(y + 1, 2);
+      const size_t c = (size_t)y * nx + x;
+      acc.add_cell(rho[c], ux[c], uy[c], rows.a[0][1], rows.a[1][1]);
+      rows.add_to(acc);
+      rows.advance();
+    }
+  }
+  __shared__ double sh[kDiagSlots][kDiagThreads];
+  diag_record(acc, sh, partials + (size_t)blockIdx.x * kDiagSlots);
 }
 
 // out[k] = records combined in a fixed order: warp k takes slot k, each lane every 32nd record,
