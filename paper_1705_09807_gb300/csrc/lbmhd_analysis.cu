@@ -32,35 +32,55 @@
 namespace lbmhd_gpu {
 namespace {
 
-// Memory-bound (8 bytes in per cell), so what matters is loads in flight: a thread adds up one
+// s 2^-k, by its exponent where that is exact; the product is a call, so that it is branched
+// around (predicated, it would take its time on the binary64 pipe in every thread).
+__device__ __noinline__ double scaled_product(double s, double inv) { return s * inv; }
+__device__ __forceinline__ double scale_down(double s, int k, double inv) {
+  const int hi = __double2hiint(s), ex = (hi >> 20) & 0x7ff;
+  if (ex > k && ex < 0x7ff) return __hiloint2double(hi - (k << 20), __double2loint(s));
+  if (((hi & 0x7fffffff) | __double2loint(s)) == 0) return s;
+  return scaled_product(s, inv);  // subnormal results, infinities, NaN
+}
+
+// Bound by memory (8 bytes in per cell) and, nearly as much, by binary64 instructions (at r = 2 the
+// three additions of a coarse cell take 6 us for 2048^2, its bytes as long): a thread adds up one
 // coarse cell, row by row from the left, with the loads of a row independent of one another; a
 // warp reads whole rows of the fine field.  VEC: 16-byte loads (r even, rows and field on 16-byte
-// boundaries).  2048^2, r = 2, cold caches: 24.5 us with 64-bit divisions per cell and a grid-stride
-// loop (a division by r^2 in every thread cost another binary64 dozen); now 14.8 us.
+// boundaries).  log2sq: 2 log2 r, or -1 when r is no power of two and the mean takes a product.
+// 2048^2, r = 2, cold caches: 24.5 us with 64-bit divisions per cell and a grid-stride loop (a division
+// by r^2 in every thread cost another binary64 dozen), 13.9 with a first addition to zero and a
+// product in every thread, now 10.1 us.
 template <bool VEC>
 __global__ void __launch_bounds__(128)
-    block_mean_kernel(const double* __restrict__ in, int nx, int mx, int my, int r, double inv,
+    block_mean_kernel(const double* __restrict__ in, int nx, int mx, int my, int r, int log2sq, double inv,
                       double* __restrict__ out) {
   const int i = blockIdx.x * 128 + threadIdx.x;
   if (i >= mx) return;
   for (int j = blockIdx.y; j < my; j += gridDim.y) {
     const double* row = in + (size_t)j * r * nx + (size_t)i * r;
-    double s = 0.0;
+    double s;
+    if constexpr (VEC) {
+      const double2 v = *reinterpret_cast<const double2*>(row);
+      s = v.x + v.y;
+    } else {
+      s = row[0];
+    }
+    int first = VEC ? 2 : 1;  // of this row
 #pragma unroll 2
-    for (int yy = 0; yy < r; ++yy, row += nx) {
+    for (int yy = 0; yy < r; ++yy, row += nx, first = 0) {
       if constexpr (VEC) {
 #pragma unroll 4
-        for (int xx = 0; xx < r; xx += 2) {
+        for (int xx = first; xx < r; xx += 2) {
           const double2 v = *reinterpret_cast<const double2*>(row + xx);
           s += v.x;
           s += v.y;
         }
       } else {
 #pragma unroll 4
-        for (int xx = 0; xx < r; ++xx) s += row[xx];
+        for (int xx = first; xx < r; ++xx) s += row[xx];
       }
     }
-    out[(size_t)j * mx + i] = s * inv;
+    out[(size_t)j * mx + i] = log2sq >= 0 ? scale_down(s, log2sq, inv) : scaled_product(s, inv);
   }
 }
 
@@ -486,11 +506,14 @@ cudaError_t launch_energy_spectrum(const double* ux, const double* uy, const dou
 cudaError_t launch_block_mean(const double* in, int nx, int ny, int r, double* out, cudaStream_t s) {
   const int mx = nx / r, my = ny / r;
   const double inv = 1.0 / ((double)r * r);  // a binary64 division per thread would outweigh the sums
+  int log2sq = -1;
+  if ((r & (r - 1)) == 0)
+    for (log2sq = 0; (1 << (log2sq / 2)) < r;) log2sq += 2;
   const dim3 grid((mx + 127) / 128, my < 65535 ? my : 65535);
   if (r % 2 == 0 && nx % 2 == 0 && reinterpret_cast<uintptr_t>(in) % 16 == 0)
-    block_mean_kernel<true><<<grid, 128, 0, s>>>(in, nx, mx, my, r, inv, out);
+    block_mean_kernel<true><<<grid, 128, 0, s>>>(in, nx, mx, my, r, log2sq, inv, out);
   else
-    block_mean_kernel<false><<<grid, 128, 0, s>>>(in, nx, mx, my, r, inv, out);
+    block_mean_kernel<false><<<grid, 128, 0, s>>>(in, nx, mx, my, r, log2sq, inv, out);
   return cudaGetLastError();
 }
 
