@@ -917,8 +917,10 @@ cudaError_t launch_net(const float* in, const unsigned char* packed, const float
 // Bound by GB300's binary64 rate, not by the 40 bytes per fine cell: with J = rho u the quotients
 // are products (J_x J_y / rho = J_x u_y, ...), 17 binary64 instructions per fine cell instead of
 // about 57 with four divisions.  A thread adds up one fine column of a coarse row, so the loads
-// are coalesced and a coarse cell occupies r threads; the r columns are then added in order.
-// 2048^2, r = 8, cold caches: 481 -> 142 us.
+// are coalesced and a coarse cell occupies r threads; the r columns are then added in order, by
+// one thread per sum and cell (one per cell, half a warp with nine sums each, cost a tenth of the
+// binary64 issue).  2048^2, r = 8, cold caches: 481 us with quotients, 141 with one adding thread
+// per cell, now 129.
 constexpr int kFilterThreads = 128;
 __global__ void __launch_bounds__(kFilterThreads)
     filter_products_kernel(const double* __restrict__ fine, int n, int r, double inv, double* __restrict__ coarse) {
@@ -929,7 +931,7 @@ __global__ void __launch_bounds__(kFilterThreads)
   const int cells = r <= kFilterThreads ? kFilterThreads / r : 1;
   for (int j = blockIdx.y; j < m; j += gridDim.y) {
     const int i0 = blockIdx.x * cells;
-    const int cols = min(cells, m - i0) * r;
+    const int ncell = min(cells, m - i0), cols = ncell * r;
     double tot[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
     for (int c0 = 0; c0 < cols; c0 += kFilterThreads) {
       const int x = c0 + (int)threadIdx.x, w = min(kFilterThreads, cols - c0);
@@ -957,18 +959,25 @@ __global__ void __launch_bounds__(kFilterThreads)
 #pragma unroll
       for (int k = 0; k < 9; ++k) sh[k][threadIdx.x] = s[k];
       __syncthreads();
-      // coarse cell t of the block (one when r exceeds the block): its columns of this pass
-      const int first = r <= kFilterThreads ? threadIdx.x * r : 0, num = r <= kFilterThreads ? r : w;
-      if ((int)threadIdx.x < (r <= kFilterThreads ? cols / r : 1)) {
-        for (int q = 0; q < num; ++q)
+      // the 9 sums of the block's coarse cells (one when r exceeds the block), one (sum, cell) pair per
+      // thread and turn: its columns of this pass, in order
+      const int num = r <= kFilterThreads ? r : w;
 #pragma unroll
-          for (int k = 0; k < 9; ++k) tot[k] += sh[k][first + q];
+      for (int k = 0; k < 9; ++k) {
+        const int e = k * kFilterThreads + (int)threadIdx.x;
+        if (e < 9 * ncell) {
+          const double* col = &sh[e / ncell][e % ncell * num];
+          double t = c0 == 0 ? col[0] : tot[k] + col[0];
+          for (int q = 1; q < num; ++q) t += col[q];
+          tot[k] = t;
+        }
       }
       __syncthreads();
     }
-    if ((int)threadIdx.x < cols / r) {
 #pragma unroll
-      for (int k = 0; k < 9; ++k) coarse[k * mm + (size_t)j * m + i0 + threadIdx.x] = tot[k] * inv;
+    for (int k = 0; k < 9; ++k) {
+      const int e = k * kFilterThreads + (int)threadIdx.x;
+      if (e < 9 * ncell) coarse[e / ncell * mm + (size_t)j * m + i0 + e % ncell] = tot[k] * inv;
     }
   }
 }
