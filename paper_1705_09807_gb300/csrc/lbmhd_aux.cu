@@ -5,6 +5,7 @@
 
 #include "lbmhd_diag.cuh"
 #include "lbmhd_internal.cuh"
+#include "lbmhd_quotient.cuh"
 
 namespace lbmhd_gpu {
 namespace {
@@ -254,23 +255,6 @@ __device__ __forceinline__ void moments_of(const float (&v)[27], const float (&U
 // in any flow this model is valid for) plain binary32 additions are exact and the pairs are not
 // needed; other cells take them.  Cold caches, conversions and sums in binary64 -> now: binary32
 // 2048^2 125 -> 91 us (memory: 92), binary16 4096^2 436 -> 268, relative binary16 2048^2 844 -> 88.
-// a / b from y = 1 / b rounded to nearest: Markstein's correction (IBM J. Res. Dev. 34 (1990) 111)
-// of a y by its exact residual, the correctly rounded quotient but for ties that 2^-100 decides.
-// in_range: exponents for which nothing over- or underflows on the way; is_zero: +-0, by integer
-// tests.  With the terms of zero c left out and one reciprocal for both velocities, the moments of
-// a binary64 state take 46 binary64 instructions a cell instead of 62: 2048^2 497 -> 363 us.
-__device__ __forceinline__ double quotient(double a, double b, double y) {
-  const double q = a * y;
-  return fma(fma(-q, b, a), y, q);
-}
-__device__ __forceinline__ bool in_range(double v) {
-  return ((unsigned)__double2hiint(v) & 0x7fffffffu) - 0x30000000u < 0x20000000u;  // 2^-255 .. 2^257
-}
-
-__device__ __forceinline__ bool is_zero(double v) {
-  return (((unsigned)__double2hiint(v) & 0x7fffffffu) | (unsigned)__double2loint(v)) == 0u;
-}
-
 // The values that a cell pulls, as stored.
 template <typename T, bool REL>
 struct CellValues {
@@ -293,6 +277,8 @@ struct CellValues {
   }
   __device__ __forceinline__ void moments(double (&out)[5]) const {
     if constexpr (sizeof(T) == 8) {
+      // with the terms of zero c left out and one reciprocal for both velocities 46 binary64
+      // instructions a cell instead of 62: 2048^2 497 -> 363 us
       double r = v[0], jx = v[1], jy = v[2], sbx = v[9], sby = v[18];
 #pragma unroll
       for (int i = 1; i < 9; ++i) {
@@ -305,7 +291,7 @@ struct CellValues {
       out[0] = 1.0 + r;
       out[3] = sbx;
       out[4] = sby;
-      if (in_range(out[0]) && (in_range(jx) || is_zero(jx)) && (in_range(jy) || is_zero(jy))) {
+      if (quotient_in_range(jx, out[0]) && quotient_in_range(jy, out[0])) {
         const double y = __drcp_rn(out[0]);
         out[1] = quotient(jx, out[0], y);
         out[2] = quotient(jy, out[0], y);

@@ -23,6 +23,7 @@
 #include "lbmhd.h"
 #include "lbmhd_handle.h"
 #include "lbmhd_internal.cuh"
+#include "lbmhd_quotient.cuh"
 #include "lbmhd_ptx.cuh"
 
 namespace lbmhd_gpu {
@@ -915,12 +916,12 @@ cudaError_t launch_net(const float* in, const unsigned char* packed, const float
 // [7] (Jx^2+Jy^2)/rho; [8] (Jx By - Jy Bx)/rho.
 //
 // Bound by GB300's binary64 rate, not by the 40 bytes per fine cell: with J = rho u the quotients
-// are products (J_x J_y / rho = J_x u_y, ...), 17 binary64 instructions per fine cell instead of
+// are products (J_x J_y / rho = J_x u_y, ...), 15 binary64 instructions per fine cell instead of
 // about 57 with four divisions.  A thread adds up one fine column of a coarse row, so the loads
 // are coalesced and a coarse cell occupies r threads; the r columns are then added in order, by
 // one thread per sum and cell (one per cell, half a warp with nine sums each, cost a tenth of the
 // binary64 issue).  2048^2, r = 8, cold caches: 481 us with quotients, 141 with one adding thread
-// per cell, now 129.
+// per cell, 129 with sums that began at zero, now 126.
 constexpr int kFilterThreads = 128;
 __global__ void __launch_bounds__(kFilterThreads)
     filter_products_kernel(const double* __restrict__ fine, int n, int r, double inv, double* __restrict__ coarse) {
@@ -935,10 +936,27 @@ __global__ void __launch_bounds__(kFilterThreads)
     double tot[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
     for (int c0 = 0; c0 < cols; c0 += kFilterThreads) {
       const int x = c0 + (int)threadIdx.x, w = min(kFilterThreads, cols - c0);
-      double s[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0}, a = 0, b = 0, c = 0, d = 0;
+      double s[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
       if (x < cols) {
         const double* p = fine + (size_t)j * r * n + (size_t)i0 * r + x;
-        for (int yy = 0; yy < r; ++yy, p += n) {
+        double a, b, c, d;
+        {  // the first row starts the sums: additions to zero are binary64 instructions too
+          const double rho = p[0], ux = p[nn], uy = p[2 * nn], bx = p[3 * nn], by = p[4 * nn];
+          const double jx = rho * ux, jy = rho * uy;
+          s[0] = rho;
+          s[1] = jx;
+          s[2] = jy;
+          s[3] = bx;
+          s[4] = by;
+          s[5] = fma(jx, uy, -bx * by);
+          a = jx * ux;
+          b = jy * uy;
+          c = bx * bx;
+          d = by * by;
+          s[8] = fma(ux, by, -uy * bx);
+        }
+        for (int yy = 1; yy < r; ++yy) {
+          p += n;
           const double rho = p[0], ux = p[nn], uy = p[2 * nn], bx = p[3 * nn], by = p[4 * nn];
           const double jx = rho * ux, jy = rho * uy;
           s[0] += rho;
@@ -989,8 +1007,10 @@ __global__ void __launch_bounds__(kFilterThreads)
 // `target`.
 //
 // Bound by binary64 divisions and their latency: a block forms u and J of its 32 x 4 cells and a
-// ring of one cell once in shared memory (two divisions per cell instead of ten), and scales by
-// reciprocals formed once per block.  256^2, cold caches: 56 -> 25 us.
+// ring of one cell once in shared memory (one reciprocal per cell instead of ten divisions), and
+// scales by reciprocals formed once per block.  256^2, cold caches: 56 -> 24 with two divisions per
+// cell -> 21 us.
+__device__ __noinline__ double divided(double a, double b) { return a / b; }  // a call: branched around
 constexpr int kFeatW = 32, kFeatH = 4, kFeatThreads = kFeatW * kFeatH;
 __global__ void __launch_bounds__(kFeatThreads)
     features_kernel(const double* __restrict__ st, int m, int velocity, const float* __restrict__ in_scale,
@@ -999,6 +1019,7 @@ __global__ void __launch_bounds__(kFeatThreads)
   constexpr int PW = kFeatW + 2, PH = kFeatH + 2;
   __shared__ double u[4][PH][PW];  // u_x, u_y, B_x, B_y
   __shared__ double J[2][PH][PW];
+  __shared__ double Ri[PH][PW];    // 1 / rho (not when `velocity`)
   __shared__ double inv[16];       // 1 / in_scale[12], 1 / out_scale[4]
   const size_t mm = (size_t)m * m;
   const int tid = threadIdx.x, lx = tid % kFeatW, ly = tid / kFeatW;
@@ -1010,13 +1031,22 @@ __global__ void __launch_bounds__(kFeatThreads)
     for (int e = tid; e < PW * PH; e += kFeatThreads) {
       const int px = e % PW, py = e / PW;
       const size_t o = (size_t)wrap_mod(y0 - 1 + py, m) * m + wrap_mod(x0 - 1 + px, m);
-      const double rho = st[o];
-#pragma unroll
-      for (int f = 0; f < 2; ++f) {
-        const double v = st[(1 + f) * mm + o];
-        J[f][py][px] = velocity ? rho * v : v;
-        u[f][py][px] = velocity ? v : v / rho;
-        u[2 + f][py][px] = st[(3 + f) * mm + o];
+      const double rho = st[o], v0 = st[mm + o], v1 = st[2 * mm + o];
+      u[2][py][px] = st[3 * mm + o];
+      u[3][py][px] = st[4 * mm + o];
+      if (velocity) {
+        J[0][py][px] = rho * v0;
+        J[1][py][px] = rho * v1;
+        u[0][py][px] = v0;
+        u[1][py][px] = v1;
+      } else {
+        const double y = __drcp_rn(rho);
+        const bool fast = quotient_in_range(v0, rho) && quotient_in_range(v1, rho);
+        J[0][py][px] = v0;
+        J[1][py][px] = v1;
+        u[0][py][px] = fast ? quotient(v0, rho, y) : divided(v0, rho);
+        u[1][py][px] = fast ? quotient(v1, rho, y) : divided(v1, rho);
+        Ri[py][px] = y;
       }
     }
     __syncthreads();
@@ -1039,7 +1069,7 @@ __global__ void __launch_bounds__(kFeatThreads)
       }
       if (analytic || target) {
         const double gj[4] = {ddx(J[0]), ddy(J[0]), ddx(J[1]), ddy(J[1])};
-        const double ir = 1.0 / st[c];
+        const double ir = velocity ? divided(1.0, st[c]) : Ri[ly + 1][lx + 1];
         const double Gxx = gj[0] * gj[0] + gj[1] * gj[1], Gyy = gj[2] * gj[2] + gj[3] * gj[3];
         const double Gxy = gj[0] * gj[2] + gj[1] * gj[3];
         const double Hxx = gb[0] * gb[0] + gb[1] * gb[1], Hyy = gb[2] * gb[2] + gb[3] * gb[3];
