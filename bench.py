@@ -43,7 +43,9 @@ sys.path.insert(0, ROOT)
 METRIC = "MLUPS and % HBM roofline per LES-LB-MHD step vs plain FP64 step, at stated L2 err"
 # 27 populations read + 27 written (binary16 relative to the local velocity: + 2 velocity planes)
 BYTES_PER_CELL = {"fp16": 108, "fp16rel": 116, "fp32": 216, "fp64": 432}
-FP64_INSTR_PER_CELL = 173  # binary64 instructions per cell-update of the FP64 step (ncu)
+# binary64 instructions per cell-update of the FP64 step (ncu): Delta = 0 71 DADD + 53 DFMA + 16 DMUL,
+# filtered 80 + 69 + 22
+FP64_INSTR_PER_CELL = {"plain": 140, "filtered": 171}
 MIN_WINDOWS = 5          # timed K-step windows, at least
 MIN_TIMED_S = 1.0        # and at least this much timed time in all
 NU = ETA = 2e-3   # see the module docstring
@@ -55,8 +57,8 @@ NU = ETA = 2e-3   # see the module docstring
 # until it is measured again.
 MEASURED_TRAFFIC = {
     # profiles/fused_step_fp32_2048.md: mean of three launches after 40 steps,
-    # (427.75 + 456.60, 426.48 + 451.04, 425.13 + 452.07) MB
-    ("c53ace2ee372db81", 2048, "fp32", 0.0): 879.69e6,
+    # (427.91 + 456.75, 425.98 + 450.80, 425.08 + 451.97) MB
+    ("6b149356a9b026d7", 2048, "fp32", 0.0): 879.50e6,
 }
 
 
@@ -445,11 +447,10 @@ def side_measurements(n, a):
                                     "256 threads, median CUDA-event time of 5 launches after one "
                                     "warm-up launch, fastest shape"}
 
-    def fp64_line(nn, ms64):
-        # 216 binary64 instructions per cell-update (ncu: 121 DADD + 64 DFMA + 31 DMUL); the ALU
-        # ceiling is the DFMA issue rate measured above (each binary64 instruction, add, mul or
-        # fma, issues at the same rate)
-        instr_rate = FP64_INSTR_PER_CELL * nn * nn / (ms64 * 1e-3)
+    def fp64_line(nn, ms64, delta):
+        # the ALU ceiling is the DFMA issue rate measured above (each binary64 instruction, add, mul
+        # or fma, issues at the same rate)
+        instr_rate = FP64_INSTR_PER_CELL["filtered" if delta else "plain"] * nn * nn / (ms64 * 1e-3)
         return {"mlups": round(nn * nn / ms64 / 1e3, 2), "ms_per_step": round(ms64, 5),
                 "hbm_frac": round(BYTES_PER_CELL["fp64"] * nn * nn / (ms64 * 1e-3) / 1e9 / peaks()[0], 4),
                 "roofline": {"bound": "alu", "achieved": round(instr_rate / 1e9, 1),
@@ -461,7 +462,7 @@ def side_measurements(n, a):
         return {"mlups": round(nn * nn / ms / 1e3, 2), "ms_per_step": round(ms, 5),
                 "hbm_frac": round(BYTES_PER_CELL[prec] * nn * nn / (ms * 1e-3) / 1e9 / peaks()[0], 4)}
 
-    res["fp64_step"] = fp64_line(n, rate(make_sim(n, "fp64", a.delta)[0], 100))
+    res["fp64_step"] = fp64_line(n, rate(make_sim(n, "fp64", a.delta)[0], 100), a.delta)
     res["fp16_step"] = hbm_line(n, rate(make_sim(n, "fp16", a.delta)[0], 1000), "fp16")
     # binary16 relative to the local velocity: 29 planes (116 B per cell update)
     res["fp16rel_step"] = hbm_line(n, rate(make_sim(n, "fp16rel", a.delta)[0], 1000), "fp16rel")
@@ -472,7 +473,7 @@ def side_measurements(n, a):
         "fp16": hbm_line(n3, rate(make_sim(n3, "fp16", 2.0, nu=nu3, delta_frac=1 / 64)[0], 600), "fp16"),
         "fp16rel": hbm_line(n3, rate(make_sim(n3, "fp16rel", 2.0, nu=nu3, delta_frac=1 / 64)[0], 500),
                             "fp16rel"),
-        "fp64": fp64_line(n3, rate(make_sim(n3, "fp64", 2.0, nu=nu3, delta_frac=1 / 64)[0], 30))}
+        "fp64": fp64_line(n3, rate(make_sim(n3, "fp64", 2.0, nu=nu3, delta_frac=1 / 64)[0], 30), 2.0)}
     msl = rate(make_sim(n, "fp32", 2.0)[0], 1000)
     res["fp32_les_delta2"] = {"mlups": round(n * n / msl / 1e3, 2)}
     msi = rate(make_sim(n, "fp32", 2.0, stencil=1)[0], 1000)

@@ -326,7 +326,7 @@ int lbmhd_diagnostics_fields_noalloc(const double* rho, const double* ux, const 
                                      double* out, void* stream);
 
 /* Measured binary64 FMA rate of the current device, the arithmetic ceiling of the LBMHD_FP64
- * step (about 173 binary64 instructions per cell update; the paper states no precision or
+ * step (140 to 171 binary64 instructions per cell update; the paper states no precision or
  * hardware, so this is a property of the GPU that runs it, not of the method).  Three shapes --
  * 4, 8 and 16 independent chains x <- x a + b per thread, (SMs x 16, 8, 4) blocks of 256
  * threads, `iters` iterations -- each one warm-up launch and `repeats` timed launches;

@@ -1,5 +1,5 @@
 // Measured binary64 fused multiply-add rate of the current GPU: the ceiling that bounds the
-// binary64 form of the fused step, which issues about 216 binary64 instructions per cell update
+// binary64 form of the step, which issues 140 to 171 binary64 instructions per cell update
 // and so reaches the arithmetic limit long before the memory one.  GB300 lists no binary64
 // figure to divide by, and its binary64 rate is a small fraction of its binary32 one, so the
 // library measures it: every thread of a few resident waves runs eight independent chains

@@ -178,7 +178,7 @@ __device__ __forceinline__ void collide(T p[kQ], T rho1, T jx, T jy, T bx, T by,
 
 // ---- binary64 collision ---------------------------------------------------------------------------
 // The binary64 step is bound by GB300's binary64 rate (528 G instructions/s, every kind alike), so
-// it is written for few instructions: 173 per cell of an LES step against 216 for the form that
+// it is written for few instructions: 171 per cell of an LES step against 216 for the form that
 // `collide` spells out, the same algebra otherwise.
 //  - Moments and non-equilibrium parts share their sums: the sums and differences of opposite
 //    populations that give rho and J (moments64) are kept until the cell is collided, and
@@ -1146,7 +1146,7 @@ __device__ __forceinline__ bool run_tile_pair(const CUtensorMap* srcp, __half* _
 // staged from its moments to its collision).  The state is bitwise that of the LES form with k = 0
 // (zero gradients go through the same operations, so the compiler contracts them alike).
 // us per step against the LES form: binary64 64^2 14.7 -> 6.3, 512^2 127 -> 81, 2048^2 1811 -> 1159
-// (140 instead of 173 binary64 instructions per cell); binary32 128^2 2.76 -> 1.86, 512^2 9.7 -> 6.6,
+// (140 instead of 171 binary64 instructions per cell); binary32 128^2 2.76 -> 1.86, 512^2 9.7 -> 6.6,
 // 1024^2 36.4 -> 34.6; binary16 512^2 9.3 -> 5.7, 1024^2 22.5 -> 19.2, its relative form 256^2 5.4 -> 3.3.
 // Larger grids of the memory-bound forms lose (plain_step_pays).
 // Returns false if a wait timed out (the block must stop; *err is set).
