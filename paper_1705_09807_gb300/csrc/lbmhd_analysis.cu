@@ -19,8 +19,9 @@
 // one the columns and adds up the shells, so the n x n spectrum is never stored.  Every n <= 4096
 // takes O(n^2 log n): radices 8, 4, 2, 3, 5, 7, 11, 13 when they factor n, Bluestein's chirp
 // convolution of power-of-two length >= 2n - 1 otherwise.  Four fields at n = 1024 took 60.1 ms with
-// direct O(n^3) sums; now rows 178 (151 of
-// them its 2.5 M binary64 warp instructions), columns and shells 210, shell totals 7 us.
+// direct O(n^3) sums, 0.40 ms with a test
+// for unit twiddles inside the last stage's loop (predicated products take binary64 time all the
+// same), now 0.38: rows 165, columns and shells 197, shell totals 7 us.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -182,10 +183,11 @@ __device__ __forceinline__ void dft(double2 (&x)[R], const double2* __restrict__
 
 // One radix-R stage over sub-blocks of ns points, in place.  Forward (decimation in frequency):
 // R-point DFT, then twiddles; natural order in, digit-reversed order out after the last stage.
-// Inverse undoes it: conjugate twiddles, then the conjugate DFT.
-template <int R, bool INVERSE>
-__device__ __forceinline__ void fft_stage(double2* buf, int lines, int len, int ns, const double2* __restrict__ tw) {
-  const int m = ns / R, per_line = len / R, tstep = len / ns;
+// Inverse undoes it: conjugate twiddles, then the conjugate DFT.  UNIT: ns = R, all twiddles one (a
+// test of m in the loop would be predicated, and the products take binary64 pipe time all the same).
+template <int R, bool INVERSE, bool UNIT>
+__device__ __forceinline__ void fft_stage_of(double2* buf, int lines, int len, int ns, const double2* __restrict__ tw) {
+  const int m = UNIT ? 1 : ns / R, per_line = len / R, tstep = len / ns;
   for (int q = threadIdx.x; q < lines * per_line; q += blockDim.x) {
     const int line = q / per_line, r = q - line * per_line;
     const int blk = r / m, j = r - blk * m;
@@ -196,7 +198,7 @@ __device__ __forceinline__ void fft_stage(double2* buf, int lines, int len, int 
     if constexpr (INVERSE) {
 #pragma unroll
       for (int k = 0; k < R; ++k) {
-        if (k > 0 && m > 1) {
+        if (k > 0 && !UNIT) {
           const double2 w = tw[j * k * tstep];
           x[k] = cmul(x[k], make_double2(w.x, -w.y));
         }
@@ -209,12 +211,18 @@ __device__ __forceinline__ void fft_stage(double2* buf, int lines, int len, int 
       dft<R>(x, tw, len);
 #pragma unroll
       for (int k = 0; k < R; ++k) {
-        if (k > 0 && m > 1) x[k] = cmul(x[k], tw[j * k * tstep]);
+        if (k > 0 && !UNIT) x[k] = cmul(x[k], tw[j * k * tstep]);
         a[k * m] = x[k];
       }
     }
   }
   __syncthreads();
+}
+
+template <int R, bool INVERSE>
+__device__ __forceinline__ void fft_stage(double2* buf, int lines, int len, int ns, const double2* __restrict__ tw) {
+  if (ns == R) fft_stage_of<R, INVERSE, true>(buf, lines, len, ns, tw);
+  else fft_stage_of<R, INVERSE, false>(buf, lines, len, ns, tw);
 }
 
 // Forward transform of the block's lines (buf[line * len + j], complete before the call).
@@ -440,9 +448,18 @@ __global__ void __launch_bounds__(32 * kTotalShells)
 FftPlan make_plan(int n) {
   FftPlan p{};
   p.n = p.len = n;
+  // Radix 8 first, so that what is left over comes last, without twiddles -- but a radix 2, whose
+  // stage has the fewest, comes first: spectra of 1024^2 fields 387 -> 378 us (2048^2 with its radix 4
+  // first 1447 -> 1457, so that stays behind).
   static const int radices[] = {8, 4, 2, 3, 5, 7, 11, 13};
   auto factor = [&](int v) {
     p.nrad = 0;
+    int twos = 0;
+    while (v >> twos > 0 && (v >> twos) % 2 == 0) ++twos;
+    if (twos % 3 == 1) {
+      p.rad[p.nrad++] = 2;
+      v /= 2;
+    }
     for (int r : radices)
       while (v % r == 0) {
         p.rad[p.nrad++] = (unsigned char)r;
