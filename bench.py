@@ -334,7 +334,7 @@ def oracle_step_times(side, steps, warmup, cores, delta=0.0, min_s=0.0):
 
 def cpu_oracle_rates(n, cores):
     """Oracle MLUPS on the host cores, median of 5 samples, on 64^2, 256^2, 1024^2 and the
-    workload's own n^2 grid (the grid the reference arm times at the driver's step counts)."""
+    workload's own n^2 grid (the grid the reference arm times at the bench's step counts)."""
     grids = {}
     t_all = time.perf_counter()
     for side in sorted({64, 256, 1024, n}):
