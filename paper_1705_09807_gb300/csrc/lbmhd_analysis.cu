@@ -19,9 +19,9 @@
 // one the columns and adds up the shells, so the n x n spectrum is never stored.  Every n <= 4096
 // takes O(n^2 log n): radices 8, 4, 2, 3, 5, 7, 11, 13 when they factor n, Bluestein's chirp
 // convolution of power-of-two length >= 2n - 1 otherwise.  Four fields at n = 1024 took 60.1 ms with
-// direct O(n^3) sums, 0.40 ms with a test
-// for unit twiddles inside the last stage's loop (predicated products take binary64 time all the
-// same), now 0.38: rows 165, columns and shells 197, shell totals 7 us.
+// direct O(n^3) sums, 0.40 ms with tests
+// for unit twiddles and for Bluestein around single products (predicated, these take binary64 time
+// all the same), now 0.35: rows 147, columns and shells 186, shell totals 7 us.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -270,9 +270,10 @@ __device__ __forceinline__ int digit_reversed(const FftPlan& p, int k) {
 
 // DFT of the block's lines; buf[line * len + j] holds point j (times chirp[j] for Bluestein, zero
 // from n on), complete before the call.  Afterwards fft_result reads the outputs.
+template <bool CHIRP>
 __device__ __forceinline__ void transform_lines(double2* buf, const FftPlan& p, const FftTables& t) {
   fft_forward(buf, p, t.tw);
-  if (p.chirp()) {
+  if constexpr (CHIRP) {
     for (int q = threadIdx.x; q < p.lines * p.len; q += blockDim.x) buf[q] = cmul(buf[q], t.filter[q % p.len]);
     __syncthreads();
     fft_inverse_pow2(buf, p, t.tw);
@@ -281,10 +282,11 @@ __device__ __forceinline__ void transform_lines(double2* buf, const FftPlan& p, 
 
 // Output k of a transformed line up to a unit factor (Bluestein leaves out the last chirp
 // product): exact for |X_k|, which is all that the columns need; `full` puts it in (the rows).
+template <bool CHIRP>
 __device__ __forceinline__ double2 fft_result(const double2* line, const FftPlan& p, const FftTables& t, int k,
                                               bool full) {
-  if (!p.chirp()) return line[digit_reversed(p, k)];
-  return full ? cmul(line[k], t.chirp[k]) : line[k];
+  if constexpr (!CHIRP) return line[digit_reversed(p, k)];
+  else return full ? cmul(line[k], t.chirp[k]) : line[k];
 }
 
 __global__ void fft_tables_kernel(FftPlan p, FftTables t) {
@@ -319,7 +321,9 @@ __global__ void fft_filter_kernel(FftPlan p, FftTables t) {
     t.filter[j] = make_double2(inv * fft_buf[j].x, inv * fft_buf[j].y);
 }
 
-// G[pair][y][kx]: row transforms of u_x + i u_y (pair 0) and B_x + i B_y (pair 1).
+// G[pair][y][kx]: row transforms of u_x + i u_y (pair 0) and B_x + i B_y (pair 1).  CHIRP: Bluestein
+// (compiled apart: its products, predicated off, would take an eighth of the binary64 issue).
+template <bool CHIRP>
 __global__ void __launch_bounds__(256)
     fft_rows_kernel(const double* __restrict__ ux, const double* __restrict__ uy, const double* __restrict__ bx,
                     const double* __restrict__ by, FftPlan p, FftTables t, double2* __restrict__ G) {
@@ -334,16 +338,16 @@ __global__ void __launch_bounds__(256)
     if (j < n) {
       const size_t c = (size_t)(y0 + line) * n + j;
       v = make_double2(re[c], im[c]);
-      if (p.chirp()) v = cmul(v, t.chirp[j]);
+      if constexpr (CHIRP) v = cmul(v, t.chirp[j]);
     }
     fft_buf[q] = v;
   }
   __syncthreads();
-  transform_lines(fft_buf, p, t);
+  transform_lines<CHIRP>(fft_buf, p, t);
   double2* g = G + (size_t)blockIdx.y * n * n + (size_t)y0 * n;
   for (int q = threadIdx.x; q < p.lines * n; q += blockDim.x) {
     const int line = q / n, k = q - line * n;
-    g[q] = fft_result(fft_buf + (size_t)line * p.len, p, t, k, true);
+    g[q] = fft_result<CHIRP>(fft_buf + (size_t)line * p.len, p, t, k, true);
   }
 }
 
@@ -358,6 +362,7 @@ __device__ __forceinline__ int half_isqrt(int v) {
 // Column transforms of pair blockIdx.y and the shell sums of this block's columns:
 // part[pair][column group][s] = sum over the group's columns kx and the ky of shell s of
 // |Z(kx, ky)|^2.  In one column a shell is two runs of consecutive ky, which one thread adds.
+template <bool CHIRP>
 __global__ void __launch_bounds__(256)
     fft_cols_kernel(const double2* __restrict__ G, FftPlan p, FftTables t, int nbins, double* __restrict__ part) {
   extern __shared__ double2 fft_buf[];
@@ -384,18 +389,18 @@ __global__ void __launch_bounds__(256)
     double2 v = make_double2(0.0, 0.0);
     if (j < n) {
       v = g[(size_t)j * n + x0 + line];
-      if (p.chirp()) v = cmul(v, t.chirp[j]);
+      if constexpr (CHIRP) v = cmul(v, t.chirp[j]);
     }
     fft_buf[line * len + j] = v;
   }
   __syncthreads();
-  transform_lines(fft_buf, p, t);
+  transform_lines<CHIRP>(fft_buf, p, t);
   // |Z|^2 in natural order first: the runs below are then consecutive (a thread that added up to 45
   // digit-reversed cells of its run held its block up)
   double* power = reinterpret_cast<double*>(fft_buf + (size_t)lines * len);  // [lines][n]
   for (int q = threadIdx.x; q < lines * n; q += blockDim.x) {
     const int c = q / n, k = q - c * n;
-    const double2 z = fft_result(fft_buf + (size_t)c * len, p, t, k, false);
+    const double2 z = fft_result<CHIRP>(fft_buf + (size_t)c * len, p, t, k, false);
     power[q] = z.x * z.x + z.y * z.y;
   }
   __syncthreads();
@@ -502,19 +507,21 @@ cudaError_t launch_energy_spectrum(const double* ux, const double* uy, const dou
   double* part = reinterpret_cast<double*>(G + 2 * nn);
   const size_t smem = (size_t)p.lines * p.len * sizeof(double2);
   const size_t smem_cols = smem + (size_t)p.lines * n * sizeof(double);  // and the power of the lines
+  const auto rows = p.chirp() ? fft_rows_kernel<true> : fft_rows_kernel<false>;
+  const auto cols = p.chirp() ? fft_cols_kernel<true> : fft_cols_kernel<false>;
   cudaError_t e = cudaSuccess;
   if (smem_cols > 48 * 1024) {
     const int b = (int)smem, bc = (int)smem_cols;
-    e = cudaFuncSetAttribute(fft_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fft_cols_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bc);
+    e = cudaFuncSetAttribute(rows, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(cols, cudaFuncAttributeMaxDynamicSharedMemorySize, bc);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fft_filter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
     if (e != cudaSuccess) return e;
   }
   const int groups = (n + p.lines - 1) / p.lines;
   fft_tables_kernel<<<(p.len + n + 127) / 128, 128, 0, s>>>(p, t);
   if (p.chirp()) fft_filter_kernel<<<1, 256, p.len * sizeof(double2), s>>>(p, t);
-  fft_rows_kernel<<<dim3(groups, 2), p.threads, smem, s>>>(ux, uy, bx, by, p, t, G);
-  fft_cols_kernel<<<dim3(groups, 2), p.threads, smem_cols, s>>>(G, p, t, nbins, part);
+  rows<<<dim3(groups, 2), p.threads, smem, s>>>(ux, uy, bx, by, p, t, G);
+  cols<<<dim3(groups, 2), p.threads, smem_cols, s>>>(G, p, t, nbins, part);
   shell_total_kernel<<<dim3((nbins + kTotalShells - 1) / kTotalShells, 2), dim3(kTotalShells, 32), 0, s>>>(part, groups, nbins,
                                                                        0.5 / ((double)nn * (double)nn), ek, em);
   return cudaGetLastError();
