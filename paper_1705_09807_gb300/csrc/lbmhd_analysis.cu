@@ -447,6 +447,11 @@ __global__ void __launch_bounds__(32 * kTotalShells)
   }
 }
 
+// Shared memory of a block, at most: one line of 8192 points (Bluestein, n > 2048), and in the columns
+// its n <= 4096 squared magnitudes.
+constexpr int kMaxRowBytes = 8192 * (int)sizeof(double2);
+constexpr int kMaxColBytes = kMaxRowBytes + 4096 * (int)sizeof(double);
+
 // Lines per block: up to 32 KB of points (binary64 work hides everything else, so small blocks
 // that fill the last wave evenly are worth more than reuse), 256 threads when a radix-8 stage
 // has that many butterflies.
@@ -509,12 +514,13 @@ cudaError_t launch_energy_spectrum(const double* ux, const double* uy, const dou
   const size_t smem_cols = smem + (size_t)p.lines * n * sizeof(double);  // and the power of the lines
   const auto rows = p.chirp() ? fft_rows_kernel<true> : fft_rows_kernel<false>;
   const auto cols = p.chirp() ? fft_cols_kernel<true> : fft_cols_kernel<false>;
-  cudaError_t e = cudaSuccess;
   if (smem_cols > 48 * 1024) {
-    const int b = (int)smem, bc = (int)smem_cols;
-    e = cudaFuncSetAttribute(rows, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(cols, cudaFuncAttributeMaxDynamicSharedMemorySize, bc);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fft_filter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+    // The limit belongs to the kernel, not to this call: every call sets the same value, the largest
+    // that any n needs, so that threads with spectra of different sizes never lower it for one another.
+    const auto limit = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    cudaError_t e = cudaFuncSetAttribute(rows, limit, kMaxRowBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(cols, limit, kMaxColBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fft_filter_kernel, limit, kMaxRowBytes);
     if (e != cudaSuccess) return e;
   }
   const int groups = (n + p.lines - 1) / p.lines;
