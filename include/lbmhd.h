@@ -346,7 +346,8 @@ const char* lbmhd_last_error(const lbmhd_t* h);
  * lbmhd_release_cached_memory. */
 void lbmhd_free(lbmhd_t* h);
 
-/* Return the device memory kept from freed handles to the device. */
+/* Return the device memory kept from freed handles to the devices it came from.  May be called from
+ * any thread, also one that has made no CUDA call; the thread's current device and context stay. */
 void lbmhd_release_cached_memory(void);
 
 #ifdef __cplusplus

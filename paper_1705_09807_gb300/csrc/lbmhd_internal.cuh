@@ -25,6 +25,7 @@
 #include <cuda_fp16.h>
 
 #include "lbmhd.h"
+#include "lbmhd_memory.h"
 #include <cuda_runtime.h>
 #include <stddef.h>
 #include <stdint.h>
@@ -184,15 +185,6 @@ const float* closure_device_params(const lbmhd_closure_t* c);
 const float* closure_device_scales(const lbmhd_closure_t* c);
 const unsigned char* closure_device_packed(const lbmhd_closure_t* c);
 cudaStream_t closure_stream(const lbmhd_closure_t* c);
-
-// Device memory of handles (lbmhd_memory.cu).  device_free keeps a block for later device_alloc calls
-// of the same size if `idle`, i.e. if no work on it can be in flight any more.
-cudaError_t device_alloc(void** out, size_t bytes);
-void device_free(void* ptr, bool idle);
-
-// Identifier of the calling thread's current context, unique for the life of the process; false if
-// it cannot be had (lbmhd_noalloc.cu).
-bool current_context_id(unsigned long long* id);
 
 // Store a message for lbmhd_last_error(NULL) on the calling thread (lbmhd_api.cu).
 void set_thread_error(const char* msg);

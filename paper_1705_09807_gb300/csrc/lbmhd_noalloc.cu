@@ -42,32 +42,27 @@ int set_error(int code, const char* msg) {
   return code;
 }
 
-// Driver calls that identify the current context, reached through the runtime's driver entry
-// point (the library does not link libcuda).  cuCtxGetId gives a context an identifier that is
-// unique for the life of the process, so a context that was destroyed and re-created (for
-// example after cudaDeviceReset) is told apart from its predecessor even if its handle value is
-// reused.
-using CtxGetCurrentFn = CUresult (*)(CUcontext*);
-using CtxGetIdFn = CUresult (*)(CUcontext, unsigned long long*);
+}  // namespace
 
-template <typename F>
-F driver_fn(const char* name, int version) {
+void* lbmhd_gpu::driver_entry(const char* name, int version) {
   void* f = nullptr;
   cudaDriverEntryPointQueryResult q;
   if (cudaGetDriverEntryPointByVersion(name, &f, version, cudaEnableDefault, &q) != cudaSuccess ||
       q != cudaDriverEntryPointSuccess)
     return nullptr;
-  return reinterpret_cast<F>(f);
+  return f;
 }
-
-}  // namespace
 
 // Identifier of the calling thread's current context; false if it cannot be had (no current
 // context yet, or a driver without cuCtxGetId), in which case the caller looks the address up
-// afresh.
+// afresh.  cuCtxGetId gives a context an identifier that is unique for the life of the process, so
+// a context that was destroyed and re-created (for example after cudaDeviceReset) is told apart
+// from its predecessor even if its handle value is reused.
 bool lbmhd_gpu::current_context_id(unsigned long long* id) {
-  static const CtxGetCurrentFn get_current = driver_fn<CtxGetCurrentFn>("cuCtxGetCurrent", 4000);
-  static const CtxGetIdFn get_id = driver_fn<CtxGetIdFn>("cuCtxGetId", 12000);
+  using CtxGetCurrentFn = CUresult (*)(CUcontext*);
+  using CtxGetIdFn = CUresult (*)(CUcontext, unsigned long long*);
+  static const auto get_current = reinterpret_cast<CtxGetCurrentFn>(driver_entry("cuCtxGetCurrent", 4000));
+  static const auto get_id = reinterpret_cast<CtxGetIdFn>(driver_entry("cuCtxGetId", 12000));
   if (!get_current || !get_id) return false;
   CUcontext ctx = nullptr;
   if (get_current(&ctx) != CUDA_SUCCESS || !ctx) return false;
