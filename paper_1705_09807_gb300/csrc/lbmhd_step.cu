@@ -917,12 +917,16 @@ __device__ __forceinline__ void store_cell_pair(__half* __restrict__ dst, const 
       }
     }
   }
+  // ghosts: columns 0, 1 at nx, nx + 1 and nx - 2, nx - 1 at -2, -1 (on a grid of three columns the
+  // middle one has both)
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const int xh = x + h;
     if (h == 1 && !both) break;
-    if (xh < 2 || xh >= g.nx - 2) {  // ghosts: logical nx, nx + 1 and -2, -1
-      __half* gp = o + h + (xh < 2 ? g.nx : -g.nx);
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+      if (side == 0 ? xh >= 2 : xh < g.nx - 2) continue;
+      __half* gp = o + h + (side == 0 ? g.nx : -g.nx);
 #pragma unroll
       for (int q = 0; q < kQ; ++q) {
         __half* a = gp + (size_t)plane_of(q) * g.plane;
