@@ -342,7 +342,7 @@ const char* lbmhd_last_error(const lbmhd_t* h);
 
 /* Release the handle and its device memory (waits for its stream).  NULL is a no-op.  The library
  * keeps up to 1 GiB of device memory of freed handles for later ones (of the same grid size and
- * precision); it is returned to the device when an allocation of the library fails, or by
+ * precision); it is returned to the device when an allocation of the library finds no memory there, or by
  * lbmhd_release_cached_memory. */
 void lbmhd_free(lbmhd_t* h);
 

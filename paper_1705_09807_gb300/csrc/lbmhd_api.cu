@@ -561,7 +561,7 @@ int lbmhd_get_populations(lbmhd_t* h, double* pops) {
   if (!pops) return fail(h, LBMHD_ERR_INVALID, "pops is NULL");
   const size_t n = (size_t)kQ * h->p.nx * h->p.ny;
   double* tmp = nullptr;
-  LB_CUDA(h, cudaMallocAsync((void**)&tmp, n * sizeof(double), h->stream));
+  LB_CUDA(h, device_malloc_async((void**)&tmp, n * sizeof(double), h->stream));
   cudaError_t e = launch_populations(h->precision, h->pops[h->cur], h->geom, tmp, h->stream);
   if (e == cudaSuccess) {
     h->launches += 1;

@@ -1184,10 +1184,10 @@ int ensure_scratch(lbmhd_closure_t* c, size_t cells) {
   for (int i = 0; i < 5; ++i) {
     if (*bufs[i]) cudaFree(*bufs[i]);
     *bufs[i] = nullptr;
-    CL_CUDA(c, cudaMalloc(bufs[i], cells * ch[i] * sizeof(float)));
+    CL_CUDA(c, device_malloc(bufs[i], cells * ch[i] * sizeof(float)));
   }
-  if (!c->wpart) CL_CUDA(c, cudaMalloc(&c->wpart, (size_t)kMaxConvBlocks * kNumParams * sizeof(float)));
-  if (!c->lpart) CL_CUDA(c, cudaMalloc(&c->lpart, (kMaxConvBlocks + 1) * sizeof(double)));
+  if (!c->wpart) CL_CUDA(c, device_malloc(&c->wpart, (size_t)kMaxConvBlocks * kNumParams * sizeof(float)));
+  if (!c->lpart) CL_CUDA(c, device_malloc(&c->lpart, (kMaxConvBlocks + 1) * sizeof(double)));
   c->cap_cells = cells;
   return LBMHD_OK;
 }
@@ -1296,13 +1296,13 @@ int lbmhd_closure_create(lbmhd_closure_t** out, const float* params, const float
   std::memcpy(c->host_scales + 12, out_scale, 4 * sizeof(float));
   cudaError_t e = cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking);
   const size_t pb = kNumParams * sizeof(float);
-  if (e == cudaSuccess) e = cudaMalloc(&c->params, pb);
-  if (e == cudaSuccess) e = cudaMalloc(&c->grad, pb);
-  if (e == cudaSuccess) e = cudaMalloc(&c->adam_m, pb);
-  if (e == cudaSuccess) e = cudaMalloc(&c->adam_v, pb);
-  if (e == cudaSuccess) e = cudaMalloc(&c->scales, 16 * sizeof(float));
-  if (e == cudaSuccess) e = cudaMalloc(&c->packed, kPackedBytes);
-  if (e == cudaSuccess) e = cudaMalloc(&c->tc_err, sizeof(unsigned));
+  if (e == cudaSuccess) e = device_malloc(&c->params, pb);
+  if (e == cudaSuccess) e = device_malloc(&c->grad, pb);
+  if (e == cudaSuccess) e = device_malloc(&c->adam_m, pb);
+  if (e == cudaSuccess) e = device_malloc(&c->adam_v, pb);
+  if (e == cudaSuccess) e = device_malloc(&c->scales, 16 * sizeof(float));
+  if (e == cudaSuccess) e = device_malloc(&c->packed, kPackedBytes);
+  if (e == cudaSuccess) e = device_malloc(&c->tc_err, sizeof(unsigned));
   if (e == cudaSuccess) e = cudaMemset(c->tc_err, 0, sizeof(unsigned));
   if (e == cudaSuccess) e = cudaMemcpy(c->params, params, pb, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemset(c->adam_m, 0, pb);

@@ -129,12 +129,12 @@ int build_work(lbmhd_ensemble_t* e, int rows_per_tile, int persistent) {
   void* aligned = host.data() + ((64 - (reinterpret_cast<uintptr_t>(host.data()) & 63)) & 63);
   pack_ensemble_members(e->precision, e->n, maps.data(), pops.data(), geoms.data(), coefs.data(),
                         aligned);
-  if (!e->d_members) ENS_CUDA(e, cudaMalloc(&e->d_members, mbytes));
+  if (!e->d_members) ENS_CUDA(e, device_malloc(&e->d_members, mbytes));
   ENS_CUDA(e, cudaMemcpyAsync(e->d_members, aligned, mbytes, cudaMemcpyHostToDevice, e->stream));
   if ((int)work.size() > e->work_capacity) {
     if (e->d_work) ENS_CUDA(e, cudaFree(e->d_work));
     e->d_work = nullptr;
-    ENS_CUDA(e, cudaMalloc(&e->d_work, work.size() * sizeof(int4)));
+    ENS_CUDA(e, device_malloc(&e->d_work, work.size() * sizeof(int4)));
     e->work_capacity = (int)work.size();
   }
   ENS_CUDA(e, cudaMemcpyAsync(e->d_work, work.data(), work.size() * sizeof(int4),
@@ -261,8 +261,8 @@ int lbmhd_ensemble_create(lbmhd_ensemble_t** out, int n, const lbmhd_params* par
     e->members.push_back(h);
   }
   int rc = LBMHD_OK;
-  if ((ce = cudaMalloc(&e->d_queue, sizeof(unsigned long long))) != cudaSuccess ||
-      (ce = cudaMalloc(&e->d_err, sizeof(unsigned))) != cudaSuccess ||
+  if ((ce = device_malloc(&e->d_queue, sizeof(unsigned long long))) != cudaSuccess ||
+      (ce = device_malloc(&e->d_err, sizeof(unsigned))) != cudaSuccess ||
       (ce = cudaMemsetAsync(e->d_err, 0, sizeof(unsigned), e->stream)) != cudaSuccess)
     rc = efail(nullptr, LBMHD_ERR_CUDA, "ensemble buffers: %s", cudaGetErrorString(ce));
   if (!rc) rc = build_work(e, 0, 0);
@@ -305,7 +305,7 @@ int lbmhd_ensemble_autotune(lbmhd_ensemble_t* e, int trial_steps, double* best_m
   int rc = LBMHD_OK;
   for (int i = 0; i < e->n && !rc; ++i) {
     lbmhd_t* m = e->members[i];
-    cudaError_t ce = cudaMallocAsync(&backup[i], m->state_bytes, e->stream);
+    cudaError_t ce = device_malloc_async(&backup[i], m->state_bytes, e->stream);
     if (ce == cudaSuccess)
       ce = cudaMemcpyAsync(backup[i], m->pops[m->cur], m->state_bytes, cudaMemcpyDeviceToDevice, e->stream);
     if (ce != cudaSuccess) rc = efail(e, LBMHD_ERR_CUDA, "autotune backup: %s", cudaGetErrorString(ce));

@@ -10,7 +10,7 @@
 // synchronised the stream that used it), only in the context it was allocated in, so it can be
 // handed to any stream, and only if that is its device's primary context (the runtime's own).  The
 // cache holds at most kMaxCached bytes (the oldest blocks go first), gives a device's blocks back when
-// an allocation there fails, and all blocks by lbmhd_release_cached_memory.  Blocks are matched by
+// an allocation of the library there finds no memory, and all blocks by lbmhd_release_cached_memory.  Blocks are matched by
 // exact size; their contents are not cleared (nor are cudaMalloc's).  A block is freed in its own
 // context, whatever the calling thread has current -- another device, another context, or none
 // yet -- and its record is dropped without that only if its context is known to be gone: a
@@ -130,7 +130,32 @@ void shrink(size_t most, int only) {
   }
 }
 
+// alloc(), once more if it found no memory and blocks of this device could be given back (under the
+// mutex).
+template <typename F>
+cudaError_t retried(F alloc) {
+  const cudaError_t e = alloc();
+  if (e != cudaErrorMemoryAllocation) return e;
+  int device = 0;
+  unsigned long long context = 0;
+  const size_t kept = g_cached_bytes;
+  if (kept > 0 && here(&device, &context)) shrink(0, device);
+  if (g_cached_bytes == kept) return e;
+  cudaGetLastError();
+  return alloc();
+}
+
 }  // namespace
+
+cudaError_t device_malloc(void** out, size_t bytes) {
+  std::lock_guard<std::mutex> lock(g_mutex);
+  return retried([&] { return cudaMalloc(out, bytes); });
+}
+
+cudaError_t device_malloc_async(void** out, size_t bytes, cudaStream_t s) {
+  std::lock_guard<std::mutex> lock(g_mutex);
+  return retried([&] { return cudaMallocAsync(out, bytes, s); });
+}
 
 cudaError_t device_alloc(void** out, size_t bytes) {
   *out = nullptr;
@@ -149,12 +174,7 @@ cudaError_t device_alloc(void** out, size_t bytes) {
         return cudaSuccess;
       }
     }
-    cudaError_t e = cudaMalloc(out, bytes);
-    if (e == cudaErrorMemoryAllocation && known && g_cached_bytes > 0) {
-      cudaGetLastError();
-      shrink(0, device);
-      e = cudaMalloc(out, bytes);
-    }
+    const cudaError_t e = retried([&] { return cudaMalloc(out, bytes); });
     if (e != cudaSuccess) {
       *out = nullptr;
       return e;

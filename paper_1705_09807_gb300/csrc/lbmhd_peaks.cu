@@ -68,7 +68,7 @@ extern "C" int lbmhd_probe_fp64_fma_rate(int iters, int repeats, double* dfma_pe
   double* sink = nullptr;
   cudaStream_t st = nullptr;
   cudaEvent_t t0 = nullptr, t1 = nullptr;
-  e = cudaMalloc(&sink, sizeof(double) * max_blocks);
+  e = lbmhd_gpu::device_malloc(&sink, sizeof(double) * max_blocks);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreate(&t0);
   if (e == cudaSuccess) e = cudaEventCreate(&t1);

@@ -53,6 +53,7 @@ cudaError_t cudaMalloc(void** p, size_t n) {
   mem[*p] = Mem{n, cur->device, cur->id};
   return cudaSuccess;
 }
+cudaError_t cudaMallocAsync(void** p, size_t n, cudaStream_t) { return cudaMalloc(p, n); }
 cudaError_t cudaFree(void* p) {
   if (!p) return cudaSuccess;
   bind();
@@ -155,6 +156,22 @@ CASES = {
   device_free(p, false);
   CHECK(used(0) == 0);
 """,
+    # the library's other allocations get them as well, those of their own device
+    "out_of_memory_elsewhere": r"""
+  capacity[0] = capacity[1] = 1000 * MiB;
+  for (int async = 0; async < 2; ++async) {
+    keep(600 * MiB);
+    cudaSetDevice(1);
+    keep(100 * MiB);
+    cudaSetDevice(0);
+    void* p = nullptr;
+    CHECK((async ? device_malloc_async(&p, 700 * MiB, nullptr) : device_malloc(&p, 700 * MiB)) == cudaSuccess);
+    CHECK(used(0) == 700 * MiB && used(1) == 100 * MiB);
+    cudaFree(p);
+  }
+  void* q = nullptr;
+  CHECK(device_malloc(&q, 1100 * MiB) == cudaErrorMemoryAllocation);
+""",
 }
 
 
@@ -179,3 +196,13 @@ def test_memory_of_freed_handles(case, tmp_path, include_dir):
     assert r.returncode == 0, r.stderr[-3000:]
     r = subprocess.run([exe], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout
+
+
+def test_every_allocation_can_have_the_kept_memory():
+    """No source file but lbmhd_memory.cu calls the runtime's allocation functions itself."""
+    import re
+    for f in sorted(os.listdir(CSRC)):
+        if f != "lbmhd_memory.cu" and os.path.isfile(os.path.join(CSRC, f)):
+            with open(os.path.join(CSRC, f)) as fh:
+                code = re.sub(r"//[^\n]*", "", fh.read())
+            assert not re.search(r"\bcudaMalloc(Async|Managed|Pitch)?\s*\(", code), f
