@@ -251,6 +251,7 @@ int create(lbmhd_t** out, const lbmhd_params* p) {
   h->state_bytes = (size_t)g.pitch * p->ny * h->elem;
   g.plain = plain_step_pays(p->precision, h->coef.kq, h->state_bytes) ? 1 : 0;
   g.band = step_band_rows(p->nx, p->ny, p->precision, sms, g.plain != 0);
+  h->corr_band = step_band_rows(p->nx, p->ny, p->precision, sms);
 #define LB_INIT(call)                 \
   do {                                \
     cudaError_t e_ = (call);          \
@@ -298,19 +299,26 @@ int create(lbmhd_t** out, const lbmhd_params* p) {
 // reads of a step from 471 MB to 427 MB (ncu without its L2 flush) and the time by 0.5%; the
 // binary16 form, bound by latency rather than memory, ran 0.7% slower with it and keeps a fixed
 // direction.
+//
+// A corrected step takes the general form also where the grid's own steps take the plain one, and
+// fewer of its blocks fit an SM: it has bands of its own.  On the plain form's bands its last wave
+// was nearly empty (Delta = 0 with correction planes: binary64 512^2 155 instead of 131 us, binary32
+// 1024^2 49.8 instead of 38.8).
 cudaError_t launch_one(lbmhd_t* h, int from, int to, const float* corr = nullptr) {
+  StepGeom g = h->geom;
+  if (corr) g.band = h->corr_band;
   switch (h->precision) {
     case LBMHD_FP64:
-      return launch_step_f64(h->tmap[from], (double*)h->pops[to], h->geom, h->coef,
+      return launch_step_f64(h->tmap[from], (double*)h->pops[to], g, h->coef,
                              h->p.grad_stencil, h->err_flag, corr, from, h->stream);
     case LBMHD_FP32:
-      return launch_step_f32(h->tmap[from], (float*)h->pops[to], h->geom, h->coef,
+      return launch_step_f32(h->tmap[from], (float*)h->pops[to], g, h->coef,
                              h->p.grad_stencil, h->err_flag, corr, from, h->stream);
     case LBMHD_FP16:
-      return launch_step_f16(h->tmap[from], (__half*)h->pops[to], h->geom, h->coef,
+      return launch_step_f16(h->tmap[from], (__half*)h->pops[to], g, h->coef,
                              h->p.grad_stencil, h->err_flag, corr, 0, h->stream);
     default:  // LBMHD_FP16_REL (no correction: refused when it is attached)
-      return launch_step_f16rel(h->tmap[from], h->umap[from], (__half*)h->pops[to], h->geom, h->coef,
+      return launch_step_f16rel(h->tmap[from], h->umap[from], (__half*)h->pops[to], g, h->coef,
                                 h->p.grad_stencil, h->err_flag, h->stream);
   }
 }

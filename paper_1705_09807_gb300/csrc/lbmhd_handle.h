@@ -16,6 +16,7 @@ struct lbmhd {
   int device = 0;
   lbmhd_gpu::StepGeom geom{};
   lbmhd_gpu::StepCoef coef{};
+  int corr_band = 0;       // rows per block of corrected steps (geom.band: of the others)
   size_t elem = 8;         // bytes per stored population value
   int nplanes = 27;        // planes per row: 27 populations (+ 2 velocity-reference planes for
                            // LBMHD_FP16_REL)
