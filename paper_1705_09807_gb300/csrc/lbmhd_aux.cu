@@ -194,9 +194,10 @@ struct PairSum {
 };
 
 // rho, u, B of one cell from its 27 pulled binary32 values (f as stored deviations; REL: relative
-// to w_i (1 + 3 c_i . U), with U[k] = {U_x, U_y} of the source cell of f_(k+1)).
+// to w_i (1 + 3 c_i . U), with U[k] = {U_x, U_y} of the source cell of f_(k+1)).  False if a value is
+// infinite or NaN: one of f makes rho and then u NaN (TwoSum subtracts infinities), one of g a sum.
 template <bool EXACT, bool REL>
-__device__ __forceinline__ void moments_of(const float (&v)[27], const float (&U)[8][2], double (&out)[5]) {
+__device__ __forceinline__ bool moments_of(const float (&v)[27], const float (&U)[8][2], double (&out)[5]) {
   PairSum r, px, py, qx, qy;
 #pragma unroll
   for (int i = 0; i < 9; ++i) {
@@ -244,6 +245,7 @@ __device__ __forceinline__ void moments_of(const float (&v)[27], const float (&U
   out[2] = widen(jy * ir);
   out[3] = qx.value<EXACT>();
   out[4] = qy.value<EXACT>();
+  return isfinite(jx * ir + (qx.hi + qy.hi));
 }
 
 // Macroscopic fields.  One cell per thread, rows of a block's columns; the ghost columns hold the
@@ -275,7 +277,8 @@ struct CellValues {
       }
     }
   }
-  __device__ __forceinline__ void moments(double (&out)[5]) const {
+  // (false: moments_of's, for the relative form only)
+  __device__ __forceinline__ bool moments(double (&out)[5]) const {
     if constexpr (sizeof(T) == 8) {
       // with the terms of zero c left out and one reciprocal for both velocities 46 binary64
       // instructions a cell instead of 62: 2048^2 497 -> 363 us
@@ -305,6 +308,7 @@ struct CellValues {
         out[1] = jx / out[0];
         out[2] = jy / out[0];
       }
+      return true;
     } else {
       float w[27], W[8][2] = {};
 #pragma unroll
@@ -320,14 +324,58 @@ struct CellValues {
         float a[3] = {0.f, 0.f, 0.f};
 #pragma unroll
         for (int q = 0; q < 27; ++q) a[q / 9] += fabsf(w[q]);
-        if (a[0] <= 1.f && a[1] <= 1.f && a[2] <= 1.f) moments_of<true, REL>(w, W, out);
-        else moments_of<false, REL>(w, W, out);
+        if (a[0] <= 1.f && a[1] <= 1.f && a[2] <= 1.f) return moments_of<true, REL>(w, W, out);
+        return moments_of<false, REL>(w, W, out);
       } else {
-        moments_of<false, REL>(w, W, out);
+        return moments_of<false, REL>(w, W, out);
       }
     }
   }
 };
+
+// Moments of a cell of the relative binary16 form with infinities or NaN among its values, from
+// binary64 sums: the pair sums make NaN of an infinite population, where rho is infinite.  A call, for
+// states that have diverged.
+template <typename T>
+__device__ __noinline__ void moments_diverged(const T* __restrict__ pops, int nx, int ny, int pitch, size_t plane,
+                                              int x, int y, double* out) {
+  StepGeom g{};
+  g.nx = nx;
+  g.ny = ny;
+  g.pitch = pitch;
+  g.plane = plane;
+  double v[27], r = 0, jx = 0, jy = 0, sbx = 0, sby = 0;
+  pull_cell<T, true>(pops, g, x, y, v);
+#pragma unroll
+  for (int i = 0; i < 9; ++i) {
+    r += v[i];
+    jx += vx(i) * v[i];
+    jy += vy(i) * v[i];
+    sbx += v[9 + i];
+    sby += v[18 + i];
+  }
+  out[0] = 1.0 + r;
+  const float ir = 1.f / (float)out[0];
+  out[1] = (double)((float)jx * ir);
+  out[2] = (double)((float)jy * ir);
+  out[3] = sbx;
+  out[4] = sby;
+}
+
+// out <- moments of cell (x, y), whose values are loaded.
+template <typename T, bool REL>
+__device__ __forceinline__ void cell_moments(const CellValues<T, REL>& cell, const T* __restrict__ pops,
+                                             const StepGeom& g, int x, int y, double (&out)[5]) {
+  const bool finite = cell.moments(out);
+  if constexpr (REL) {
+    if (!finite) {
+      double d[5];
+      moments_diverged(pops, g.nx, g.ny, g.pitch, g.plane, x, y, d);
+#pragma unroll
+      for (int k = 0; k < 5; ++k) out[k] = d[k];
+    }
+  }
+}
 
 template <typename T, bool REL = false>
 __global__ void __launch_bounds__(128)
@@ -340,7 +388,7 @@ __global__ void __launch_bounds__(128)
     double out[5];
     CellValues<T, REL> cell;
     cell.load(pops, g, x, y);
-    cell.moments(out);
+    cell_moments(cell, pops, g, x, y, out);
     rho[c] = out[0];
     ux[c] = out[1];
     uy[c] = out[2];
@@ -406,7 +454,7 @@ __global__ void __launch_bounds__(kDiagThreads, 4)
       }
       if (tid < cols) {
         if (!kAhead) cell.load(pops, g, x0 + tid, wrapi(y, ny));
-        cell.moments(m);
+        cell_moments(cell, pops, g, x0 + tid, wrapi(y, ny), m);
         if (kAhead && y < y1) cell.load(pops, g, x0 + tid, wrapi(y + 1, ny));
         sb[par][0][tid + 1] = m[3];
         sb[par][1][tid + 1] = m[4];
@@ -418,7 +466,8 @@ __global__ void __launch_bounds__(kDiagThreads, 4)
         PairSum p;
 #pragma unroll
         for (int k = 0; k < 9; ++k) p.add(load_as<float>(h[k]));
-        sb[par][lane & 1][lane >> 1 ? cols + 1 : 0] = p.value();
+        // (moments_diverged: sums of binary16 values do not overflow, so hi has the infinities)
+        sb[par][lane & 1][lane >> 1 ? cols + 1 : 0] = REL && !isfinite(p.hi) ? widen(p.hi) : p.value();
       }
       __syncthreads();  // the buffers of this parity are rewritten after the next row's barrier
       if (tid < cols) {
