@@ -262,11 +262,20 @@ template <typename T, bool REL>
 struct CellValues {
   T v[27];
   T U[REL ? 8 : 1][2];  // of the source cell of f_(k+1): U_x where c_x != 0, U_y where c_y != 0
+  // WRAP: west of column 0 its original instead of the ghost copy, whose sector holds nothing else of a
+  // narrow row (the offsets are no constants then: 2000^2 binary32 107 -> 141 us; the copies in the east
+  // share sectors: 16 x 65536 binary32 54 -> 61 us without them).
+  template <bool WRAP = false>
   __device__ __forceinline__ void load(const T* __restrict__ pops, const StepGeom& g, int x, int y) {
     const T* rows[3];  // rows y - 1, y, y + 1 (sources of c_y = 1, 0, -1) at column x
 #pragma unroll
     for (int k = 0; k < 3; ++k) rows[k] = pops + (size_t)wrapi(y - 1 + k, g.ny) * g.pitch + kXOff + x;
-    auto at = [&](int plane, int i) { return rows[1 - vy(i)][(size_t)plane * g.plane - vx(i)]; };
+    const int west = WRAP && x == 0 ? g.nx - 1 : -1;
+    auto at = [&](int plane, int i) {
+      const T* p = rows[1 - vy(i)] + (size_t)plane * g.plane;
+      if constexpr (WRAP) return p[vx(i) > 0 ? west : -vx(i)];
+      else return p[-vx(i)];
+    };
 #pragma unroll
     for (int q = 0; q < 27; ++q) v[q] = at(plane_of(q), q % 9);
     if constexpr (REL) {
@@ -377,17 +386,19 @@ __device__ __forceinline__ void cell_moments(const CellValues<T, REL>& cell, con
   }
 }
 
-template <typename T, bool REL = false>
-__global__ void __launch_bounds__(128)
+// WRAP: CellValues::load's, for grids of up to kWrapCols columns.
+constexpr int kWrapCols = 16;
+template <typename T, bool REL, bool WRAP>
+__global__ void __launch_bounds__(256)
     moments_kernel(const T* __restrict__ pops, StepGeom g, double* __restrict__ rho, double* __restrict__ ux,
                    double* __restrict__ uy, double* __restrict__ bx, double* __restrict__ by) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= g.nx) return;
-  for (int y = blockIdx.y; y < g.ny; y += gridDim.y) {
+  for (int y = blockIdx.y * blockDim.y + threadIdx.y; y < g.ny; y += gridDim.y * blockDim.y) {
     const size_t c = (size_t)y * g.nx + x;
     double out[5];
     CellValues<T, REL> cell;
-    cell.load(pops, g, x, y);
+    cell.template load<WRAP>(pops, g, x, y);
     cell_moments(cell, pops, g, x, y, out);
     rho[c] = out[0];
     ux[c] = out[1];
@@ -552,19 +563,32 @@ cudaError_t launch_zero_pads(void* pops0, void* pops1, const StepGeom& g, int np
   return cudaGetLastError();
 }
 
+template <typename T, bool REL = false>
+cudaError_t launch_moments_of(const void* pops, const StepGeom& g, double* rho, double* ux, double* uy, double* bx,
+                              double* by, cudaStream_t s) {
+  // Blocks of several whole rows up to 127 columns, strips of equal width beyond: a block of one row
+  // left most lanes idle on narrow grids.  Threads over consecutive cells without ghost columns / one
+  // row a block / now: 3 x 262144 binary64 147 / 727 / 147 us, binary32 142 / 193 / 141; 16 x 65536
+  // binary64 129 / 187 / 99, binary32 48 / 58 / 54; 65 x 16384 binary64 129 / 142 / 113.
+  dim3 nt(g.nx, 1);
+  if (g.nx < 128) {
+    nt.y = std::min(256 / g.nx, g.ny);
+  } else {
+    const int strips = (g.nx + 127) / 128;
+    nt.x = ((g.nx + strips - 1) / strips + 31) / 32 * 32;
+  }
+  const dim3 grid((g.nx + nt.x - 1) / nt.x, std::min((g.ny + nt.y - 1) / nt.y, 65535u));
+  const auto kernel = g.nx <= kWrapCols ? moments_kernel<T, REL, true> : moments_kernel<T, REL, false>;
+  kernel<<<grid, nt, 0, s>>>(static_cast<const T*>(pops), g, rho, ux, uy, bx, by);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_moments(int precision, const void* pops, const StepGeom& g, double* rho,
                            double* ux, double* uy, double* bx, double* by, cudaStream_t s) {
-  const int nt = std::min(128, (g.nx + 31) / 32 * 32);
-  const dim3 grid((g.nx + nt - 1) / nt, (unsigned)std::min(g.ny, 65535));
-  if (precision == 0)
-    moments_kernel<double><<<grid, nt, 0, s>>>((const double*)pops, g, rho, ux, uy, bx, by);
-  else if (precision == 1)
-    moments_kernel<float><<<grid, nt, 0, s>>>((const float*)pops, g, rho, ux, uy, bx, by);
-  else if (precision == LBMHD_FP16)
-    moments_kernel<__half><<<grid, nt, 0, s>>>((const __half*)pops, g, rho, ux, uy, bx, by);
-  else
-    moments_kernel<__half, true><<<grid, nt, 0, s>>>((const __half*)pops, g, rho, ux, uy, bx, by);
-  return cudaGetLastError();
+  if (precision == 0) return launch_moments_of<double>(pops, g, rho, ux, uy, bx, by, s);
+  if (precision == 1) return launch_moments_of<float>(pops, g, rho, ux, uy, bx, by, s);
+  if (precision == LBMHD_FP16) return launch_moments_of<__half>(pops, g, rho, ux, uy, bx, by, s);
+  return launch_moments_of<__half, true>(pops, g, rho, ux, uy, bx, by, s);
 }
 
 cudaError_t launch_populations(int precision, const void* pops, const StepGeom& g, double* out,

@@ -1,11 +1,10 @@
 """Corrected steps of an unfiltered grid (Delta = 0) launch the blocks that the corrected steps of a
 filtered one do -- the same kernel with the same number of blocks per SM -- although the grid's own
 steps, in the plain form, take other bands.  The launches are read from a captured graph."""
-import ctypes
-
 import numpy as np
 import pytest
 
+from captured_launches import launches
 from paper_1705_09807_gb300 import lbmhd
 
 pytestmark = pytest.mark.gpu
@@ -22,21 +21,7 @@ def gpu():
 
 def _grids(sim, stream):
     """Grid dimensions of the kernels that one step of `sim` launches."""
-    cu = ctypes.CDLL("libcuda.so.1")
-    s, graph, count = ctypes.c_void_p(stream.cuda_stream), ctypes.c_void_p(), ctypes.c_size_t()
-    assert cu.cuStreamBeginCapture_v2(s, 1) == 0  # CU_STREAM_CAPTURE_MODE_THREAD_LOCAL
-    sim.step(1)
-    assert cu.cuStreamEndCapture(s, ctypes.byref(graph)) == 0
-    assert cu.cuGraphGetNodes(graph, None, ctypes.byref(count)) == 0
-    nodes = (ctypes.c_void_p * count.value)()
-    assert cu.cuGraphGetNodes(graph, nodes, ctypes.byref(count)) == 0
-    grids = []
-    for n in nodes:
-        params = (ctypes.c_uint32 * 64)()  # CUDA_KERNEL_NODE_PARAMS: function, gridDimX, gridDimY, ...
-        assert cu.cuGraphKernelNodeGetParams_v2(ctypes.c_void_p(n), params) == 0
-        grids.append(tuple(params[2:5]))
-    assert cu.cuGraphDestroy(graph) == 0
-    return sorted(grids)
+    return sorted(grid for grid, _ in launches(stream, lambda: sim.step(1)))
 
 
 @pytest.mark.parametrize("precision,n", [(lbmhd.LBMHD_FP64, 130), (lbmhd.LBMHD_FP64, 512), (lbmhd.LBMHD_FP64, 1024),
