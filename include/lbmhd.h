@@ -136,7 +136,8 @@ int lbmhd_get_populations(lbmhd_t* h, double* pops);
  * [5] sum rho |u|^2 / 2  [6] sum |B|^2 / 2  [7] max |div B| (isotropic stencil)
  * [8] max |div B| (central stencil)  [9] max |d_beta B_alpha| (isotropic stencil).
  * Sums are reduced in a fixed order (bitwise reproducible).  Synchronises; the moment fields
- * of a binary64 state go through the handle's device buffer (allocated on first use).  Returns
+ * of a binary64 state, or of a grid of up to 64 columns and more than 1216 rows, go through the
+ * handle's device buffer (allocated on first use).  Returns
  * LBMHD_ERR_UNSTABLE (with out[] filled) if any cell has a NaN/Inf, rho <= 0 or |u| > 0.4. */
 int lbmhd_diagnostics(lbmhd_t* h, double* out);
 

@@ -417,7 +417,8 @@ __global__ void __launch_bounds__(256)
 // thread and two rows ahead, which four lanes of one warp, another one each row, add up.  One
 // tile per block, four blocks per SM, tiles of at least one row: a small grid takes the time of
 // three rows.  The next row's populations are loaded before this row's binary64 work where the
-// registers allow it (not with REL's eight more values).
+// registers allow it (not with REL's eight more values).  Cells of the relative form whose values are not
+// finite make NaN of an infinite moment; lbmhd_diagnostics then takes the way through the fields.
 // Kernels at 2048^2 binary32: moments 98 + reduction 224 -> 268 us.
 // Call of lbmhd_diagnostics with moments and reduction apart -> now: binary32 64^2 57 -> 48, 256^2 59
 // -> 58, 1024^2 146 -> 123, 2048^2 369 -> 307 us; binary16 2048^2 341 -> 281, relative 358 -> 330.
@@ -465,7 +466,7 @@ __global__ void __launch_bounds__(kDiagThreads, 4)
       }
       if (tid < cols) {
         if (!kAhead) cell.load(pops, g, x0 + tid, wrapi(y, ny));
-        cell_moments(cell, pops, g, x0 + tid, wrapi(y, ny), m);
+        cell.moments(m);
         if (kAhead && y < y1) cell.load(pops, g, x0 + tid, wrapi(y + 1, ny));
         sb[par][0][tid + 1] = m[3];
         sb[par][1][tid + 1] = m[4];
@@ -477,8 +478,7 @@ __global__ void __launch_bounds__(kDiagThreads, 4)
         PairSum p;
 #pragma unroll
         for (int k = 0; k < 9; ++k) p.add(load_as<float>(h[k]));
-        // (moments_diverged: sums of binary16 values do not overflow, so hi has the infinities)
-        sb[par][lane & 1][lane >> 1 ? cols + 1 : 0] = REL && !isfinite(p.hi) ? widen(p.hi) : p.value();
+        sb[par][lane & 1][lane >> 1 ? cols + 1 : 0] = p.value();
       }
       __syncthreads();  // the buffers of this parity are rewritten after the next row's barrier
       if (tid < cols) {
@@ -605,13 +605,20 @@ cudaError_t launch_populations(int precision, const void* pops, const StepGeom& 
   return cudaGetLastError();
 }
 
+// Binary64 moments take 46 binary64 instructions a cell, too many to form them again in the tiles' halo
+// rows: lbmhd_diagnostics at 256^2 60 us through the fields, 80 straight from the populations; 2048^2
+// 751 and 777 (both with the 62 instructions of a division per velocity).  The tiles of
+// diag_pops_kernel are one grid wide, so on narrow grids most of their lanes idle: from three rows a
+// block on the grouped pieces over the fields are faster (binary32, straight / through the fields: 16 x
+// 256 48 / 50 us, 16 x 1024 53 / 53, 16 x 2048 62 / 56, 16 x 65536 388 / 163, 63 x 65536 448 / 379).
+bool diagnostics_through_fields(int precision, int nx, int ny) {
+  return precision == 0 || (nx <= kDiagThreads / 2 && ny > 2 * kDiagPopsBlocks);
+}
+
 cudaError_t launch_diagnostics(int precision, const void* pops, const StepGeom& g, double* fields, double* partials,
-                               double* out, cudaStream_t s) {
-  // binary64 moments take 46 binary64 instructions a cell, too many to form them again in the
-  // tiles' halo rows: lbmhd_diagnostics at 256^2 60 us through the fields, 80 straight from the
-  // populations; 2048^2 751 and 777 (both with the 62 instructions of a division per velocity)
-  const bool through_fields = precision == 0;
-  const DiagTiles t = through_fields ? diag_tiles(g.nx, g.ny, kDiagBlocks) : diag_tiles(g.nx, g.ny, kDiagPopsBlocks, 1);
+                               double* out, bool through_fields, cudaStream_t s) {
+  const DiagTiles t = through_fields ? diag_tiles(g.nx, g.ny, kDiagBlocks, true, kDiagMinRows)
+                                     : diag_tiles(g.nx, g.ny, kDiagPopsBlocks, false, 1);
   if (through_fields) {
     const size_t n = (size_t)g.nx * g.ny;
     cudaError_t e = launch_moments(precision, pops, g, fields, fields + n, fields + 2 * n, fields + 3 * n,

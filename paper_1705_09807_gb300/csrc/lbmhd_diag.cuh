@@ -27,16 +27,23 @@ constexpr int kDiagThreads = 128;  // columns of a tile
 constexpr int kDiagMinRows = 4;    // rows of a tile, at least (halo rows are formed twice)
 
 // Tiles of kDiagThreads columns x `rows` rows: as few rows as keep the tiles within max_blocks.
+// `grouped`: on grids of up to half as many columns a tile is `groups` pieces of `cols` = nx columns, one
+// below the other, so that few lanes idle.  Fields to values, threads over consecutive cells / one
+// piece / now: 3 x 65536 82 / 164 / 30 us, 16 x 65536 170 / 164 / 80, 64 x 65536 581 / 269 / 236.
 struct DiagTiles {
   int strips, rows, blocks;
+  int cols, groups;
   long tiles;
 };
-inline DiagTiles diag_tiles(int nx, int ny, int max_blocks, int min_rows = kDiagMinRows) {
+inline DiagTiles diag_tiles(int nx, int ny, int max_blocks, bool grouped, int min_rows) {
   DiagTiles t;
   t.strips = (nx + kDiagThreads - 1) / kDiagThreads;
-  const long rows = ((long)t.strips * ny + max_blocks - 1) / max_blocks;
+  t.groups = grouped && nx <= kDiagThreads / 2 ? kDiagThreads / nx : 1;
+  t.cols = t.groups > 1 ? nx : kDiagThreads;
+  const long pieces = (long)max_blocks * t.groups;
+  const long rows = ((long)t.strips * ny + pieces - 1) / pieces;
   t.rows = (int)(rows < min_rows ? min_rows : (rows > ny ? ny : rows));
-  t.tiles = (long)t.strips * ((ny + t.rows - 1) / t.rows);
+  t.tiles = (long)t.strips * ((ny + (long)t.rows * t.groups - 1) / ((long)t.rows * t.groups));
   t.blocks = (int)(t.tiles < max_blocks ? t.tiles : max_blocks);
   return t;
 }
@@ -142,10 +149,12 @@ __global__ void __launch_bounds__(kDiagThreads)
                         double* __restrict__ partials) {
   DiagAcc acc;
   acc.clear();
+  const int group = (int)threadIdx.x / t.cols, col = (int)threadIdx.x - group * t.cols;
   for (long tile = blockIdx.x; tile < t.tiles; tile += gridDim.x) {
-    const int x = (int)(tile % t.strips) * kDiagThreads + threadIdx.x;
-    const int y0 = (int)(tile / t.strips) * t.rows, y1 = min(y0 + t.rows, ny);
-    if (x >= nx) continue;
+    const int x = (int)(tile % t.strips) * kDiagThreads + col;
+    const long top = (tile / t.strips * t.groups + group) * t.rows;
+    if (x >= nx || group >= t.groups || top >= ny) continue;
+    const int y0 = (int)top, y1 = (int)min(top + t.rows, (long)ny);
     const int xe = x + 1 == nx ? 0 : x + 1, xw = x == 0 ? nx - 1 : x - 1;
     DiagRows rows;
     auto row = [&](int y, int k) {

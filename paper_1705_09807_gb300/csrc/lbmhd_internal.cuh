@@ -156,12 +156,13 @@ cudaError_t launch_populations(int precision, const void* pops, const StepGeom& 
                                cudaStream_t s);
 // Diagnostics of the current populations: block partials into `partials` (kDiagBlocks x kDiagSlots
 // doubles, lbmhd_diag.cuh), then a single-block fixed-order reduction into out[kDiagSlots] (device).
-// Binary64 storage goes through `fields` (rho, ux, uy, bx, by, each nx*ny, contiguous), which the
-// other forms do not use.
+// `through_fields`: by way of `fields` (rho, ux, uy, bx, by, each nx*ny, contiguous), else from the
+// populations (not for binary64); diagnostics_through_fields says which is faster.
+bool diagnostics_through_fields(int precision, int nx, int ny);
 constexpr int kDiagBlocks = 1024;
 constexpr int kDiagSlots = LBMHD_NDIAG + 1;  // the public values and the instability flag
 cudaError_t launch_diagnostics(int precision, const void* pops, const StepGeom& g, double* fields,
-                               double* partials, double* out, cudaStream_t s);
+                               double* partials, double* out, bool through_fields, cudaStream_t s);
 
 // Analysis kernels (lbmhd_analysis.cu): r x r block mean, and the shell-summed energy spectra
 // of a square n x n field set into device outputs e_kin[nbins], e_mag[nbins], using `work` of

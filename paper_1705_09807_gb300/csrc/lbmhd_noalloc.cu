@@ -129,7 +129,7 @@ extern "C" int lbmhd_diagnostics_fields_noalloc(const double* rho, const double*
   int rc = partials_address(&partials);
   if (rc) return rc;
   // a quarter of the records fills the GPU; every record read is written first
-  const DiagTiles t = diag_tiles(nx, ny, kMaxBlocks / 4);
+  const DiagTiles t = diag_tiles(nx, ny, kMaxBlocks / 4, true, kDiagMinRows);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   diag_partial_kernel<<<t.blocks, kDiagThreads, 0, s>>>(rho, ux, uy, bx, by, nx, ny, t, partials);
   cudaError_t e = cudaGetLastError();
