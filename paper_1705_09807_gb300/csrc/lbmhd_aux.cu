@@ -572,7 +572,8 @@ cudaError_t launch_moments_of(const void* pops, const StepGeom& g, double* rho, 
   // binary64 129 / 187 / 99, binary32 48 / 58 / 54; 65 x 16384 binary64 129 / 142 / 113.
   dim3 nt(g.nx, 1);
   if (g.nx < 128) {
-    nt.y = std::min(256 / g.nx, g.ny);
+    // (as few rows as keep four blocks on every SM: 64^2 in blocks of four rows leaves most SMs idle)
+    nt.y = std::max(1, std::min(256 / g.nx, g.ny / (4 * 152)));
   } else {
     const int strips = (g.nx + 127) / 128;
     nt.x = ((g.nx + strips - 1) / strips + 31) / 32 * 32;
