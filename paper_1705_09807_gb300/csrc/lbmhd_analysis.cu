@@ -51,13 +51,16 @@ __device__ __forceinline__ double scale_down(double s, int k, double inv) {
 // 2048^2, r = 2, cold caches: 24.5 us with 64-bit divisions per cell and a grid-stride loop (a division
 // by r^2 in every thread cost another binary64 dozen), 13.9 with a first addition to zero and a
 // product in every thread, now 10.1 us.
-template <bool VEC>
+// UNROLL: loads in flight; few additions wait on one another in small cells and the remainder of a row
+// costs more (1300^2, r = 10: 4 12.3 us, 8 14.4; r = 26: 46, 55), in large ones the loads do (2048^2,
+// r = 32: 72, 57; r = 1024: 58 and 46 ms).
+template <bool VEC, int UNROLL>
 __global__ void __launch_bounds__(128)
     block_mean_kernel(const double* __restrict__ in, int nx, int mx, int my, int r, int log2sq, double inv,
                       double* __restrict__ out) {
-  const int i = blockIdx.x * 128 + threadIdx.x;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= mx) return;
-  for (int j = blockIdx.y; j < my; j += gridDim.y) {
+  for (int j = blockIdx.y * blockDim.y + threadIdx.y; j < my; j += gridDim.y * blockDim.y) {
     const double* row = in + (size_t)j * r * nx + (size_t)i * r;
     double s;
     if constexpr (VEC) {
@@ -70,14 +73,14 @@ __global__ void __launch_bounds__(128)
 #pragma unroll 2
     for (int yy = 0; yy < r; ++yy, row += nx, first = 0) {
       if constexpr (VEC) {
-#pragma unroll 4
+#pragma unroll UNROLL
         for (int xx = first; xx < r; xx += 2) {
           const double2 v = *reinterpret_cast<const double2*>(row + xx);
           s += v.x;
           s += v.y;
         }
       } else {
-#pragma unroll 4
+#pragma unroll UNROLL
         for (int xx = first; xx < r; ++xx) s += row[xx];
       }
     }
@@ -539,11 +542,19 @@ cudaError_t launch_block_mean(const double* in, int nx, int ny, int r, double* o
   int log2sq = -1;
   if ((r & (r - 1)) == 0)
     for (log2sq = 0; (1 << (log2sq / 2)) < r;) log2sq += 2;
-  const dim3 grid((mx + 127) / 128, my < 65535 ? my : 65535);
-  if (r % 2 == 0 && nx % 2 == 0 && reinterpret_cast<uintptr_t>(in) % 16 == 0)
-    block_mean_kernel<true><<<grid, 128, 0, s>>>(in, nx, mx, my, r, log2sq, inv, out);
-  else
-    block_mean_kernel<false><<<grid, 128, 0, s>>>(in, nx, mx, my, r, log2sq, inv, out);
+  // several whole rows of means to a block (but four blocks on every SM) where they are short: with one
+  // row to a block 4 x 262144, r = 4, took 86 us and 64 x 65536, r = 8, 39; now 7 and 14
+  dim3 nt(mx < 128 ? mx : 128, 1);
+  if (mx < 128) {
+    const int fit = 128 / mx, spread = my / (4 * 152);
+    nt.y = fit < spread ? fit : (spread > 1 ? spread : 1);
+  }
+  const int rows = (my + (int)nt.y - 1) / (int)nt.y;
+  const dim3 grid((mx + nt.x - 1) / nt.x, rows < 65535 ? rows : 65535);
+  const bool vec = r % 2 == 0 && nx % 2 == 0 && reinterpret_cast<uintptr_t>(in) % 16 == 0;
+  const auto kernel = r < 32 ? (vec ? block_mean_kernel<true, 4> : block_mean_kernel<false, 4>)
+                             : (vec ? block_mean_kernel<true, 8> : block_mean_kernel<false, 8>);
+  kernel<<<grid, nt, 0, s>>>(in, nx, mx, my, r, log2sq, inv, out);
   return cudaGetLastError();
 }
 
