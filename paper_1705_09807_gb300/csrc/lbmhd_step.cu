@@ -226,7 +226,10 @@ __device__ __forceinline__ double reciprocal(double r) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(r));
   const double e = fma(-r, y, 1.0);  // y (1 + e + e^2): relative error e^3 < 2^-57
-  return fma(y, fma(e, e, e), y);
+  // r = 0 or infinite (a state that has diverged): the estimate is the quotient and e is NaN
+  // (an integer test: the binary64 unit is the busy one)
+  const bool exact = (__double2hiint(e) & 0x7ff00000) == 0x7ff00000;
+  return exact ? y : fma(y, fma(e, e, e), y);
 }
 
 // One magnetic component toward b w_i -+ 3 w_i E (t = 3 w E on the axis, u on the diagonals):
