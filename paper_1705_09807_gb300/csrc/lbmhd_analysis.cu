@@ -499,9 +499,10 @@ size_t spectrum_work_bytes(int n) {
 
 cudaError_t launch_energy_spectrum(const double* ux, const double* uy, const double* bx,
                                    const double* by, int n, int nbins, double* ek, double* em,
-                                   void* work, cudaStream_t s) {
+                                   void* work, cudaStream_t s, int* launches) {
   const size_t nn = (size_t)n * n;
   const FftPlan p = make_plan(n);
+  if (launches) *launches = p.chirp() ? 5 : 4;
   // work: tables (len < 4n: at most 9n points), two complex planes, the column groups' shells
   // (at most n x nbins per pair): 144 n + 32 n^2 + 16 n^2 bytes within spectrum_work_bytes(n)
   FftTables t{};

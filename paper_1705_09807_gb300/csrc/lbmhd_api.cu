@@ -628,9 +628,10 @@ int lbmhd_energy_spectrum(lbmhd_t* h, int nbins, double* e_kin, double* e_mag) {
   double* f = h->fields;
   LB_CUDA(h, launch_moments(h->precision, h->pops[h->cur], h->geom, f, f + ncell, f + 2 * ncell,
                             f + 3 * ncell, f + 4 * ncell, h->stream));
+  int nl = 0;
   LB_CUDA(h, launch_energy_spectrum(f + ncell, f + 2 * ncell, f + 3 * ncell, f + 4 * ncell, n, nbins,
-                                    dk, dm, h->spec_work, h->stream));
-  h->launches += 5;
+                                    dk, dm, h->spec_work, h->stream, &nl));
+  h->launches += 1 + nl;
   LB_CUDA(h, cudaMemcpyAsync(e_kin, dk, nbins * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   LB_CUDA(h, cudaMemcpyAsync(e_mag, dm, nbins * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   LB_CUDA(h, cudaStreamSynchronize(h->stream));

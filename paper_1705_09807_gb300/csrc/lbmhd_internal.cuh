@@ -166,12 +166,12 @@ cudaError_t launch_diagnostics(int precision, const void* pops, const StepGeom& 
 
 // Analysis kernels (lbmhd_analysis.cu): r x r block mean, and the shell-summed energy spectra
 // of a square n x n field set into device outputs e_kin[nbins], e_mag[nbins], using `work` of
-// spectrum_work_bytes(n) bytes.
+// spectrum_work_bytes(n) bytes (*launches: its kernel launches).
 cudaError_t launch_block_mean(const double* in, int nx, int ny, int r, double* out, cudaStream_t s);
 size_t spectrum_work_bytes(int n);
 cudaError_t launch_energy_spectrum(const double* ux, const double* uy, const double* bx,
                                    const double* by, int n, int nbins, double* ek, double* em,
-                                   void* work, cudaStream_t s);
+                                   void* work, cudaStream_t s, int* launches = nullptr);
 
 // Learned closure (lbmhd_closure.cu): correction planes corr [4][ny][nx] (physical units) for
 // the current populations of a square binary64 (precision 0) or binary32 (1) grid, in one launch
