@@ -26,6 +26,7 @@
 
 #include <cmath>
 #include <cstdio>
+#include <type_traits>
 
 #include "lbmhd.h"
 #include "lbmhd_internal.cuh"
@@ -54,13 +55,15 @@ __device__ __forceinline__ double scale_down(double s, int k, double inv) {
 // UNROLL: loads in flight; few additions wait on one another in small cells and the remainder of a row
 // costs more (1300^2, r = 10: 4 12.3 us, 8 14.4; r = 26: 46, 55), in large ones the loads do (2048^2,
 // r = 32: 72, 57; r = 1024: 58 and 46 ms).
-template <bool VEC, int UNROLL>
+// ROWS: several rows of means to a block (else its row is the same in all threads).
+template <bool VEC, int UNROLL, bool ROWS>
 __global__ void __launch_bounds__(128)
     block_mean_kernel(const double* __restrict__ in, int nx, int mx, int my, int r, int log2sq, double inv,
                       double* __restrict__ out) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= mx) return;
-  for (int j = blockIdx.y * blockDim.y + threadIdx.y; j < my; j += gridDim.y * blockDim.y) {
+  const int rows = ROWS ? blockDim.y : 1;
+  for (int j = blockIdx.y * rows + (ROWS ? threadIdx.y : 0); j < my; j += gridDim.y * rows) {
     const double* row = in + (size_t)j * r * nx + (size_t)i * r;
     double s;
     if constexpr (VEC) {
@@ -553,8 +556,12 @@ cudaError_t launch_block_mean(const double* in, int nx, int ny, int r, double* o
   const int rows = (my + (int)nt.y - 1) / (int)nt.y;
   const dim3 grid((mx + nt.x - 1) / nt.x, rows < 65535 ? rows : 65535);
   const bool vec = r % 2 == 0 && nx % 2 == 0 && reinterpret_cast<uintptr_t>(in) % 16 == 0;
-  const auto kernel = r < 32 ? (vec ? block_mean_kernel<true, 4> : block_mean_kernel<false, 4>)
-                             : (vec ? block_mean_kernel<true, 8> : block_mean_kernel<false, 8>);
+  const auto pick = [&](auto rows_tag) {
+    constexpr bool R = decltype(rows_tag)::value;
+    return r < 32 ? (vec ? block_mean_kernel<true, 4, R> : block_mean_kernel<false, 4, R>)
+                  : (vec ? block_mean_kernel<true, 8, R> : block_mean_kernel<false, 8, R>);
+  };
+  const auto kernel = nt.y > 1 ? pick(std::true_type{}) : pick(std::false_type{});
   kernel<<<grid, nt, 0, s>>>(in, nx, mx, my, r, log2sq, inv, out);
   return cudaGetLastError();
 }

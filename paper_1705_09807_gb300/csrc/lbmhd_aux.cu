@@ -386,15 +386,18 @@ __device__ __forceinline__ void cell_moments(const CellValues<T, REL>& cell, con
   }
 }
 
-// WRAP: CellValues::load's, for grids of up to kWrapCols columns.
+// ROWS: several rows per block.  WRAP: CellValues::load's, for grids of up to kWrapCols columns.
 constexpr int kWrapCols = 16;
-template <typename T, bool REL, bool WRAP>
-__global__ void __launch_bounds__(256)
+template <typename T, bool REL, bool ROWS, bool WRAP>
+__global__ void __launch_bounds__(ROWS ? 256 : 128)
     moments_kernel(const T* __restrict__ pops, StepGeom g, double* __restrict__ rho, double* __restrict__ ux,
                    double* __restrict__ uy, double* __restrict__ bx, double* __restrict__ by) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= g.nx) return;
-  for (int y = blockIdx.y * blockDim.y + threadIdx.y; y < g.ny; y += gridDim.y * blockDim.y) {
+  // (a block's one row is known to be the same in all threads: with the row per thread 2048^2 binary32
+  // took 113 instead of 99 us)
+  const int rows = ROWS ? blockDim.y : 1, y0 = blockIdx.y * rows + (ROWS ? threadIdx.y : 0);
+  for (int y = y0; y < g.ny; y += gridDim.y * rows) {
     const size_t c = (size_t)y * g.nx + x;
     double out[5];
     CellValues<T, REL> cell;
@@ -579,7 +582,9 @@ cudaError_t launch_moments_of(const void* pops, const StepGeom& g, double* rho, 
     nt.x = ((g.nx + strips - 1) / strips + 31) / 32 * 32;
   }
   const dim3 grid((g.nx + nt.x - 1) / nt.x, std::min((g.ny + nt.y - 1) / nt.y, 65535u));
-  const auto kernel = g.nx <= kWrapCols ? moments_kernel<T, REL, true> : moments_kernel<T, REL, false>;
+  const auto kernel = g.nx <= kWrapCols ? moments_kernel<T, REL, true, true>
+                      : nt.y > 1        ? moments_kernel<T, REL, true, false>
+                                        : moments_kernel<T, REL, false, false>;
   kernel<<<grid, nt, 0, s>>>(static_cast<const T*>(pops), g, rho, ux, uy, bx, by);
   return cudaGetLastError();
 }
@@ -607,8 +612,8 @@ cudaError_t launch_populations(int precision, const void* pops, const StepGeom& 
 }
 
 // Binary64 moments take 46 binary64 instructions a cell, too many to form them again in the tiles' halo
-// rows: lbmhd_diagnostics at 256^2 60 us through the fields, 80 straight from the populations; 2048^2
-// 751 and 777 (both with the 62 instructions of a division per velocity).  The tiles of
+// rows: lbmhd_diagnostics at 256^2 57 us through the fields, 75 straight from the populations; 1024^2 205
+// and 222; 2048^2 636 and 661 (below that 128^2 56.5 and 54.3).  The tiles of
 // diag_pops_kernel are one grid wide, so on narrow grids most of their lanes idle: from three rows a
 // block on the grouped pieces over the fields are faster (binary32, straight / through the fields: 16 x
 // 256 48 / 50 us, 16 x 1024 53 / 53, 16 x 2048 62 / 56, 16 x 65536 388 / 163, 63 x 65536 448 / 379).
@@ -625,8 +630,7 @@ cudaError_t launch_diagnostics(int precision, const void* pops, const StepGeom& 
     cudaError_t e = launch_moments(precision, pops, g, fields, fields + n, fields + 2 * n, fields + 3 * n,
                                    fields + 4 * n, s);
     if (e != cudaSuccess) return e;
-    diag_partial_kernel<<<t.blocks, kDiagThreads, 0, s>>>(fields, fields + n, fields + 2 * n, fields + 3 * n,
-                                                           fields + 4 * n, g.nx, g.ny, t, partials);
+    launch_diag_partials(fields, fields + n, fields + 2 * n, fields + 3 * n, fields + 4 * n, g.nx, g.ny, t, partials, s);
   } else if (precision == 1) {
     diag_pops_kernel<float><<<t.blocks, kDiagThreads, 0, s>>>((const float*)pops, g, t, partials);
   } else if (precision == LBMHD_FP16) {

@@ -131,7 +131,7 @@ extern "C" int lbmhd_diagnostics_fields_noalloc(const double* rho, const double*
   // a quarter of the records fills the GPU; every record read is written first
   const DiagTiles t = diag_tiles(nx, ny, kMaxBlocks / 4, true, kDiagMinRows);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  diag_partial_kernel<<<t.blocks, kDiagThreads, 0, s>>>(rho, ux, uy, bx, by, nx, ny, t, partials);
+  launch_diag_partials(rho, ux, uy, bx, by, nx, ny, t, partials, s);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) {
     diag_final_kernel<<<1, 32 * kDiagSlots, 0, s>>>(partials, t.blocks, out);
