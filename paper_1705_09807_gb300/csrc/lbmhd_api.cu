@@ -587,9 +587,14 @@ int lbmhd_diagnostics(lbmhd_t* h, double* out) {
   if (!out) return fail(h, LBMHD_ERR_INVALID, "out is NULL");
   bool through_fields = diagnostics_through_fields(h->precision, h->p.nx, h->p.ny);
   double res[kDiagSlots];
-  for (;;) {
+  for (bool have = false;; have = true) {
     int frc = through_fields ? ensure_fields(h) : LBMHD_OK;
-    if (frc) return frc;
+    if (frc) {  // no memory for the fields: straight from the populations where that form exists
+      if (h->precision == LBMHD_FP64) return frc;
+      cudaGetLastError();
+      if (have) break;
+      through_fields = false;
+    }
     LB_CUDA(h, launch_diagnostics(h->precision, h->pops[h->cur], h->geom, h->fields, h->partials, h->diag_out,
                                   through_fields, h->stream));
     h->launches += through_fields ? 3 : 2;
