@@ -220,6 +220,42 @@ __global__ void __launch_bounds__(kConvThreads, 2)
   }
 }
 
+// Forward convolution with one thread per cell (all outputs; weights a shared-memory load per FMA): for
+// sets of narrow, low or small grids, whose tiles are mostly empty (conv).  Same order of sums, so
+// the results are bitwise those of the tiles.
+template <int CIN, int COUT, bool TANH>
+__global__ void __launch_bounds__(kThreads)
+    conv_cell_kernel(const float* __restrict__ in, const float* __restrict__ params, int batch, int H, int W,
+                     float* __restrict__ out) {
+  __shared__ float sw[COUT * CIN * 9 + COUT];
+  for (int i = threadIdx.x; i < COUT * CIN * 9 + COUT; i += blockDim.x) sw[i] = params[i];
+  __syncthreads();
+  const long plane = (long)H * W, total = (long)batch * plane;
+  for (long c = blockIdx.x * (long)blockDim.x + threadIdx.x; c < total; c += (long)gridDim.x * blockDim.x) {
+    const int b = (int)(c / plane);
+    const long cell = c % plane;
+    const int y = (int)(cell / W), x = (int)(cell % W);
+    long off[9];
+#pragma unroll
+    for (int t = 0; t < 9; ++t) off[t] = (long)wrapi(y + t / 3 - 1, H) * W + wrapi(x + t % 3 - 1, W);
+    float acc[COUT];
+#pragma unroll
+    for (int co = 0; co < COUT; ++co) acc[co] = sw[COUT * CIN * 9 + co];
+    const float* ib = in + (size_t)b * CIN * plane;
+    for (int ci = 0; ci < CIN; ++ci) {
+#pragma unroll
+      for (int t = 0; t < 9; ++t) {
+        const float v = ib[(size_t)ci * plane + off[t]];
+#pragma unroll
+        for (int co = 0; co < COUT; ++co) acc[co] = fmaf(sw[(co * CIN + ci) * 9 + t], v, acc[co]);
+      }
+    }
+    float* ob = out + (size_t)b * COUT * plane + cell;
+#pragma unroll
+    for (int co = 0; co < COUT; ++co) ob[(size_t)co * plane] = TANH ? tanhf(acc[co]) : acc[co];
+  }
+}
+
 // ---- weight gradients ----------------------------------------------------------------------------
 // dW[co][ci][t] = sum_z dy[co](z) a[ci](z + d_t), db[co] = sum_z dy[co](z).  Bound by binary32 FMAs
 // (18,432 flops per cell for the 32 x 32 layer).  Lane l of a warp holds channel l of the
@@ -1202,6 +1238,18 @@ template <int CIN, int COUT, int EPI, bool BWD = false>
 cudaError_t conv(const float* in, const float* params, const float* aux, int batch, int H, int W, float* out,
                  double* loss_part, cudaStream_t s) {
   using Sh = ConvShape<CIN, COUT>;
+  if constexpr (!BWD && (EPI == kEpiNone || EPI == kEpiTanh)) {
+    // A full tile takes about a third of the time of as many cells with a thread each, an empty one
+    // as long as a full one; up to one wave of tiles costs the same 80 us for the network.  Binary32 forward
+    // pass by cells / by tiles: 65536 x 8 892 / 1234 us, 65536 x 16 1668 / 1227, 4 x 65536 505 / 687, 1024
+    // grids of 8 x 8 147 / 362, 4096 of 4 x 4 151 / 1388; 64 of 4 x 4 97 / 82; 3 x 3 83 / 85, one cell 75 / 107.
+    const long cells = (long)batch * H * W;
+    const long tiles = (long)batch * ((H + Sh::kRows - 1) / Sh::kRows) * ((W + kTileW - 1) / kTileW);
+    if (cells < 9 || (tiles > kMaxConvBlocks && 3 * cells < (long)Sh::kRows * kTileW * tiles)) {
+      conv_cell_kernel<CIN, COUT, EPI == kEpiTanh><<<grid_for(cells), kThreads, 0, s>>>(in, params, batch, H, W, out);
+      return cudaGetLastError();
+    }
+  }
   auto k = conv_tile_kernel<CIN, COUT, EPI, BWD>;
   if (Sh::kSmem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::kSmem);
