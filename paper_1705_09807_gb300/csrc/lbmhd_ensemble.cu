@@ -27,6 +27,7 @@ struct lbmhd_ensemble {
   int n = 0;
   int precision = 0;
   int stencil = 0;
+  bool three = false;              // a member has three columns
   int num_sms = 152;
   std::vector<lbmhd_t*> members;
   cudaStream_t stream = nullptr;
@@ -151,7 +152,7 @@ int build_work(lbmhd_ensemble_t* e, int rows_per_tile, int persistent) {
 
 int launch_one(lbmhd_ensemble_t* e, int parity) {
   if (e->persistent) ENS_CUDA(e, cudaMemsetAsync(e->d_queue, 0, sizeof(unsigned long long), e->stream));
-  ENS_CUDA(e, launch_ensemble_step(e->precision, e->stencil, e->d_members, e->d_work, e->nwork, parity,
+  ENS_CUDA(e, launch_ensemble_step(e->precision, e->stencil, e->three, e->d_members, e->d_work, e->nwork, parity,
                                    e->persistent ? e->d_queue : nullptr, e->grid, e->d_err, e->stream));
   return LBMHD_OK;
 }
@@ -259,6 +260,7 @@ int lbmhd_ensemble_create(lbmhd_ensemble_t** out, int n, const lbmhd_params* par
     }
     h->in_ensemble = true;
     e->members.push_back(h);
+    e->three = e->three || h->p.nx == 3;
   }
   int rc = LBMHD_OK;
   if ((ce = device_malloc(&e->d_queue, sizeof(unsigned long long))) != cudaSuccess ||

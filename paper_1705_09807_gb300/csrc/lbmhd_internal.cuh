@@ -140,7 +140,8 @@ unsigned bounds_check_flags();
 size_t ensemble_member_bytes(int precision);
 void pack_ensemble_members(int precision, int n, const CUtensorMap* maps, void* const* pops,
                            const StepGeom* geoms, const StepCoef* coefs, void* host_out);
-cudaError_t launch_ensemble_step(int precision, int stencil, const void* members, const int4* work,
+// three: a member may have three columns (binary16).
+cudaError_t launch_ensemble_step(int precision, int stencil, bool three, const void* members, const int4* work,
                                  int nwork, int parity, unsigned long long* queue, int grid,
                                  unsigned* err, cudaStream_t s);
 int resident_step_blocks(int precision, int num_sms);

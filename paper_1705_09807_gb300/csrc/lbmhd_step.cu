@@ -920,17 +920,15 @@ __device__ __forceinline__ void store_cell_pair(__half* __restrict__ dst, const 
       }
     }
   }
-  // ghosts: columns 0, 1 at nx, nx + 1 and nx - 2, nx - 1 at -2, -1; the middle one of three columns
-  // has both, in a second turn of the loop (written out for either side the stores grow to twice the
-  // code and the steps by 2 to 5%: 4096^2 and the relative form at 2047 x 2048)
+  // ghosts: columns 0, 1 at nx, nx + 1 and nx - 2, nx - 1 at -2, -1 (of three columns the middle one only at
+  // nx + 1: a second ghost of a column, in any form, took other grids 1 to 5% more time; run_tile_pair with
+  // THREE, the only reader of -2, does without)
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const int xh = x + h;
     if (h == 1 && !both) break;
-    int shift = xh < 2 ? g.nx : (xh >= g.nx - 2 ? -g.nx : 0);
-#pragma unroll 1
-    while (shift != 0) {
-      __half* gp = o + h + shift;
+    if (xh < 2 || xh >= g.nx - 2) {
+      __half* gp = o + h + (xh < 2 ? g.nx : -g.nx);
 #pragma unroll
       for (int q = 0; q < kQ; ++q) {
         __half* a = gp + (size_t)plane_of(q) * g.plane;
@@ -943,7 +941,6 @@ __device__ __forceinline__ void store_cell_pair(__half* __restrict__ dst, const 
           if (LB_IN(a >= dst && a < end, 2)) *a = h ? __high2half(uh[comp]) : __low2half(uh[comp]);
         }
       }
-      shift = shift > 0 && xh >= g.nx - 2 ? -g.nx : 0;
     }
   }
 }
@@ -957,7 +954,9 @@ __device__ __forceinline__ void store_cell_pair(__half* __restrict__ dst, const 
 // ring, the pulled f values are taken relative to their source cells' U (staged_pair_rel), and
 // the post-collision f values are stored relative to this cell's own velocity, which is stored
 // in binary16 as its U.
-template <int ISO, int NST, bool REL = false>
+// THREE: the grid may have three columns (forms of their own: the choice in every row took other grids
+// 0.5 to 2% more time).
+template <int ISO, int NST, bool REL, bool THREE>
 __device__ __forceinline__ bool run_tile_pair(const CUtensorMap* srcp, __half* __restrict__ dst, const StepGeom& g,
                                               const KCoef<float>& c1, int x0, int y0, int band_parity,
                                               uint32_t& kbase, unsigned* __restrict__ err,
@@ -1044,8 +1043,8 @@ __device__ __forceinline__ bool run_tile_pair(const CUtensorMap* srcp, __half* _
       rho_next = r1;
     }
     float r1, jx, jy, bx, by;
-    if (t == 0) {
-      moments_one_rel<BW, REL>(st, GE, LEAD - 1, ur, r1, jx, jy, bx, by);
+    if (t == 0) {  // (of three columns: column 2, the same cell, whose sources are all written)
+      moments_one_rel<BW, REL>(st, GE, THREE && nx == 3 ? LEAD + 2 : LEAD - 1, ur, r1, jx, jy, bx, by);
       rg[0 * RW + 1] = jx;
       rg[1 * RW + 1] = jy;
       rg[2 * RW + 1] = bx;
@@ -1288,7 +1287,7 @@ __device__ __forceinline__ bool run_any_tile(const CUtensorMap* srcp, S* __restr
                                              int band_parity, uint32_t& kbase, unsigned* __restrict__ err,
                                              const float* __restrict__ corr = nullptr) {
   if constexpr (sizeof(S) == 2)
-    return run_tile_pair<ISO, NST>(srcp, dst, g, c, x0, y0, band_parity, kbase, err);
+    return run_tile_pair<ISO, NST, false, CORR>(srcp, dst, g, c, x0, y0, band_parity, kbase, err);
   else
     return run_tile<S, ISO, NST, CORR>(srcp, dst, g, c, x0, y0, band_parity, kbase, err, corr);
 }
@@ -1317,7 +1316,7 @@ __device__ __forceinline__ void tile_of_block(int& strip, int& band) {
 }
 
 // One grid: one block per tile (strip, band), see tile_of_block.  CORR: add the correction planes
-// corr[4][ny][nx].  flip (0 / 1, the source copy's index, so it alternates from step to step)
+// corr[4][ny][nx]; binary16, which takes none: the form for three columns.  flip (0 / 1, the source copy's index, so it alternates from step to step)
 // reverses every band's marching direction: a band then starts each step at the rows it (and its
 // neighbour) wrote last in the previous step, which are still in L2 (about the last 5 rows per
 // band at 2048^2 binary32), instead of at the far end, long evicted.
@@ -1352,7 +1351,7 @@ __global__ void __launch_bounds__(step_threads<S>(), MINB)
 
 // Relative binary16 storage (LBMHD_FP16_REL; single grids): fused_step_kernel's binary16 step
 // with the U planes' tensor map (fixed marching direction, as for binary16).
-template <int ISO, int NST, int MINB>
+template <int ISO, int NST, int MINB, bool THREE>
 __global__ void __launch_bounds__(kStepThreads / 2, MINB)
     fused_step_rel_kernel(const __grid_constant__ CUtensorMap src, const __grid_constant__ CUtensorMap usrc,
                           __half* __restrict__ dst, StepGeom g, KCoef<float> c, unsigned* __restrict__ err) {
@@ -1362,7 +1361,7 @@ __global__ void __launch_bounds__(kStepThreads / 2, MINB)
   init_stage_barriers(step_smem<__half, NST, true>(), &src, &usrc);
   grid_dependency_wait();
   uint32_t kbase = 0;
-  run_tile_pair<ISO, NST, true>(&src, dst, g, c, strip * kStepThreads, band * g.band, band, kbase, err, &usrc);
+  run_tile_pair<ISO, NST, true, THREE>(&src, dst, g, c, strip * kStepThreads, band * g.band, band, kbase, err, &usrc);
 }
 
 // Ensemble: every member grid advances one step in this launch.  work[i] = {member, x0, y0,
@@ -1376,7 +1375,8 @@ struct EnsembleMember {
   KCoef<typename ArithOf<S>::type> c;
 };
 
-template <typename S, int ISO, int NST, int MINB>
+// THREE (binary16): a member may have three columns.
+template <typename S, int ISO, int NST, int MINB, bool THREE>
 __global__ void __launch_bounds__(step_threads<S>(), MINB)
     ensemble_step_kernel(const EnsembleMember<S>* __restrict__ members, const int4* __restrict__ work,
                          int nwork, int parity, unsigned long long* queue, unsigned* __restrict__ err) {
@@ -1396,7 +1396,7 @@ __global__ void __launch_bounds__(step_threads<S>(), MINB)
     // the march direction alternates with the step (parity) as for single grids: not for
     // binary16 storage
     const int flip = sizeof(S) == 2 ? 0 : parity;
-    if (!run_any_tile<S, ISO, NST>(&mb.map[parity], mb.pops[parity ^ 1], mb.g, mb.c, it.y, it.z, it.w + flip,
+    if (!run_any_tile<S, ISO, NST, THREE>(&mb.map[parity], mb.pops[parity ^ 1], mb.g, mb.c, it.y, it.z, it.w + flip,
                                    kbase, err))
       return;
     if (queue) {
@@ -1540,9 +1540,9 @@ constexpr size_t smem_bytes() {
   return sizeof(StepSmem<S, StepConfig<S>::kStages>) + 128;  // + alignment slack
 }
 
-template <int ISO>
+template <int ISO, bool THREE = false>
 constexpr auto rel_kernel_ptr() {
-  return &fused_step_rel_kernel<ISO, StepConfig<__half>::kStages, StepConfig<__half>::kMinBlocks>;
+  return &fused_step_rel_kernel<ISO, StepConfig<__half>::kStages, StepConfig<__half>::kMinBlocks, THREE>;
 }
 constexpr size_t rel_smem_bytes() { return sizeof(StepSmem<__half, StepConfig<__half>::kStages, true>) + 128; }
 // six relative-form blocks per SM: 6 x (rel_smem_bytes + 1 KB reserved) within 228 KB
@@ -1571,6 +1571,9 @@ cudaError_t launch_step(const CUtensorMap& src, S* dst, const StepGeom& g, const
   if (g.plain)
     return launch_programmatic(plain_kernel_ptr<S>(), grid, nt, plain_smem_bytes<S>(), s, src, src, dst, g, k, err, flip);
   const float* none = nullptr;
+  if (sizeof(S) == 2 && g.nx == 3)
+    return stencil == 1 ? launch_programmatic(kernel_ptr<S, 1, true>(), grid, nt, sm, s, src, dst, g, k, err, none, flip)
+                        : launch_programmatic(kernel_ptr<S, 0, true>(), grid, nt, sm, s, src, dst, g, k, err, none, flip);
   return stencil == 1 ? launch_programmatic(kernel_ptr<S, 1>(), grid, nt, sm, s, src, dst, g, k, err, none, flip)
                       : launch_programmatic(kernel_ptr<S, 0>(), grid, nt, sm, s, src, dst, g, k, err, none, flip);
 }
@@ -1584,13 +1587,16 @@ cudaError_t launch_step_rel(const CUtensorMap& src, const CUtensorMap& usrc, __h
     return launch_programmatic(plain_kernel_ptr<__half, true>(), grid, nt, plain_smem_bytes<__half, true>(), s, src, usrc,
                                dst, g, k, err, 0);
   const size_t sm = rel_smem_bytes();
+  if (g.nx == 3)
+    return stencil == 1 ? launch_programmatic(rel_kernel_ptr<1, true>(), grid, nt, sm, s, src, usrc, dst, g, k, err)
+                        : launch_programmatic(rel_kernel_ptr<0, true>(), grid, nt, sm, s, src, usrc, dst, g, k, err);
   return stencil == 1 ? launch_programmatic(rel_kernel_ptr<1>(), grid, nt, sm, s, src, usrc, dst, g, k, err)
                       : launch_programmatic(rel_kernel_ptr<0>(), grid, nt, sm, s, src, usrc, dst, g, k, err);
 }
 
-template <typename S, int ISO>
+template <typename S, int ISO, bool THREE = false>
 constexpr auto ensemble_kernel_ptr() {
-  return &ensemble_step_kernel<S, ISO, StepConfig<S>::kStages, StepConfig<S>::kMinBlocks>;
+  return &ensemble_step_kernel<S, ISO, StepConfig<S>::kStages, StepConfig<S>::kMinBlocks, THREE>;
 }
 
 template <typename S>
@@ -1607,16 +1613,20 @@ cudaError_t set_smem_attr() {
       e = cudaFuncSetAttribute(plain_kernel_ptr<S, true>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)plain_smem_bytes<S, true>());
   }
-  if constexpr (sizeof(S) != 2) {
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(kernel_ptr<S, 0, true>(), cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(kernel_ptr<S, 1, true>(), cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-  }
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(kernel_ptr<S, 0, true>(), cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(kernel_ptr<S, 1, true>(), cudaFuncAttributeMaxDynamicSharedMemorySize, b);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(ensemble_kernel_ptr<S, 0>(), cudaFuncAttributeMaxDynamicSharedMemorySize, b);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(ensemble_kernel_ptr<S, 1>(), cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+  if constexpr (sizeof(S) == 2) {
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(ensemble_kernel_ptr<S, 0, true>(), cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(ensemble_kernel_ptr<S, 1, true>(), cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+  }
   return e;
 }
 
@@ -1635,20 +1645,17 @@ void pack_members(int n, const CUtensorMap* maps, void* const* pops, const StepG
 }
 
 template <typename S>
-cudaError_t launch_ens(int stencil, const void* members, const int4* work, int nwork, int parity,
+cudaError_t launch_ens(int stencil, bool three, const void* members, const int4* work, int nwork, int parity,
                        unsigned long long* queue, int grid, unsigned* err, cudaStream_t s) {
   const EnsembleMember<S>* mb = static_cast<const EnsembleMember<S>*>(members);
+  auto kernel = stencil == 1 ? ensemble_kernel_ptr<S, 1>() : ensemble_kernel_ptr<S, 0>();
+  if constexpr (sizeof(S) == 2)
+    if (three) kernel = stencil == 1 ? ensemble_kernel_ptr<S, 1, true>() : ensemble_kernel_ptr<S, 0, true>();
   if (!queue)  // static schedule: the previous launch is the previous step kernel
-    return stencil == 1
-               ? launch_programmatic(ensemble_kernel_ptr<S, 1>(), dim3(grid), step_threads<S>(), smem_bytes<S>(), s,
-                                     mb, work, nwork, parity, queue, err)
-               : launch_programmatic(ensemble_kernel_ptr<S, 0>(), dim3(grid), step_threads<S>(), smem_bytes<S>(), s,
-                                     mb, work, nwork, parity, queue, err);
+    return launch_programmatic(kernel, dim3(grid), step_threads<S>(), smem_bytes<S>(), s, mb, work, nwork, parity,
+                               queue, err);
   // persistent schedule: a memset of the tile counter precedes each launch; ordinary ordering
-  if (stencil == 1)
-    ensemble_kernel_ptr<S, 1>()<<<grid, step_threads<S>(), smem_bytes<S>(), s>>>(mb, work, nwork, parity, queue, err);
-  else
-    ensemble_kernel_ptr<S, 0>()<<<grid, step_threads<S>(), smem_bytes<S>(), s>>>(mb, work, nwork, parity, queue, err);
+  kernel<<<grid, step_threads<S>(), smem_bytes<S>(), s>>>(mb, work, nwork, parity, queue, err);
   return cudaGetLastError();
 }
 
@@ -1671,6 +1678,10 @@ cudaError_t prepare_step_kernels() {
     e = cudaFuncSetAttribute(rel_kernel_ptr<0>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rel_smem_bytes());
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(rel_kernel_ptr<1>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rel_smem_bytes());
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(rel_kernel_ptr<0, true>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rel_smem_bytes());
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(rel_kernel_ptr<1, true>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rel_smem_bytes());
 #ifdef LBMHD_BOUNDS_CHECK
   const char* env = getenv("LBMHD_BOUNDS_FORCE");
   const unsigned force = env ? (unsigned)strtoul(env, nullptr, 0) : 0u;
@@ -1714,12 +1725,12 @@ void pack_ensemble_members(int precision, int n, const CUtensorMap* maps, void* 
   else pack_members<__half>(n, maps, pops, geoms, coefs, host_out);
 }
 
-cudaError_t launch_ensemble_step(int precision, int stencil, const void* members, const int4* work,
+cudaError_t launch_ensemble_step(int precision, int stencil, bool three, const void* members, const int4* work,
                                  int nwork, int parity, unsigned long long* queue, int grid,
                                  unsigned* err, cudaStream_t s) {
-  if (precision == 0) return launch_ens<double>(stencil, members, work, nwork, parity, queue, grid, err, s);
-  if (precision == 1) return launch_ens<float>(stencil, members, work, nwork, parity, queue, grid, err, s);
-  return launch_ens<__half>(stencil, members, work, nwork, parity, queue, grid, err, s);
+  if (precision == 0) return launch_ens<double>(stencil, three, members, work, nwork, parity, queue, grid, err, s);
+  if (precision == 1) return launch_ens<float>(stencil, three, members, work, nwork, parity, queue, grid, err, s);
+  return launch_ens<__half>(stencil, three, members, work, nwork, parity, queue, grid, err, s);
 }
 
 int resident_step_blocks(int precision, int num_sms) {
