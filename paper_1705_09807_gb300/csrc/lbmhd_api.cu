@@ -249,7 +249,7 @@ int create(lbmhd_t** out, const lbmhd_params* p) {
   // undivided differences: central a(+1)-a(-1) = 2 d; isotropic 12 d
   h->coef.kq = p->grad_stencil == LBMHD_GRAD_ISOTROPIC ? kd / 144.0 : kd / 4.0;
   h->state_bytes = (size_t)g.pitch * p->ny * h->elem;
-  g.plain = plain_step_pays(p->precision, h->coef.kq, h->state_bytes) ? 1 : 0;
+  g.plain = plain_step_pays(p->precision, h->coef.kq, p->nx, h->state_bytes) ? 1 : 0;
   g.band = step_band_rows(p->nx, p->ny, p->precision, sms, g.plain != 0);
   h->corr_band = step_band_rows(p->nx, p->ny, p->precision, sms);
 #define LB_INIT(call)                 \

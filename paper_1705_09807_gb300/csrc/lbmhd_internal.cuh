@@ -124,7 +124,7 @@ cudaError_t launch_step_f16rel(const CUtensorMap& src, const CUtensorMap& usrc, 
 // Whether a single grid's steps without correction planes take the plain form (no moments of other
 // cells; needs kq == 0), and the rows per block of its step (one wave of resident blocks when
 // possible).
-bool plain_step_pays(int precision, double kq, size_t state_bytes);
+bool plain_step_pays(int precision, double kq, int nx, size_t state_bytes);
 int step_band_rows(int nx, int ny, int precision, int num_sms, bool plain = false);
 // Opt the step kernels in to their dynamic shared memory (once per process and device).
 cudaError_t prepare_step_kernels();

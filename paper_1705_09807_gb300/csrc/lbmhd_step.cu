@@ -1151,8 +1151,9 @@ __device__ __forceinline__ bool run_tile_pair(const CUtensorMap* srcp, __half* _
 // ring, no halo columns, and a band stages exactly its own rows.  Each thread takes its 27 values
 // out of the stage, one CTA barrier frees the stage for the row NST further on, and moments,
 // collision and stores run from registers, so all NST rows are in flight (the LES form keeps a row
-// staged from its moments to its collision).  The state is bitwise that of the LES form with k = 0
-// (zero gradients go through the same operations, so the compiler contracts them alike).
+// staged from its moments to its collision).  The state is bitwise that of the LES form with vanishing
+// gradients in binary64 and binary16, whose FMAs are written out; in binary32 the compiler chooses the
+// contractions, and a step may round differently by an ulp of the deviations.
 // us per step against the LES form: binary64 64^2 14.7 -> 6.3, 512^2 127 -> 81, 2048^2 1811 -> 1159
 // (140 instead of 171 binary64 instructions per cell); binary32 128^2 2.76 -> 1.86, 512^2 9.7 -> 6.6,
 // 1024^2 36.4 -> 34.6; binary16 512^2 9.3 -> 5.7, 1024^2 22.5 -> 19.2, its relative form 256^2 5.4 -> 3.3.
@@ -1746,9 +1747,22 @@ int resident_step_blocks(int precision, int num_sms) {
 // grids, and the box columns that two strips share are then read from DRAM twice (2048^2 binary32:
 // 507 instead of 470 MB read per step, 158 instead of 142 us; 1448^2, 235 MB a copy: 79.5 against
 // 73.1; 1150^2, 147 MB: 45.7 against 45.9; 1024^2, 120 MB: 34.6 against 36.4; binary16 1700^2, 161
-// MB: 63.4 against 62.0; 1448^2, 118 MB: 43.7 against 46.9).
-bool plain_step_pays(int precision, double kq, size_t state_bytes) {
-  return kq == 0.0 && (precision == 0 || state_bytes <= (size_t)128 << 20);
+// MB: 63.4 against 62.0; 1448^2, 118 MB: 43.7 against 46.9).  Grids of few strips, hence of many short bands
+// one below the other, lose earlier (filtered / plain, by MiB of a copy: one strip, 64 columns binary16 48
+// 23.4 / 19.7, 64 31.6 / 33.0, 125 58.0 / 65.9; 128 columns binary32 48 11.1 / 9.3, 64 18.1 / 18.9, 96 29.1 /
+// 31.6; two strips, 192 columns binary32 64 20.6 / 19.9, 96 32.3 / 33.8, binary16 64 30.6 / 29.7, 96 43.6 /
+// 47.2; three to seven, 640 columns binary32 96 30.2 / 28.8, 125 40.2 / 41.8, binary16 96 39.0 / 37.1, 125 49.2
+// / 52.2; eight, binary32 96 30.8 / 29.3, binary16 96 39.4 / 36.8, at 125 no difference).
+// Sparse strips keep the filtered form waiting longer than memory does, so there the plain one pays up to the
+// same size as on wide grids (64 columns relative 64 36.0 / 33.6, 96 no difference; 192 columns relative 125 67 /
+// 64, 300 columns 73 / 60).
+bool plain_step_pays(int precision, double kq, int nx, size_t state_bytes) {
+  const int strips = (nx + kStepThreads - 1) / kStepThreads, lanes = strips * kStepThreads;
+  const bool half = precision == LBMHD_FP16, rel = precision == LBMHD_FP16_REL;
+  const bool sparse = 4 * nx <= lanes || (rel && (strips == 1 ? 2 * nx <= lanes : 5 * nx < 4 * lanes));
+  size_t most = 128;  // MiB
+  if (!sparse) most = strips == 1 ? 56 : strips == 2 ? (half ? 56 : 72) : strips == 3 && half ? 88 : strips < 8 ? 104 : 128;
+  return kq == 0.0 && (precision == 0 || state_bytes <= most << 20);
 }
 
 // Rows per block: with the blocks that fit on the GPU at once (`resident`), give every strip
