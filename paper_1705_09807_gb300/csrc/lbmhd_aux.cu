@@ -343,25 +343,27 @@ struct CellValues {
 };
 
 // Moments of a cell of the relative binary16 form with infinities or NaN among its values, from
-// binary64 sums: the pair sums make NaN of an infinite population, where rho is infinite.  A call, for
-// states that have diverged.
+// binary64 sums: the pair sums make NaN of an infinite population, where rho is infinite.  For states that
+// have diverged: a loop over the populations, so that it takes no registers from the others (1025 x 1024
+// 27.9 us with a call, 27.6 now, 27.5 without).
 template <typename T>
-__device__ __noinline__ void moments_diverged(const T* __restrict__ pops, int nx, int ny, int pitch, size_t plane,
-                                              int x, int y, double* out) {
-  StepGeom g{};
-  g.nx = nx;
-  g.ny = ny;
-  g.pitch = pitch;
-  g.plane = plane;
-  double v[27], r = 0, jx = 0, jy = 0, sbx = 0, sby = 0;
-  pull_cell<T, true>(pops, g, x, y, v);
-#pragma unroll
+__device__ __forceinline__ void moments_diverged(const T* __restrict__ pops, const StepGeom& g, int x, int y,
+                                                 double (&out)[5]) {
+  double r = 0, jx = 0, jy = 0, sbx = 0, sby = 0;
+#pragma unroll 1
   for (int i = 0; i < 9; ++i) {
-    r += v[i];
-    jx += vx(i) * v[i];
-    jy += vy(i) * v[i];
-    sbx += v[9 + i];
-    sby += v[18 + i];
+    const int cx = vx(i), cy = vy(i);
+    const T* p = pops + (size_t)wrapi(y - cy, g.ny) * g.pitch + kXOff + wrapi(x - cx, g.nx);
+    double f = load_as<double>(p[(size_t)plane_of(i) * g.plane]);
+    if (i > 0) {
+      const double Ux = load_as<double>(p[(size_t)kQ * g.plane]), Uy = load_as<double>(p[(size_t)(kQ + 1) * g.plane]);
+      f += 3.0 * wt(i) * (cx * Ux + cy * Uy);
+    }
+    r += f;
+    jx += cx * f;
+    jy += cy * f;
+    sbx += load_as<double>(p[(size_t)plane_of(9 + i) * g.plane]);
+    sby += load_as<double>(p[(size_t)plane_of(18 + i) * g.plane]);
   }
   out[0] = 1.0 + r;
   const float ir = 1.f / (float)out[0];
@@ -377,12 +379,7 @@ __device__ __forceinline__ void cell_moments(const CellValues<T, REL>& cell, con
                                              const StepGeom& g, int x, int y, double (&out)[5]) {
   const bool finite = cell.moments(out);
   if constexpr (REL) {
-    if (!finite) {
-      double d[5];
-      moments_diverged(pops, g.nx, g.ny, g.pitch, g.plane, x, y, d);
-#pragma unroll
-      for (int k = 0; k < 5; ++k) out[k] = d[k];
-    }
+    if (!finite) moments_diverged(pops, g, x, y, out);
   }
 }
 
